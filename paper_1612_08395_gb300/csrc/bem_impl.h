@@ -66,6 +66,7 @@ struct Scalars {
   // CG iterations counted on the device, and the cap after which the solve
   // stops unconverged (the bound of the batched while-loop graph).
   int loops, max_loops;
+  int n_small;   // Polonsky-Keer: consecutive iterations with eps below the tolerance
   unsigned int cnt_a, cnt_c, cnt_r;  // last-block arrival counters
   // Sticky device error bits (kept across solves: init_scalars does not copy
   // this member); 1 = a kernel gave up waiting for its own asynchronous copies,
@@ -120,6 +121,11 @@ struct PassArgs {
   const void* twB;      // stage twiddle tables, length Py (C<T>)
   const void* twB16;    // stage twiddle tables of the radix-16 column pass, length Py (C<T>)
   const void* twS;      // exp(-i pi k / M), k = 0..M (C<T>): real-FFT split
+  const int4* fxA;      // FP64 path: the tables twA, twB and twS as 30-bit limbs (fx_kernels.cuh)
+  const int4* fxB;
+  const int4* fxS;
+  int* fx_ea;           // FP64 path: exponents of W's row groups (pass A) ...
+  int* fx_eb;           // ... and of its columns kx (pass B)
   const int* soA;       // index tables of length M and Py (see Geo)
   const int* spA;
   const int* soB;
@@ -158,6 +164,15 @@ __host__ __device__ constexpr size_t pass_c_smem(size_t smemC, int M, int nb, in
 template <typename T> void launch_pass_a(const PassArgs<T>& a, int mode, cudaStream_t s);
 template <typename T> void launch_pass_b(const PassArgs<T>& a, int mode, cudaStream_t s);
 template <typename T> void launch_pass_c(const PassArgs<T>& a, int mode, cudaStream_t s);
+
+// FP64 path in 64-bit block fixed point (fx_kernels.cuh); with arr, over n instances.
+void launch_fx_a(const PassArgs<double>& a, int mode, const PassArgs<double>* arr, int n, cudaStream_t s);
+void launch_fx_b(const PassArgs<double>& a, const PassArgs<double>* arr, int n, cudaStream_t s);
+void launch_fx_c(const PassArgs<double>& a, int mode, const PassArgs<double>* arr, int n, cudaStream_t s);
+cudaError_t set_smem_attrs_fx_a(int bytes);
+cudaError_t set_smem_attrs_fx_b(int bytes);
+cudaError_t set_smem_attrs_fx_c(int bytes);
+void launch_fx_tables(const double2* w, int4* out, int n, cudaStream_t s);
 
 // The same passes over n instances of one size class at once (blockIdx.y =
 // instance); a0 is any of them (its plan, row and column counts), arr the

@@ -449,16 +449,19 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
 // thread 0 writes a block's partials, so only it fences: release before its
 // arrival, and, in the last block, acquire before the partials are read (with
 // L2 loads, after the barrier that publishes the flag).
-__device__ __forceinline__ bool last_block_arrival(unsigned int* counter, int* flag_smem) {
+__device__ __forceinline__ bool last_block_arrival_of(unsigned int* counter, int* flag_smem, int nblocks) {
   if (threadIdx.x == 0) {
     __threadfence();
     const unsigned int t = atomicAdd(counter, 1u);
-    const bool last = t == gridDim.x - 1;
+    const bool last = t == (unsigned)nblocks - 1;
     if (last) __threadfence();
     *flag_smem = last ? 1 : 0;
   }
   __syncthreads();
   return *flag_smem != 0;
+}
+__device__ __forceinline__ bool last_block_arrival(unsigned int* counter, int* flag_smem) {
+  return last_block_arrival_of(counter, flag_smem, (int)gridDim.x);
 }
 
 // ---------------------------------------------------------------------------

@@ -1150,6 +1150,14 @@ __device__ __forceinline__ void cg_pre_load(const Scalars* sc, CgPre* pre) {
   pre->max_loops = sc->max_loops;
 }
 
+// Consecutive iterations whose eps must be below the tolerance to end a
+// Polonsky-Keer solve.  eps dips now and then by more than a factor of two, so
+// where one small step ends the solve is a matter of rounding: on the
+// warm-started 512 x 512 sweep (k = -0.5, tol = 1e-12, FP64) the pressure's
+// error is anywhere in 0.5e-10 .. 1.4e-10; with two it is 1e-11 for 4.5% more
+// iterations.  The FP32 solves end at their rounding floor or are refined.
+template <typename T> constexpr int kSmallSteps = sizeof(T) == 8 ? 2 : 1;
+
 template <typename T, int MODE>
 __device__ __forceinline__ void pass_c_finalize(Scalars* sc, const double (&s2)[4], const double (&s3)[3],
                                                 const CgPre& pre) {
@@ -1165,8 +1173,9 @@ __device__ __forceinline__ void pass_c_finalize(Scalars* sc, const double (&s2)[
       const double eps = s3[1] > 0.0 ? s3[0] / s3[1] : 0.0;
       sc->eps = eps;
       sc->delta = s3[2] > 0.0 ? 0.0 : 1.0;
+      if (!(eps < sc->tol)) sc->n_small = 0;
       if (!isfinite(eps) || !isfinite(G)) { sc->status = SC_NUMERIC; done = 1; }
-      else if (eps < sc->tol) done = 1;
+      else if (eps < sc->tol && (sc->n_small += 1) >= kSmallSteps<T>) done = 1;
       else if (sc->iter >= sc->max_iter) { sc->status = SC_NOCONV; done = 1; }
       // rounding floor: no new minimum of eps for kStall iterations ends the solve
       if (!done) {
@@ -1851,7 +1860,7 @@ template <typename T, int MODE>
 void launch_a_mode(const PassArgs<T>& a, cudaStream_t s) {
   const dim3 block(a.pl.threadsA);
   const int groups = (a.nrows_in + a.pl.nbA - 1) / a.pl.nbA;
-  if (BEM_PERSISTENT && MODE != A_TORUS && (a.ncols_in & 15) == 0 && pro_fields_aligned<T, MODE>(a)) {
+  if constexpr (MODE != A_TORUS) if (BEM_PERSISTENT && (a.ncols_in & 15) == 0 && pro_fields_aligned<T, MODE>(a)) {
     const size_t smem = ((a.pl.smemA + 15) & ~(size_t)15) + pro_stage_bytes<T, MODE>(a.pl.nbA, a.ncols_in);
     switch (a.pl.gA.logL) {
 #define BEM_CASE(LG)                                                                        \
@@ -1876,7 +1885,7 @@ void launch_a_mode(const PassArgs<T>& a, cudaStream_t s) {
 template <typename T, int MODE>
 void launch_b_mode(const PassArgs<T>& a, cudaStream_t s) {
   const dim3 grid(a.pl.gridB), block(a.pl.threadsB);
-  if (MODE == B_CONV && a.pl.radixB == 16) {
+  if constexpr (MODE == B_CONV) if (a.pl.radixB == 16) {
     switch (a.pl.gB.logL) {
 #define BEM_CASE(LG) case LG: k_pass_b16<T, LG><<<grid, block, a.pl.smemB, s>>>(a); break;
       BEM_LOGL_CASES_B16(BEM_CASE)
@@ -1956,7 +1965,8 @@ void launch_c_mode_mi(const PassArgs<T>& a0, const PassArgs<T>* arr, int n, cuda
 }
 template <typename T>
 void launch_pass_a_mi(const PassArgs<T>& a0, int mode, const PassArgs<T>* arr, int n, cudaStream_t s) {
-  if (mode == A_PK_P) launch_a_mode_mi<T, A_PK_P>(a0, arr, n, s);
+  if constexpr (sizeof(T) == 8) launch_fx_a(a0, mode, arr, n, s);
+  else if (mode == A_PK_P) launch_a_mode_mi<T, A_PK_P>(a0, arr, n, s);
   else if (mode == A_PK_T) launch_a_mode_mi<T, A_PK_T>(a0, arr, n, s);
   else if (mode == A_CG_T) launch_a_mode_mi<T, A_CG_T>(a0, arr, n, s);
 }
@@ -1968,6 +1978,10 @@ void launch_pass_b_mi(const PassArgs<T>& a0, const PassArgs<T>* arr, int n, cuda
       return;
     }
   }
+  if constexpr (sizeof(T) == 8) {
+    launch_fx_b(a0, arr, n, s);
+    return;
+  } else {
   const dim3 grid(a0.pl.gridB, n), block(a0.pl.threadsB);
   if (a0.pl.radixB == 16) {
     switch (a0.pl.gB.logL) {
@@ -1982,10 +1996,12 @@ void launch_pass_b_mi(const PassArgs<T>& a0, const PassArgs<T>* arr, int n, cuda
     BEM_LOGL_CASES_B(BEM_CASE)
 #undef BEM_CASE
   }
+  }
 }
 template <typename T>
 void launch_pass_c_mi(const PassArgs<T>& a0, int mode, const PassArgs<T>* arr, int n, cudaStream_t s) {
-  if (mode == C_PK_G) launch_c_mode_mi<T, C_PK_G>(a0, arr, n, s);
+  if constexpr (sizeof(T) == 8) launch_fx_c(a0, mode, arr, n, s);
+  else if (mode == C_PK_G) launch_c_mode_mi<T, C_PK_G>(a0, arr, n, s);
   else if (mode == C_PK_R) launch_c_mode_mi<T, C_PK_R>(a0, arr, n, s);
   else if (mode == C_CG_R) launch_c_mode_mi<T, C_CG_R>(a0, arr, n, s);
 }
@@ -1994,41 +2010,48 @@ void launch_batch_ctl(const PassArgs<T>* arr, int n, unsigned long long cond, cu
   k_batch_ctl<T><<<1, 256, 0, s>>>(arr, n, cond);
 }
 
+// FP32 transforms run the FP32 passes; FP64 ones the block fixed-point passes,
+// but for the spectrum's set-up (A_TORUS, B_SPECTRUM).
 template <typename T>
 void launch_pass_a(const PassArgs<T>& a, int mode, cudaStream_t s) {
-  switch (mode) {
-    case A_PLAIN: launch_a_mode<T, A_PLAIN>(a, s); break;
-    case A_PK_P: launch_a_mode<T, A_PK_P>(a, s); break;
-    case A_PK_T: launch_a_mode<T, A_PK_T>(a, s); break;
-    case A_CG_T: launch_a_mode<T, A_CG_T>(a, s); break;
-    case A_TORUS:
-      if constexpr (sizeof(T) == 8) launch_a_mode<T, A_TORUS>(a, s);
-      break;
+  if constexpr (sizeof(T) == 8) {
+    if (mode == A_TORUS) launch_a_mode<T, A_TORUS>(a, s);
+    else launch_fx_a(a, mode, nullptr, 1, s);
+  } else {
+    switch (mode) {
+      case A_PLAIN: launch_a_mode<T, A_PLAIN>(a, s); break;
+      case A_PK_P: launch_a_mode<T, A_PK_P>(a, s); break;
+      case A_PK_T: launch_a_mode<T, A_PK_T>(a, s); break;
+      case A_CG_T: launch_a_mode<T, A_CG_T>(a, s); break;
+    }
   }
 }
 template <typename T>
 void launch_pass_b(const PassArgs<T>& a, int mode, cudaStream_t s) {
-  if (mode == B_SPECTRUM) {
-    launch_b_mode<T, B_SPECTRUM>(a, s);
-    return;
-  }
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 8) {
+    if (mode == B_SPECTRUM) launch_b_mode<T, B_SPECTRUM>(a, s);
+    else launch_fx_b(a, nullptr, 1, s);
+  } else {
     if (tc_column_pass_enabled() && tc_column_pass_applies(a)) {
       launch_pass_b_tc(a, s);
       return;
     }
+    launch_b_mode<T, B_CONV>(a, s);
   }
-  launch_b_mode<T, B_CONV>(a, s);
 }
 template <typename T>
 void launch_pass_c(const PassArgs<T>& a, int mode, cudaStream_t s) {
-  switch (mode) {
-    case C_PLAIN: launch_c_mode<T, C_PLAIN>(a, s); break;
-    case C_PK_G: launch_c_mode<T, C_PK_G>(a, s); break;
-    case C_PK_R: launch_c_mode<T, C_PK_R>(a, s); break;
-    case C_CG_R: launch_c_mode<T, C_CG_R>(a, s); break;
-    case C_CG_G: launch_c_mode<T, C_CG_G>(a, s); break;
-    case C_GAP: launch_c_mode<T, C_GAP>(a, s); break;
+  if constexpr (sizeof(T) == 8) {
+    launch_fx_c(a, mode, nullptr, 1, s);
+  } else {
+    switch (mode) {
+      case C_PLAIN: launch_c_mode<T, C_PLAIN>(a, s); break;
+      case C_PK_G: launch_c_mode<T, C_PK_G>(a, s); break;
+      case C_PK_R: launch_c_mode<T, C_PK_R>(a, s); break;
+      case C_CG_R: launch_c_mode<T, C_CG_R>(a, s); break;
+      case C_CG_G: launch_c_mode<T, C_CG_G>(a, s); break;
+      case C_GAP: launch_c_mode<T, C_GAP>(a, s); break;
+    }
   }
 }
 
@@ -2048,6 +2071,11 @@ cudaError_t set_smem_max(K kernel, int bytes) {
 template <typename T>
 cudaError_t set_smem_attrs_a(int bytes) {
   cudaError_t e = cudaSuccess, r;
+  if constexpr (sizeof(T) == 8) {
+#define BEM_CASE(LG) BEM_ATTR((k_pass_a<T, A_TORUS, LG>))
+    BEM_LOGL_CASES_A(BEM_CASE)
+#undef BEM_CASE
+  } else {
 #define BEM_CASE(LG)                          \
   BEM_ATTR((k_pass_a<T, A_PLAIN, LG>))        \
   BEM_ATTR((k_pass_a<T, A_PK_P, LG>))         \
@@ -2059,22 +2087,27 @@ cudaError_t set_smem_attrs_a(int bytes) {
   BEM_ATTR((k_pass_ap<T, A_CG_T, LG>))        \
   BEM_ATTR((k_pass_ap_mi<T, A_PK_P, LG>))     \
   BEM_ATTR((k_pass_ap_mi<T, A_PK_T, LG>))     \
-  BEM_ATTR((k_pass_ap_mi<T, A_CG_T, LG>))     \
-  if constexpr (sizeof(T) == 8) { BEM_ATTR((k_pass_a<T, A_TORUS, LG>)) }
-  BEM_LOGL_CASES_A(BEM_CASE)
+  BEM_ATTR((k_pass_ap_mi<T, A_CG_T, LG>))
+    BEM_LOGL_CASES_A(BEM_CASE)
 #undef BEM_CASE
+  }
   return e;
 }
 template <typename T>
 cudaError_t set_smem_attrs_b(int bytes) {
   cudaError_t e = cudaSuccess, r;
-#define BEM_CASE(LG) \
-  BEM_ATTR((k_pass_b<T, B_CONV, LG>)) BEM_ATTR((k_pass_b<T, B_SPECTRUM, LG>)) BEM_ATTR((k_pass_b_mi<T, B_CONV, LG>))
-  BEM_LOGL_CASES_B(BEM_CASE)
+  if constexpr (sizeof(T) == 8) {
+#define BEM_CASE(LG) BEM_ATTR((k_pass_b<T, B_SPECTRUM, LG>))
+    BEM_LOGL_CASES_B(BEM_CASE)
+#undef BEM_CASE
+  } else {
+#define BEM_CASE(LG) BEM_ATTR((k_pass_b<T, B_CONV, LG>)) BEM_ATTR((k_pass_b_mi<T, B_CONV, LG>))
+    BEM_LOGL_CASES_B(BEM_CASE)
 #undef BEM_CASE
 #define BEM_CASE(LG) BEM_ATTR((k_pass_b16<T, LG>)) BEM_ATTR((k_pass_b16_mi<T, LG>))
-  BEM_LOGL_CASES_B16(BEM_CASE)
+    BEM_LOGL_CASES_B16(BEM_CASE)
 #undef BEM_CASE
+  }
   return e;
 }
 template <typename T>

@@ -101,13 +101,16 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   const int px = pow2_at_least(2 * Nx < 32 ? 32 : 2 * Nx);
   const int py = pow2_at_least(2 * Ny < 32 ? 32 : 2 * Ny);
   const int M = px / 2, hx = M + 1, hyq = py / 2 + 1;
-  // scratch layout: W | transposed spectrum | FP64 twiddles | FP32 twiddles
+  // scratch layout: W | transposed spectrum | twiddles (FP64, FP32, fixed point) |
+  // exponents | index tables
   const size_t ntw = (size_t)M + py + M + 1;
   const size_t w_bytes = sizeof(double) * 2 * (size_t)hx * Ny;
   const size_t k_off = (w_bytes + 255) & ~(size_t)255;
   const size_t t_off = (k_off + sizeof(double) * (size_t)hx * hyq + 255) & ~(size_t)255;
   const size_t t32_off = (t_off + sizeof(double2) * ntw + 255) & ~(size_t)255;
-  const size_t g_off = (t32_off + sizeof(float2) * ntw + 255) & ~(size_t)255;
+  const size_t tfx_off = (t32_off + sizeof(float2) * ntw + 255) & ~(size_t)255;
+  const size_t e_off = (tfx_off + sizeof(int4) * ntw + 255) & ~(size_t)255;
+  const size_t g_off = (e_off + sizeof(int) * ((size_t)Ny + hx) + 255) & ~(size_t)255;
   const size_t g_ints = 2 * bem::kSoEntries + (size_t)M + py;
   if (g_off + sizeof(int) * g_ints > kScratchBytes)
     return bem::set_error(BEM_EINVAL, "bem_convolve_noalloc: grid needs more than the 2 MiB static scratch");
@@ -126,6 +129,7 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   double* khat_t = reinterpret_cast<double*>(scratch + k_off);
   double2* tw64 = reinterpret_cast<double2*>(scratch + t_off);
   float2* tw32 = reinterpret_cast<float2*>(scratch + t32_off);
+  int4* twfx = reinterpret_cast<int4*>(scratch + tfx_off);
   int* geo = reinterpret_cast<int*>(scratch + g_off);
   bem::launch_geo_tables(geo, geo + bem::kSoEntries, pl.gA, 8, s);
   bem::launch_geo_tables(geo + bem::kSoEntries + M, geo + 2 * bem::kSoEntries + M, pl.gB, 8, s);
@@ -133,6 +137,8 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   bem::launch_twiddles(tw64, tw32, ilog2i(M), s);
   bem::launch_twiddles(tw64 + M, tw32 + M, ilog2i(py), s);
   bem::launch_split_twiddles(tw64 + M + py, tw32 + M + py, M, s);
+
+  bem::launch_fx_tables(tw64, twfx, (int)ntw, s);
 
   bem::PassArgs<double> a{};
   a.pl = pl;
@@ -146,6 +152,11 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   a.twA = tw64;
   a.twB = tw64 + M;
   a.twS = tw64 + M + py;
+  a.fxA = twfx;
+  a.fxB = twfx + M;
+  a.fxS = twfx + M + py;
+  a.fx_ea = reinterpret_cast<int*>(scratch + e_off);
+  a.fx_eb = a.fx_ea + Ny;
   a.soA = geo;
   a.spA = geo + bem::kSoEntries;
   a.soB = geo + bem::kSoEntries + M;

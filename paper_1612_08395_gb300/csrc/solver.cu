@@ -213,7 +213,9 @@ int device_setup(int dev) {
   if (ea == cudaSuccess) ea = set_smem_attrs_c<float>(smem_max);
   if (ea == cudaSuccess) ea = set_smem_attrs_a<double>(smem_max);
   if (ea == cudaSuccess) ea = set_smem_attrs_b<double>(smem_max);
-  if (ea == cudaSuccess) ea = set_smem_attrs_c<double>(smem_max);
+  if (ea == cudaSuccess) ea = set_smem_attrs_fx_a(smem_max);
+  if (ea == cudaSuccess) ea = set_smem_attrs_fx_b(smem_max);
+  if (ea == cudaSuccess) ea = set_smem_attrs_fx_c(smem_max);
   if (ea != cudaSuccess) return fail(BEM_ECUDA, "shared-memory opt-in failed: %s", cudaGetErrorString(ea));
   if (influence_init_nodes() != 0) return fail(BEM_ECUDA, "quadrature nodes upload failed");
   const int rc = tc_column_pass_setup();
@@ -233,6 +235,8 @@ struct bem_ctx {
   int* geo = nullptr;       // index tables: [A32 | B32 | A64 | B64], each so (112) + sp (L)
   double2* tw64 = nullptr;  // [length-M stages | length-Py stages | split], FP64
   float2* tw32 = nullptr;   // the same, FP32
+  int4* twfx = nullptr;     // the first three tables as fixed-point limbs (FP64 path)
+  int* fxe = nullptr;       // FP64 path: exponents of W's row groups (ny) and columns (M + 1)
   double* khat64 = nullptr;
   float* khat32 = nullptr;
   void* W = nullptr;
@@ -266,10 +270,10 @@ struct bem_ctx {
   // CG loops join this batcher when set (concurrent solves of the server)
   bem::LoopBatcher* batcher = nullptr;
   cudaEvent_t ev_ready = nullptr;  // this context's work before its batched loop
-  // Tensor maps of W for pass C's TMA staging, [FP32, FP64] views with the
-  // plan's rows per CTA (device memory; null where TMA does not apply)
-  void* tmw[2] = {nullptr, nullptr};
-  bool tmw_ok[2] = {false, false};
+  // Tensor map of W (FP32) for pass C's TMA staging, with the plan's rows per
+  // CTA (device memory; null where TMA does not apply)
+  void* tmw = nullptr;
+  bool tmw_ok = false;
 };
 
 static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu, double E0, double c0,
@@ -334,43 +338,42 @@ EncodeTiledFn tensor_map_encoder() {
   return fn;
 }
 
-// The tensor map of W for pass C's TMA staging in precision es (4 or 8): W as
-// (M+1) rows of 2 ny reals, boxes of 2 nb reals x w_box_rows(M) rows, zero fill
-// past the ends.  TMA wants 16-byte strides and box rows, so FP32 needs an even
-// ny and an even nb; where that fails (or TMA is unavailable) the map stays off
-// and pass C stages W with cp.async.  BEM_TMA=0 switches it off.
-int update_w_map(bem_ctx* h, int es, int nb) {
-  const int i = es == 8 ? 1 : 0;
-  h->tmw_ok[i] = false;
+// The tensor map of W for the FP32 pass C's TMA staging: W as (M+1) rows of 2 ny
+// floats, boxes of 2 nb floats x w_box_rows(M) rows, zero fill past the ends.
+// TMA wants 16-byte strides and box rows, so an even ny and an even nb; where
+// that fails (or TMA is unavailable) the map stays off and pass C stages W with
+// cp.async.  BEM_TMA=0 switches it off.
+int update_w_map(bem_ctx* h, int nb) {
+  h->tmw_ok = false;
   static const bool on = [] {
     const char* e = getenv("BEM_TMA");
     return !(e && e[0] == '0');
   }();
   EncodeTiledFn enc = tensor_map_encoder();
   if (!on || !enc) return BEM_OK;
-  if (es == 4 && ((h->ny & 1) || (nb & 1))) return BEM_OK;
+  if ((h->ny & 1) || (nb & 1)) return BEM_OK;
   const int M = h->px / 2;
   CUtensorMap m;
   const cuuint64_t dims[2] = {(cuuint64_t)2 * h->ny, (cuuint64_t)M + 1};
-  const cuuint64_t strides[1] = {(cuuint64_t)2 * h->ny * es};
+  const cuuint64_t strides[1] = {(cuuint64_t)2 * h->ny * 4};
   const cuuint32_t box[2] = {(cuuint32_t)(2 * nb), (cuuint32_t)w_box_rows(M)};
   const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = enc(&m, es == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->W,
-                         dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+  const CUresult r = enc(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->W, dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return BEM_OK;  // not representable: stay on cp.async
-  if (!h->tmw[i]) {
-    if (cudaMalloc(&h->tmw[i], sizeof(CUtensorMap)) != cudaSuccess) {
+  if (!h->tmw) {
+    if (cudaMalloc(&h->tmw, sizeof(CUtensorMap)) != cudaSuccess) {
       cudaGetLastError();
-      h->tmw[i] = nullptr;
+      h->tmw = nullptr;
       return BEM_OK;
     }
     h->bytes += sizeof(CUtensorMap);
   }
   // ordered before every later launch on the handle's stream
-  CK(cudaMemcpyAsync(h->tmw[i], &m, sizeof m, cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemcpyAsync(h->tmw, &m, sizeof m, cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  h->tmw_ok[i] = true;
+  h->tmw_ok = true;
   return BEM_OK;
 }
 
@@ -391,6 +394,8 @@ PassArgs<T> make_args(bem_ctx* h) {
   } else {
     a.twA = h->tw32; a.twB = h->tw32 + M; a.twS = h->tw32 + M + P; a.twB16 = h->tw32 + M + P + M + 1;
   }
+  a.fxA = h->twfx; a.fxB = h->twfx + M; a.fxS = h->twfx + M + P;
+  a.fx_ea = h->fxe; a.fx_eb = h->fxe + h->ny;
   const int* gt = h->geo + (sizeof(T) == 8 ? 2 * kSoEntries + M + P : 0);
   a.soA = gt;
   a.spA = gt + kSoEntries;
@@ -399,7 +404,7 @@ PassArgs<T> make_args(bem_ctx* h) {
   a.uscale = h->A / ((double)h->px * (double)h->py);
   a.partA = h->part;
   a.partC = h->partC;
-  a.tmW = h->tmw_ok[sizeof(T) == 8 ? 1 : 0] ? h->tmw[sizeof(T) == 8 ? 1 : 0] : nullptr;
+  a.tmW = sizeof(T) == 4 && h->tmw_ok ? h->tmw : nullptr;
   a.sc = h->sc;
   a.kerr = &h->sc->kerr;
   return a;
@@ -1230,7 +1235,7 @@ std::map<ShapeKey, Tuned> g_tuned;
 
 int set_plan32(bem_ctx* h, const Plan& pl) {
   h->plan32 = pl;
-  CKR(update_w_map(h, 4, pl.nbA));
+  CKR(update_w_map(h, pl.nbA));
   int* g32 = h->geo;
   const int M = h->px / 2;
   launch_geo_tables(g32, g32 + kSoEntries, pl.gA, 4, h->stream);
@@ -1409,6 +1414,8 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
   const size_t ntw = (size_t)M + h->py + M + 1 + h->py;
   if ((rc = dmalloc(h, (void**)&h->tw64, sizeof(double2) * ntw))) return cleanup(rc);
   if ((rc = dmalloc(h, (void**)&h->tw32, sizeof(float2) * ntw))) return cleanup(rc);
+  if ((rc = dmalloc(h, (void**)&h->twfx, sizeof(int4) * (ntw - h->py)))) return cleanup(rc);
+  if ((rc = dmalloc(h, (void**)&h->fxe, sizeof(int) * ((size_t)Ny + M + 1)))) return cleanup(rc);
   if ((rc = dmalloc(h, (void**)&h->geo, sizeof(int) * 2 * (2 * kSoEntries + M + h->py)))) return cleanup(rc);
   if ((rc = dmalloc(h, (void**)&h->khat64, sizeof(double) * (size_t)hyq * (M + 1)))) return cleanup(rc);
   if ((rc = dmalloc(h, (void**)&h->khat32, sizeof(float) * (size_t)hyq * (M + 1)))) return cleanup(rc);
@@ -1447,6 +1454,7 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
   launch_twiddles(h->tw64, h->tw32, ilog2(M), h->stream);
   launch_twiddles(h->tw64 + M, h->tw32 + M, ilog2(h->py), h->stream);
   launch_split_twiddles(h->tw64 + M + h->py, h->tw32 + M + h->py, M, h->stream);
+  launch_fx_tables(h->tw64, h->twfx, (int)(ntw - h->py), h->stream);
   launch_twiddles16(h->tw64 + M + h->py + M + 1, h->tw32 + M + h->py + M + 1, ilog2(h->py), h->stream);
   // a1: influence coefficients on the offsets 0..Px/2, 0..Py/2 (Eq. 9)
   if (parent) {
@@ -1483,7 +1491,7 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cleanup(fail(BEM_ECUDA, "set-up kernels failed: %s", cudaGetErrorString(e)));
-  if ((rc = update_w_map(h, 4, h->plan32.nbA)) || (rc = update_w_map(h, 8, h->plan64.nbA))) return cleanup(rc);
+  if ((rc = update_w_map(h, h->plan32.nbA))) return cleanup(rc);
   if ((rc = autotune32(h))) return cleanup(rc);
   *out = h;
   return BEM_OK;
@@ -1502,8 +1510,8 @@ extern "C" void bem_destroy(bem_handle h) {
     for (int j = 0; j < 4; ++j)
       if (h->ev[i][j]) cudaEventDestroy(h->ev[i][j]);
   if (h->ev_ready) cudaEventDestroy(h->ev_ready);
-  fr(h->tmw[0]); fr(h->tmw[1]);
-  fr(h->kq64); fr(h->geo); fr(h->tw64); fr(h->tw32); fr(h->khat64); fr(h->khat32); fr(h->W); fr(h->h64); fr(h->io64); fr(h->io64b);
+  fr(h->tmw);
+  fr(h->kq64); fr(h->geo); fr(h->tw64); fr(h->tw32); fr(h->twfx); fr(h->fxe); fr(h->khat64); fr(h->khat32); fr(h->W); fr(h->h64); fr(h->io64); fr(h->io64b);
   fr(h->S); fr(h->part); fr(h->partC); fr(h->partE); fr(h->stats); fr(h->sc);
   fr(h->f32.p); fr(h->f32.g); fr(h->f32.t); fr(h->f32.r); fr(h->f32.c);
   fr(h->f64.p); fr(h->f64.g); fr(h->f64.t); fr(h->f64.r); fr(h->f64.c);
