@@ -174,6 +174,34 @@ cudaError_t set_smem_attrs_fx_b(int bytes);
 cudaError_t set_smem_attrs_fx_c(int bytes);
 void launch_fx_tables(const double2* w, int4* out, int n, cudaStream_t s);
 
+// CG loops of small grids in one thread-block cluster (resident.cuh): lm = log2 M
+// in 4..8, lp = log2 Py in 5..9, n instances.
+struct ResArgs {
+  const PassArgs<float>* arr;  // several instances (blockIdx.y), or null: `one`
+  PassArgs<float> one;
+  int resume;       // continue a loop that ended at its launch's iteration bound
+  int max_launch;   // iterations of this launch at most
+};
+cudaError_t launch_resident_cg(const ResArgs& r, int lm, int lp, int n, cudaStream_t s);
+cudaError_t launch_resident_pk(const ResArgs& r, int lm, int lp, int n, cudaStream_t s);
+cudaError_t resident_setup_cg(bool* runs);  // once per device
+cudaError_t resident_setup_pk(bool* runs);
+
+// CG loops of medium grids in one cooperative launch (coop.cuh): lm = log2 M in
+// 8..10, lp = log2 Py in 9..11, an even number of grid rows.
+struct CoopArgs {
+  PassArgs<float> one;
+  void* shared;     // barrier and partial sums, coop_shared_bytes() of device memory
+  int R;            // rows per CTA (set by the launch)
+  int rows;         // grid rows that can hold pressure: 0 .. rows - 1
+  int resume, max_launch;  // as ResArgs
+};
+size_t coop_shared_bytes();
+cudaError_t launch_coop_cg(const CoopArgs& r, int lm, int lp, cudaStream_t s);
+cudaError_t launch_coop_pk(const CoopArgs& r, int lm, int lp, cudaStream_t s);
+cudaError_t coop_setup_cg();  // once per device
+cudaError_t coop_setup_pk();
+
 // The same passes over n instances of one size class at once (blockIdx.y =
 // instance); a0 is any of them (its plan, row and column counts), arr the
 // device array of all n instances' arguments.  Only the CG-loop modes and the

@@ -1,0 +1,648 @@
+// CG loops of medium grids in one cooperative launch (FP32 path).
+//
+// On sub-grids of 256 to 1024 elements a side the three passes of a fixed-set
+// CG iteration take 36 us on the 2048^2 torus although their instructions need
+// about 15: each pass starts cold (launch gap, scalar reads, staging set-up,
+// first loads) and ends with one CTA adding everybody's sums.  Here the whole
+// loop is one kernel of one CTA per SM:
+//   - a CTA owns R grid rows for the whole loop and keeps their p, g, t and r
+//     (or c) in shared memory; only W crosses the chip, through L2;
+//   - phases are separated by a grid barrier (arrive on a counter, poll it):
+//     three per transform;
+//   - every CTA adds all CTAs' partial sums itself, in the same order, and takes
+//     the scalar decisions from its own copy, so no CTA waits for another's
+//     serial tail beyond the barrier.
+// Only the rows that can hold pressure (the box of the held or overlap set) are
+// transformed.  The arithmetic is that of the passes; the order of the partial
+// sums differs.  Every wait is bounded: a CTA that gives up sets the handle's
+// error word and leaves, and so do the others.
+#pragma once
+#include "resident.cuh"
+
+namespace bem {
+
+template <int LM, int LP>
+struct CoopGeo {
+  static constexpr int M = 1 << LM, P = 1 << LP, NY = P / 2;
+  static constexpr int TR = M / 8, TC = P / 8;
+  // four columns a round (2048 points: 1024 threads of 64 registers)
+  static constexpr int NT = LP == 11 ? 1024 : LP == 10 || LM == 10 ? 512 : 256;
+  static constexpr int RPR = NT / TR < 8 ? NT / TR : 8, CPR = NT / TC < 8 ? NT / TC : 8;  // rows, columns per round
+  static constexpr int RS = M + kGeo8[LM - 3].pad[res_lg(RPR)];
+  static constexpr int CZ = P + kGeo8[LP - 3].pad[res_lg(CPR)];
+  static constexpr int work = (RPR * RS > CPR * CZ ? RPR * RS : CPR * CZ);  // float2
+  static constexpr int RMAX = 2 * RPR < 16 ? 2 * RPR : 16;                  // rows per CTA at most
+};
+
+// State of the grid barrier and the partial sums (device memory of the handle).
+struct CoopShared {
+  unsigned int count, fail;
+  unsigned int pad[30];
+  float2 part[2][256 * 8];  // alternating between consecutive sums
+};
+size_t coop_shared_bytes();
+
+template <int LM, int LP>
+struct Coop {
+  using Gm = CoopGeo<LM, LP>;
+  using FR = FftC<float, LM>;
+  using FC = FftC<float, LP>;
+  static constexpr int M = Gm::M, P = Gm::P;
+  static __device__ __forceinline__ constexpr int slot(int e) {
+    return FR::R0 == 0 ? e : FR::R0 == 2 ? (e >> 2) * 2 + (e & 1) : e >> 1;
+  }
+  template <int N> static __device__ __forceinline__ void group_sync(int g) {
+    if (N <= 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(N) : "memory");
+  }
+
+  struct Ctx {
+    const PassArgs<float>* a;
+    CoopShared* cs;
+    float2* work;
+    int R, rows, nb, blk;  // rows per CTA, rows in all, CTAs, this CTA
+    unsigned target;       // barrier count of the next barrier
+    int* bad;              // shared: a wait ran out
+    int magic;             // ceil(65536 / (R / 2))
+  };
+
+  // Every CTA's earlier global writes are visible to every CTA afterwards (read
+  // with L2 loads).  False: the wait ran out.
+  static __device__ __forceinline__ bool grid_sync(Ctx& c) {
+    __syncthreads();
+    c.target += c.nb;
+    if (threadIdx.x == 0) {
+      unsigned old;
+      asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(&c.cs->count) : "memory");
+      unsigned v = old + 1;
+      unsigned long long t0 = 0;
+      for (int i = 0; (int)(v - c.target) < 0; ++i) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&c.cs->count) : "memory");
+        if ((i & 1023) == 1023) {
+          const unsigned long long t = global_ns();
+          if (!t0) t0 = t;
+          else if (t - t0 > kMbarMaxNs) { *c.bad = 1; break; }
+        }
+      }
+    }
+    __syncthreads();
+    return *c.bad == 0;
+  }
+
+  // Rows: transform input x(row slot, element pair index) -> W.
+  template <class GetX>
+  static __device__ __forceinline__ void phase_a(Ctx& c, GetX&& getx) {
+    const PassArgs<float>& a = *c.a;
+    const int tid = threadIdx.x, b = tid / Gm::TR, t = tid % Gm::TR;
+    const float2* tw = reinterpret_cast<const float2*>(a.twA);
+    const float2* tws = reinterpret_cast<const float2*>(a.twS);
+    const int* sp = a.spA;
+    float2* W = reinterpret_cast<float2*>(a.W);
+    for (int r0 = 0; r0 < c.R; r0 += Gm::RPR) {
+      const int sl = r0 + b, row = c.blk * c.R + sl;
+      const bool ra = b < Gm::RPR && sl < c.R && row < c.rows;  // whole row groups
+      if (r0) __syncthreads();  // the previous rows' spectra are stored
+      if (ra) {
+        float2* buf = c.work + b * Gm::RS;
+        float2 v[8];
+        getx(sl, t, v);
+        FR::stage0_fwd(v, t, tw);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) buf[FR::ix0(t, e)] = v[e];
+        group_sync<Gm::TR>(b);
+#pragma unroll
+        for (int ls = FR::LS_TOP; ls >= 0; ls -= 3) {
+          FR::dif(buf, t, ls, tw);
+          group_sync<Gm::TR>(b);
+        }
+      }
+      __syncthreads();
+      const int rr = min(Gm::RPR, c.R - r0), rp = rr >> 1;  // even
+      const int magic = rr == c.R ? c.magic : (65535 + rp) / rp;
+      for (int idx = tid; idx < (M / 2 + 1) * rp; idx += Gm::NT) {
+        const int k = (idx * magic) >> 16, bb = 2 * (idx - k * rp);
+        const int y = c.blk * c.R + r0 + bb;
+        if (y >= c.rows) continue;
+        const float2* s0 = c.work + bb * Gm::RS;
+        const float2* s1 = s0 + Gm::RS;
+        const bool two = y + 1 < c.rows;
+        float2 xk0, xm0, xk1 = make_float2(0.f, 0.f), xm1 = make_float2(0.f, 0.f);
+        if (k == 0) {
+          const float2 z0 = s0[0];
+          xk0 = make_float2(z0.x + z0.y, 0.f);
+          xm0 = make_float2(z0.x - z0.y, 0.f);
+          if (two) {
+            const float2 z1 = s1[0];
+            xk1 = make_float2(z1.x + z1.y, 0.f);
+            xm1 = make_float2(z1.x - z1.y, 0.f);
+          }
+        } else {
+          const int pk = __ldg(sp + k), pm = __ldg(sp + M - k);
+          const float2 w = __ldg(tws + k);
+          split_two<float>(s0, pk, pm, w, xk0, xm0);
+          if (two) split_two<float>(s1, pk, pm, w, xk1, xm1);
+        }
+        const int km = k == 0 ? M : M - k;
+        // rows_w is even: the pair is inside W's row even where y + 1 is past the last row
+        __stcg(reinterpret_cast<float4*>(W + (size_t)k * a.rows_w + y), make_float4(xk0.x, xk0.y, xk1.x, xk1.y));
+        if (km != k)
+          __stcg(reinterpret_cast<float4*>(W + (size_t)km * a.rows_w + y), make_float4(xm0.x, xm0.y, xm1.x, xm1.y));
+      }
+    }
+  }
+
+  static __device__ __forceinline__ void phase_b(Ctx& c) {
+    const PassArgs<float>& a = *c.a;
+    constexpr int L = P, L8 = Gm::TC, hyq = L / 2 + 1;
+    const int tid = threadIdx.x, cc = tid / Gm::TC, t = tid % Gm::TC;
+    const float2* tw = reinterpret_cast<const float2*>(a.twB);
+    float2* W = reinterpret_cast<float2*>(a.W);
+    float2* cz = c.work + (cc < Gm::CPR ? cc : 0) * Gm::CZ;
+    const int k0 = (int)((long long)(M + 1) * c.blk / c.nb), k1 = (int)((long long)(M + 1) * (c.blk + 1) / c.nb);
+    const int sp0 = __ldg(a.spB + t);
+    for (int kb = k0; kb < k1; kb += Gm::CPR) {
+      const int kx = kb + cc;
+      if (cc >= Gm::CPR || kx >= k1) {
+        if (Gm::TC > 32) continue;  // whole column groups
+      }
+      float2* w = W + (size_t)kx * a.rows_w;
+      float2 v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        v[e] = make_float2(0.f, 0.f);
+        if (!FC::first_half(e)) continue;
+        const int y = FC::n0(t, e);
+        if (y < c.rows) v[e] = __ldcg(w + y);
+      }
+      FC::stage0_fwd(v, t, tw);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) cz[FC::ix0(t, e)] = v[e];
+      group_sync<Gm::TC>(cc);
+#pragma unroll
+      for (int ls = FC::LS_TOP; ls >= 3; ls -= 3) {
+        FC::dif(cz, t, ls, tw);
+        group_sync<Gm::TC>(cc);
+      }
+      {
+        const float* kc = a.khat + (size_t)kx * hyq;
+        float kf[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int ky = t + q * L8;
+          kf[q] = __ldg(kc + (ky <= (L >> 1) ? ky : L - ky));
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = cz[sp0 ^ r];
+        dft8<float, -1>(v);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = scale<float>(v[q], kf[q]);
+        dft8<float, 1>(v);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) cz[sp0 ^ r] = v[r];
+      }
+      group_sync<Gm::TC>(cc);
+#pragma unroll
+      for (int ls = 3; ls <= FC::LS_TOP; ls += 3) {
+        FC::dit(cz, t, ls, tw);
+        group_sync<Gm::TC>(cc);
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = cz[FC::ix0(t, e)];
+      FC::stage0_inv(v, t, tw);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        if (!FC::first_half(e)) continue;
+        const int y = FC::n0(t, e);
+        if (y < c.rows) __stcg(w + y, v[e]);
+      }
+    }
+  }
+
+  // Rows: W -> the inverse transform's values v (unscaled) of each row slot.
+  template <class Put>
+  static __device__ __forceinline__ void phase_c(Ctx& c, Put&& put) {
+    const PassArgs<float>& a = *c.a;
+    const int tid = threadIdx.x, b = tid / Gm::TR, t = tid % Gm::TR;
+    const float2* tw = reinterpret_cast<const float2*>(a.twA);
+    const float2* tws = reinterpret_cast<const float2*>(a.twS);
+    const int* sp = a.spA;
+    const float2* W = reinterpret_cast<const float2*>(a.W);
+    for (int r0 = 0; r0 < c.R; r0 += Gm::RPR) {
+      if (r0) __syncthreads();
+      const int rr = min(Gm::RPR, c.R - r0), rp = rr >> 1;
+      const int magic = rr == c.R ? c.magic : (65535 + rp) / rp;
+#pragma unroll 2
+      for (int idx = tid; idx < (M / 2 + 1) * rp; idx += Gm::NT) {
+        const int k = (idx * magic) >> 16, bb = 2 * (idx - k * rp);
+        const int y = c.blk * c.R + r0 + bb;
+        if (y >= c.rows) continue;
+        const float4 fk = __ldcg(reinterpret_cast<const float4*>(W + (size_t)k * a.rows_w + y));
+        const float4 fm = __ldcg(reinterpret_cast<const float4*>(W + (size_t)(M - k) * a.rows_w + y));
+        const int pk = __ldg(sp + k), pm = k ? __ldg(sp + M - k) : 0;
+        const float2 wk = conj<float>(__ldg(tws + k));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float2* s = c.work + (bb + h) * Gm::RS;
+          const float2 xk = h ? make_float2(fk.z, fk.w) : make_float2(fk.x, fk.y);
+          const float2 xm = h ? make_float2(fm.z, fm.w) : make_float2(fm.x, fm.y);
+          const float2 E = add<float>(xk, conj<float>(xm));
+          const float2 O = mul<float>(sub<float>(xk, conj<float>(xm)), wk);
+          s[pk] = add<float>(E, mul_si<float, 1>(O));
+          if (k != 0 && k != M - k) {
+            const float2 wm = make_float2(-wk.x, wk.y);
+            const float2 E2 = add<float>(xm, conj<float>(xk));
+            const float2 O2 = mul<float>(sub<float>(xm, conj<float>(xk)), wm);
+            s[pm] = add<float>(E2, mul_si<float, 1>(O2));
+          }
+        }
+      }
+      __syncthreads();
+      const int sl = r0 + b, row = c.blk * c.R + sl;
+      if (b < Gm::RPR && sl < c.R && row < c.rows) {
+        float2* buf = c.work + b * Gm::RS;
+#pragma unroll
+        for (int ls = 0; ls <= FR::LS_TOP; ls += 3) {
+          FR::dit(buf, t, ls, tw);
+          group_sync<Gm::TR>(b);
+        }
+        float2 v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = buf[FR::ix0(t, e)];
+        FR::stage0_inv(v, t, tw);
+        put(sl, t, v);
+      }
+    }
+  }
+
+  // Grid sums of NQ per-thread values: the totals (float-float) in every lane of
+  // warp 0 of every CTA, the same in all.  Includes a grid barrier.
+  template <int NQ>
+  static __device__ __forceinline__ bool sum(Ctx& c, const float* acc, float2* red, int* par, float2* v) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int nw = Gm::NT / 32;
+    float2* part = c.cs->part[*par];
+    *par ^= 1;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) v[q] = make_float2(acc[q], 0.f);
+    warp_sum_store<NQ>(v, red, 32, wid);
+    __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) v[q] = lane < nw ? red[q * 32 + lane] : make_float2(0.f, 0.f);
+      warp_sum_store<NQ>(v, part + c.blk * 8, 1, 0);
+    }
+    if (!grid_sync(c)) return false;
+    // one partial per lane of the first warps, then their sums
+    const int ns = (c.nb + 31) >> 5;
+    if (wid < ns) {
+      const int i = lane + 32 * wid;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) v[q] = i < c.nb ? __ldcg(part + i * 8 + q) : make_float2(0.f, 0.f);
+      warp_sum_store<NQ>(v, red, 32, wid);
+    }
+    __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) v[q] = lane < ns ? red[q * 32 + lane] : make_float2(0.f, 0.f);
+      warp_sum_ff<NQ>(v);
+    }
+    return true;
+  }
+
+  template <bool PK>
+  static __device__ __forceinline__ void loop(const CoopArgs& ca) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ Scalars sc;
+    __shared__ float2 red[5 * 32];
+    __shared__ int bad;
+    const PassArgs<float>& a = ca.one;
+    const int tid = threadIdx.x;
+    Ctx c;
+    c.a = &a;
+    c.cs = reinterpret_cast<CoopShared*>(ca.shared);
+    c.work = reinterpret_cast<float2*>(smem_raw);
+    c.R = ca.R;
+    c.rows = ca.rows;
+    c.nb = gridDim.x;
+    c.blk = blockIdx.x;
+    c.target = 0;
+    c.bad = &bad;
+    c.magic = (65535 + c.R / 2) / (c.R / 2);
+    float2* fld = c.work + Gm::work;  // [field][row slot][M/2] pairs: p, g, t, x (c or r)
+    const int pl = c.R * (M / 2);
+    float2 *fp = fld, *fg = fld + pl, *ft = fld + 2 * pl, *fx = fld + 3 * pl;
+    if (tid == 0) bad = 0;
+    for (int i = tid; i < (int)(sizeof(Scalars) / 4); i += Gm::NT)
+      reinterpret_cast<int*>(&sc)[i] = __ldcg(reinterpret_cast<const int*>(a.sc) + i);
+    const int nx = a.pl.nx;
+    const int b = tid / Gm::TR, t = tid % Gm::TR;
+    const float us = (float)a.uscale;
+    int par = 0;
+    unsigned on = 0, S = 0;  // 8 bits per round of rows: on the grid, in the held set
+    for (int r0 = 0, rd = 0; r0 < c.R; r0 += Gm::RPR, ++rd) {
+      const int sl = r0 + b, row = c.blk * c.R + sl;
+      if (!(b < Gm::RPR && sl < c.R)) continue;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        if (!FR::first_half(e)) continue;
+        const int n = FR::n0(t, e);
+        float vp[2] = {0, 0}, vg[2] = {0, 0}, vt[2] = {0, 0}, vx[2] = {0, 0};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int col = 2 * n + h;
+          if (row < c.rows && col < nx) {
+            const size_t j = (size_t)row * nx + col;
+            const unsigned bit = 1u << (8 * rd + 2 * slot(e) + h);
+            on |= bit;
+            if (PK) {
+              vp[h] = a.f.p[j];
+              vx[h] = a.f.c[j];
+              if (ca.resume) { vt[h] = a.f.t[j]; vg[h] = a.f.g[j]; }
+            } else if (a.f.S[j]) {
+              S |= bit;
+              vp[h] = a.f.p[j];
+              if (ca.resume) { vg[h] = a.f.g[j]; vt[h] = a.f.t[j]; vx[h] = a.f.r[j]; }
+              else vx[h] = a.f.c[j];
+            }
+          }
+        }
+        const int i = sl * (M / 2) + n;
+        if (n < M / 2) {
+          fp[i] = make_float2(vp[0], vp[1]); fg[i] = make_float2(vg[0], vg[1]);
+          ft[i] = make_float2(vt[0], vt[1]); fx[i] = make_float2(vx[0], vx[1]);
+        }
+      }
+    }
+    __syncthreads();
+    bool ok = true;
+    float2 v5[5];
+    if (!PK && !ca.resume) {  // the initial residual
+      phase_a(c, [&](int sl, int t_, float2* v) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          v[e] = FR::first_half(e) ? fp[sl * (M / 2) + FR::n0(t_, e)] : make_float2(0.f, 0.f);
+      });
+      ok = grid_sync(c);
+      if (ok) { phase_b(c); ok = grid_sync(c); }
+      float acc[2] = {0.f, 0.f};
+      if (ok) {
+        phase_c(c, [&](int sl, int t_, float2* v) {
+          const unsigned Sr = S >> (8 * (sl / Gm::RPR));
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            if (!FR::first_half(e)) continue;
+            const int i = sl * (M / 2) + FR::n0(t_, e);
+            const float2 cv = fx[i];
+            float2 gv;
+            gv.x = Sr >> (2 * slot(e)) & 1 ? us * v[e].x + cv.x : 0.f;
+            gv.y = Sr >> (2 * slot(e) + 1) & 1 ? us * v[e].y + cv.y : 0.f;
+            acc[0] += gv.x * gv.x + gv.y * gv.y;
+            acc[1] += cv.x * cv.x + cv.y * cv.y;
+            fg[i] = gv;
+            fx[i] = make_float2(0.f, 0.f);
+          }
+        });
+        ok = sum<2>(c, acc, red, &par, v5);
+        if (ok && tid < 32) finalize_cg_g(&sc, v5);
+        __syncthreads();
+      }
+    }
+    for (int it = 0; ok && it < ca.max_launch && !sc.done; ++it) {
+      const bool upd = sc.have_tau != 0;
+      const float tau = (float)sc.tau;
+      if (PK) {
+        float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+        phase_a(c, [&](int sl, int t_, float2* v) {
+          const unsigned onr = on >> (8 * (sl / Gm::RPR));
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            v[e] = make_float2(0.f, 0.f);
+            if (!FR::first_half(e)) continue;
+            const int i = sl * (M / 2) + FR::n0(t_, e);
+            float2 pv = fp[i];
+            const float2 tv = ft[i], gv = fg[i];
+            PIn<float> q;
+            if (onr >> (2 * slot(e)) & 1) {
+              q.p = pv.x; q.t = tv.x; q.g = gv.x;
+              pv.x = pro_value<float, A_PK_P>(q, upd, tau, 0.f, acc);
+            }
+            if (onr >> (2 * slot(e) + 1) & 1) {
+              q.p = pv.y; q.t = tv.y; q.g = gv.y;
+              pv.y = pro_value<float, A_PK_P>(q, upd, tau, 0.f, acc);
+            }
+            if (upd) fp[i] = pv;
+            v[e] = pv;
+          }
+        });
+        if (!(ok = grid_sync(c))) break;
+        phase_b(c);
+        if (!(ok = grid_sync(c))) break;
+        phase_c(c, [&](int sl, int t_, float2* v) {
+          const unsigned onr = on >> (8 * (sl / Gm::RPR));
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            if (!FR::first_half(e)) continue;
+            const int i = sl * (M / 2) + FR::n0(t_, e);
+            const float2 cv = fx[i], pv = fp[i];
+            float2 gv = make_float2(0.f, 0.f);
+            if (onr >> (2 * slot(e)) & 1) {
+              gv.x = us * v[e].x + cv.x;
+              if (pv.x > 0.f) { acc[3] += gv.x * gv.x; acc[4] += 1.f; }
+            }
+            if (onr >> (2 * slot(e) + 1) & 1) {
+              gv.y = us * v[e].y + cv.y;
+              if (pv.y > 0.f) { acc[3] += gv.y * gv.y; acc[4] += 1.f; }
+            }
+            fg[i] = gv;
+          }
+        });
+        if (!(ok = sum<5>(c, acc, red, &par, v5))) break;
+        if (tid < 32) finalize_pk_g(&sc, v5);
+        __syncthreads();
+        if (sc.done) break;
+        const float beta = (float)sc.beta;
+        phase_a(c, [&](int sl, int t_, float2* v) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            v[e] = make_float2(0.f, 0.f);
+            if (!FR::first_half(e)) continue;
+            const int i = sl * (M / 2) + FR::n0(t_, e);
+            const float2 pv = fp[i], gv = fg[i];
+            float2 tv = ft[i];
+            tv.x = pv.x > 0.f ? gv.x + beta * tv.x : 0.f;
+            tv.y = pv.y > 0.f ? gv.y + beta * tv.y : 0.f;
+            ft[i] = tv;
+            v[e] = tv;
+          }
+        });
+        if (!(ok = grid_sync(c))) break;
+        phase_b(c);
+        if (!(ok = grid_sync(c))) break;
+        float ac2[2] = {0.f, 0.f};
+        phase_c(c, [&](int sl, int t_, float2* v) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            if (!FR::first_half(e)) continue;
+            const int i = sl * (M / 2) + FR::n0(t_, e);
+            const float2 pv = fp[i], gv = fg[i], tv = ft[i];
+            if (pv.x > 0.f) { ac2[0] += gv.x * tv.x; ac2[1] += us * v[e].x * tv.x; }
+            if (pv.y > 0.f) { ac2[0] += gv.y * tv.y; ac2[1] += us * v[e].y * tv.y; }
+          }
+        });
+        if (!(ok = sum<2>(c, ac2, red, &par, v5))) break;
+        if (tid < 32) finalize_pk_r(&sc, v5);
+        __syncthreads();
+      } else {
+        const float beta = (float)sc.beta;
+        phase_a(c, [&](int sl, int t_, float2* v) {
+          const unsigned Sr = S >> (8 * (sl / Gm::RPR));
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            v[e] = make_float2(0.f, 0.f);
+            if (!FR::first_half(e)) continue;
+            const int i = sl * (M / 2) + FR::n0(t_, e);
+            float2 gv = fg[i], tv = ft[i];
+            if (upd) {
+              const float2 xv = fx[i];
+              float2 pv = fp[i];
+              pv.x -= tau * tv.x; pv.y -= tau * tv.y;
+              gv.x -= tau * xv.x; gv.y -= tau * xv.y;
+              fp[i] = pv;
+              fg[i] = gv;
+            }
+            tv.x = Sr >> (2 * slot(e)) & 1 ? gv.x + beta * tv.x : 0.f;
+            tv.y = Sr >> (2 * slot(e) + 1) & 1 ? gv.y + beta * tv.y : 0.f;
+            ft[i] = tv;
+            v[e] = tv;
+          }
+        });
+        if (!(ok = grid_sync(c))) break;
+        phase_b(c);
+        if (!(ok = grid_sync(c))) break;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        phase_c(c, [&](int sl, int t_, float2* v) {
+          const unsigned Sr = S >> (8 * (sl / Gm::RPR));
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            if (!FR::first_half(e)) continue;
+            const int i = sl * (M / 2) + FR::n0(t_, e);
+            const float2 gv = fg[i], tv = ft[i];
+            float2 rv;
+            rv.x = Sr >> (2 * slot(e)) & 1 ? us * v[e].x : 0.f;
+            rv.y = Sr >> (2 * slot(e) + 1) & 1 ? us * v[e].y : 0.f;
+            fx[i] = rv;
+            acc[0] += rv.x * tv.x; acc[1] += rv.x * gv.x; acc[2] += rv.x * rv.x; acc[3] += gv.x * gv.x;
+            acc[0] += rv.y * tv.y; acc[1] += rv.y * gv.y; acc[2] += rv.y * rv.y; acc[3] += gv.y * gv.y;
+          }
+        });
+        if (!(ok = sum<4>(c, acc, red, &par, v5))) break;
+        if (tid < 32) finalize_cg_r(&sc, v5);
+        __syncthreads();
+      }
+    }
+    if (!ok) {  // a wait ran out: give up together
+      if (tid == 0 && a.kerr) atomicOr(a.kerr, 1u);
+      return;
+    }
+    // a fixed-set solve may end with its last update pending
+    const bool fin = !PK && sc.done && sc.have_tau;
+    const float tau = (float)sc.tau;
+    for (int r0 = 0; r0 < c.R; r0 += Gm::RPR) {
+      const int sl = r0 + b, row = c.blk * c.R + sl;
+      if (!(b < Gm::RPR && sl < c.R && row < c.rows)) continue;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        if (!FR::first_half(e)) continue;
+        const int n = FR::n0(t, e), i = sl * (M / 2) + n;
+        const float2 tv = ft[i], xv = fx[i];
+        float2 pv = fp[i], gv = fg[i];
+        if (fin) {
+          pv.x -= tau * tv.x; pv.y -= tau * tv.y;
+          gv.x -= tau * xv.x; gv.y -= tau * xv.y;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int col = 2 * n + h;
+          if (col >= nx) continue;
+          const size_t j = (size_t)row * nx + col;
+          a.f.p[j] = h ? pv.y : pv.x;
+          a.f.g[j] = h ? gv.y : gv.x;
+          a.f.t[j] = h ? tv.y : tv.x;
+          if (!PK) a.f.r[j] = h ? xv.y : xv.x;
+        }
+      }
+    }
+    // rows past c.rows hold no pressure
+    for (size_t i = (size_t)c.rows * nx + (size_t)blockIdx.x * Gm::NT + tid; i < (size_t)a.pl.ny * nx;
+         i += (size_t)c.nb * Gm::NT)
+      a.f.p[i] = 0.f;
+    if (blockIdx.x == 0) {  // the scalars, all but the sticky error word
+      __syncthreads();
+      if (tid == 0 && fin) sc.have_tau = 0;
+      __syncthreads();
+      for (int i = tid; i < (int)(offsetof(Scalars, kerr) / 4); i += Gm::NT)
+        reinterpret_cast<int*>(a.sc)[i] = reinterpret_cast<const int*>(&sc)[i];
+    }
+  }
+};
+
+template <int LM, int LP, bool PK>
+__global__ void __launch_bounds__(CoopGeo<LM, LP>::NT, 1) k_coop(const __grid_constant__ CoopArgs r) {
+  Coop<LM, LP>::template loop<PK>(r);
+}
+
+#define BEM_COOP_CASES(X) X(8, 9) X(8, 10) X(8, 11) X(9, 9) X(9, 10) X(9, 11) X(10, 9) X(10, 10) X(10, 11)
+
+template <int LM, int LP>
+constexpr size_t coop_smem(int R) { return 8 * (size_t)CoopGeo<LM, LP>::work + 16 * (size_t)R * CoopGeo<LM, LP>::M; }
+
+// CTAs and rows per CTA of the loop over `rows` rows: as many CTAs as give every
+// one a round of columns, at most one per SM; an even number of rows each, so
+// that W is read and written in 16-byte pairs.
+template <int LM, int LP>
+inline void coop_shape(int rows, int nsm, int* nb, int* R) {
+  using Gm = CoopGeo<LM, LP>;
+  *nb = std::min(std::min(nsm, 256), (Gm::M + 1 + Gm::CPR - 1) / Gm::CPR);
+  *R = 2 * std::max(1, (rows + 2 * *nb - 1) / (2 * *nb));
+}
+
+template <bool PK>
+cudaError_t launch_coop_kind(CoopArgs r, int lm, int lp, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  // a fresh barrier for every launch
+  cudaError_t e = cudaMemsetAsync(r.shared, 0, 2 * sizeof(unsigned int), s);
+  if (e != cudaSuccess) return e;
+  switch (lm * 16 + lp) {
+#define BEM_CASE(LM, LP)                                                     \
+  case LM * 16 + LP: {                                                       \
+    int nb = 0;                                                              \
+    coop_shape<LM, LP>(r.rows, r.one.pl.nsm, &nb, &r.R);                     \
+    if (r.R > CoopGeo<LM, LP>::RMAX) return cudaErrorInvalidValue;           \
+    cfg.gridDim = dim3(nb);                                                  \
+    cfg.blockDim = dim3(CoopGeo<LM, LP>::NT);                                \
+    cfg.dynamicSmemBytes = coop_smem<LM, LP>(r.R);                           \
+    return cudaLaunchKernelEx(&cfg, k_coop<LM, LP, PK>, r);                  \
+  }
+    BEM_COOP_CASES(BEM_CASE)
+#undef BEM_CASE
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <bool PK>
+cudaError_t coop_setup_kind() {
+  cudaError_t e = cudaSuccess, r;
+#define BEM_CASE(LM, LP) \
+  if ((r = set_smem_max(k_coop<LM, LP, PK>, 227 * 1024)) != cudaSuccess && e == cudaSuccess) e = r;
+  BEM_COOP_CASES(BEM_CASE)
+#undef BEM_CASE
+  return e;
+}
+
+}  // namespace bem

@@ -85,6 +85,8 @@ constexpr int kChunk = BEM_CHUNK;  // CG iterations per captured graph launch
 #define BEM_LOOP_BODY 4
 #endif
 constexpr int kLoopBody = BEM_LOOP_BODY;
+// CG iterations of one launch of a resident loop (resident.cuh) at most
+constexpr int kResidentIters = 4096;
 
 // Threads per CTA of the row passes (rows per CTA x M/8); 512 keeps two CTAs
 // resident per SM at the passes' register use.
@@ -199,6 +201,13 @@ Plan default_plan(int nx, int ny, int px, int py, int esize, int nsm) {
 }
 bool plan_fits(const Plan& pl, int esize) { return shape_fits(pl, esize); }
 
+// Devices whose clusters hold the resident loops (set once by device_setup).
+static bool g_resident[64] = {};
+// ... and whether it takes cooperative launches; one cooperative loop runs on a
+// device at a time (its CTAs wait for one another and fill the SMs).
+static bool g_coop[64] = {};
+static std::mutex g_coop_mu[64];
+
 // Once per device and process, with that device current: opt every pass kernel
 // into the shared memory it may ask for, and upload the quadrature nodes.
 int device_setup(int dev) {
@@ -220,6 +229,13 @@ int device_setup(int dev) {
   if (influence_init_nodes() != 0) return fail(BEM_ECUDA, "quadrature nodes upload failed");
   const int rc = tc_column_pass_setup();
   if (rc != BEM_OK) return rc;
+  bool cg = false, pk = false;
+  if (resident_setup_cg(&cg) != cudaSuccess || resident_setup_pk(&pk) != cudaSuccess) cudaGetLastError();
+  g_resident[dev] = cg && pk;
+  int coop = 0;
+  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) cudaGetLastError();
+  g_coop[dev] = coop && coop_setup_cg() == cudaSuccess && coop_setup_pk() == cudaSuccess;
+  if (!g_coop[dev]) cudaGetLastError();
   init_done[dev] = true;
   return BEM_OK;
 }
@@ -270,6 +286,8 @@ struct bem_ctx {
   // CG loops join this batcher when set (concurrent solves of the server)
   bem::LoopBatcher* batcher = nullptr;
   cudaEvent_t ev_ready = nullptr;  // this context's work before its batched loop
+  void* coop = nullptr;  // barrier and partial sums of the cooperative CG loop
+  int rows_used = 0;     // sub-contexts: rows of the box (pressure lies in rows 0 .. rows_used - 1)
   // Tensor map of W (FP32) for pass C's TMA staging, with the plan's rows per
   // CTA (device memory; null where TMA does not apply)
   void* tmw = nullptr;
@@ -664,6 +682,9 @@ void attach_batcher(::bem_ctx* h, LoopBatcher* b) {
 
 namespace {
 
+bool resident_applies(const bem_ctx* h, int es);
+cudaError_t launch_resident(const ResArgs& r, const bem_ctx* h, bool pk, int n, cudaStream_t s);
+
 // Size class of a loop request: requests with equal keys share every launch
 // shape, so one several-instance launch per pass serves them all.
 std::vector<int> loop_key(const LoopReq& r) {
@@ -738,13 +759,21 @@ int launch_group(LoopBatcher* b, std::vector<LoopReq*>& g, const std::vector<int
   gk.push_back(n);
   LoopBatcher::Entry& en = b->graphs[gk];
   if (!en.d_args) CK(cudaMalloc(&en.d_args, sizeof(PassArgs<T>) * (size_t)n));
-  if (!en.exec) {
+  const bool resident = resident_applies(g[0]->h, (int)sizeof(T));
+  if (!resident && !en.exec) {
     CKR(capture_loop_mi<T>(b, host[0], g[0]->pk, n,
                            reinterpret_cast<const PassArgs<T>*>(en.d_args), &en.exec));
   }
   // pageable source: the copy is staged before the call returns
   CK(cudaMemcpyAsync(en.d_args, host.data(), sizeof(PassArgs<T>) * (size_t)n, cudaMemcpyHostToDevice, b->stream));
-  CK(cudaGraphLaunch(en.exec, b->stream));
+  if (resident) {
+    ResArgs r{};
+    r.arr = reinterpret_cast<const PassArgs<float>*>(en.d_args);
+    r.max_launch = kResidentIters;
+    CK(launch_resident(r, g[0]->h, g[0]->pk, n, b->stream));
+  } else {
+    CK(cudaGraphLaunch(en.exec, b->stream));
+  }
   b->launches += 1;
   b->instances += n;
   CK(cudaEventRecord(b->ev, b->stream));
@@ -816,6 +845,10 @@ int run_loop_batched(bem_ctx* h, bool pk, int es, bool* solo) {
   *solo = r.solo;
   if (r.solo) return BEM_OK;
   CKR(read_scalars(h));
+  if (resident_applies(h, es)) {
+    h->launches += 1;
+    return BEM_OK;
+  }
   const int ran = h->sc_host->loops - loops0 + 1;
   h->launches += (unsigned long long)((ran + kLoopBody - 1) / kLoopBody) * kLoopBody * (pk ? 6 : 3);
   if (!h->sc_host->done) return fail(BEM_ECUDA, "a batched CG loop stopped before the solve was done");
@@ -864,6 +897,75 @@ int run_loop(bem_ctx* h, cudaGraphExec_t g, cudaGraphExec_t g_timed, int max_ite
   return BEM_OK;
 }
 
+// Whether this context's CG loops in precision es run inside one cluster: FP32,
+// grids of at most 256 x 256 (the cluster's sixteen SMs hold and transform them
+// faster than the chip-wide passes start and end; above that the passes win).
+// Pass timing needs the separate passes.
+bool resident_applies(const bem_ctx* h, int es) {
+  return es == 4 && h->px <= 512 && h->py <= 512 && !h->timing && g_resident[h->device];
+}
+
+// One cluster launch over n instances (arr) or this context alone; a launch runs
+// at most kResidentIters iterations, so that no kernel runs without end.
+cudaError_t launch_resident(const ResArgs& r, const bem_ctx* h, bool pk, int n, cudaStream_t s) {
+  const int lm = ilog2(h->px / 2), lp = ilog2(h->py);
+  return pk ? launch_resident_pk(r, lm, lp, n, s) : launch_resident_cg(r, lm, lp, n, s);
+}
+
+// Whether the loop may run as one cooperative launch over the chip (coop.cuh):
+// FP32, row transforms of 256 to 1024 points and columns of 512 to 2048, the
+// sizes at which the passes' starts and tails cost as much as their work.  The
+// server's loops share launches instead.
+bool coop_applies(const bem_ctx* h, int es) {
+  return es == 4 && h->px >= 512 && h->px <= 2048 && h->py >= 512 && h->py <= 2048 && (h->ny & 1) == 0 &&
+         !h->timing && !h->batcher && g_coop[h->device];
+}
+
+// The whole CG loop over `rows` grid rows as cooperative launches.  *ran = false:
+// another one is running on this device; the caller takes the passes.
+int run_coop(bem_ctx* h, bool pk, int rows, bool* ran) {
+  std::unique_lock<std::mutex> lk(g_coop_mu[h->device], std::try_to_lock);
+  *ran = lk.owns_lock();
+  if (!*ran) return BEM_OK;
+  if (!h->coop) CKR(dmalloc(h, &h->coop, coop_shared_bytes()));
+  CoopArgs r{};
+  r.one = make_args<float>(h);
+  r.shared = h->coop;
+  r.rows = rows < 1 ? 1 : rows;
+  r.max_launch = kResidentIters;
+  const int lm = ilog2(h->px / 2), lp = ilog2(h->py);
+  do {
+    CK(pk ? launch_coop_pk(r, lm, lp, h->stream) : launch_coop_cg(r, lm, lp, h->stream));
+    h->launches += 1;
+    CKR(read_scalars(h));
+    r.resume = 1;
+  } while (!h->sc_host->done);
+  return BEM_OK;
+}
+
+// The whole CG loop (fixed-set: with its initial residual and final update) as
+// cluster launches, batched with the loops of other solves where they wait.
+int run_resident(bem_ctx* h, bool pk) {
+  bool solo = true;
+  if (h->batcher) CKR(run_loop_batched(h, pk, 4, &solo));
+  ResArgs r{};
+  r.one = make_args<float>(h);
+  r.max_launch = kResidentIters;
+  r.resume = solo ? 0 : 1;
+  if (solo) {
+    CK(launch_resident(r, h, pk, 1, h->stream));
+    h->launches += 1;
+    CKR(read_scalars(h));
+  }
+  while (!h->sc_host->done) {
+    r.resume = 1;
+    CK(launch_resident(r, h, pk, 1, h->stream));
+    h->launches += 1;
+    CKR(read_scalars(h));
+  }
+  return BEM_OK;
+}
+
 struct StepOut {
   int iterations = 0;
   double eps = 0;
@@ -898,12 +1000,20 @@ int run_pk(bem_ctx* h, double d, double tol, int max_iter, bool warm, StepOut* s
     CKR(pick_sub(h, &sub));
     if (sub) return pk_in_box<T>(h, sub, d, tol, max_iter, warm, so);
   }
-  if (!pf.pk_graph[0]) CKR(capture_chunk<T>(h, true, false, &pf.pk_graph[0]));
-  if (h->timing && !pf.pk_graph[1]) CKR(capture_chunk<T>(h, true, true, &pf.pk_graph[1]));
   launch_pk_init<T>(plan_of<T>(h), h->h64, d, pf.c, pf.p, pf.t, warm ? 1 : 0, h->ew_ngrid, h->stream);
   h->launches += 1;
   CKR(init_scalars(h, tol, max_iter, 0.0));
-  CKR(run_loop(h, pf.pk_graph[0], pf.pk_graph[1], max_iter, true, (int)sizeof(T)));
+  bool ran = false;
+  if (coop_applies(h, (int)sizeof(T))) CKR(run_coop(h, true, h->is_sub ? h->rows_used : h->ny, &ran));
+  if (!ran && resident_applies(h, (int)sizeof(T))) {
+    CKR(run_resident(h, true));
+    ran = true;
+  }
+  if (!ran) {
+    if (!pf.pk_graph[0]) CKR(capture_chunk<T>(h, true, false, &pf.pk_graph[0]));
+    if (h->timing && !pf.pk_graph[1]) CKR(capture_chunk<T>(h, true, true, &pf.pk_graph[1]));
+    CKR(run_loop(h, pf.pk_graph[0], pf.pk_graph[1], max_iter, true, (int)sizeof(T)));
+  }
   so->iterations += h->sc_host->iter;
   so->eps = h->sc_host->eps;
   if (h->sc_host->status != SC_OK) so->status = map_status(h->sc_host->status);
@@ -981,6 +1091,7 @@ void absorb_sub(bem_ctx* h, bem_ctx* sub) {
 template <typename T>
 int pk_in_box(bem_ctx* h, bem_ctx* sub, double d, double tol, int max_iter, bool warm, StepOut* so) {
   const int x0 = h->sc_host->col0, y0 = h->sc_host->band0;
+  sub->rows_used = h->sc_host->band1 - y0 + 1;
   const size_t n = (size_t)h->nx * h->ny;
   PrecFields<T>& pf = fields_of<T>(h);
   CKR(ensure_fields<T>(sub));
@@ -1016,6 +1127,7 @@ int pk_in_box(bem_ctx* h, bem_ctx* sub, double d, double tol, int max_iter, bool
 template <typename T>
 int fixed_cg_in_box(bem_ctx* h, bem_ctx* sub, double tol, int max_iter, double pcrit, StepOut* so) {
   const int x0 = h->sc_host->col0, y0 = h->sc_host->band0;
+  sub->rows_used = h->sc_host->band1 - y0 + 1;
   PrecFields<T>& pf = fields_of<T>(h);
   CKR(ensure_fields<T>(sub));
   PrecFields<T>& bf = fields_of<T>(sub);
@@ -1041,36 +1153,56 @@ int run_fixed_cg(bem_ctx* h, double tol, int max_iter, double pcrit, StepOut* so
   CKR(ensure_fields<T>(h));
   PrecFields<T>& pf = fields_of<T>(h);
   CKR(init_scalars(h, tol, max_iter, pcrit));
-  launch_box(plan_of<T>(h), h->S, h->sc, h->stream);
-  h->launches += 1;
+  const bool coop = coop_applies(h, (int)sizeof(T)), resident = resident_applies(h, (int)sizeof(T));
+  bool boxed = !h->is_sub || !(coop || resident);
+  if (boxed) {
+    launch_box(plan_of<T>(h), h->S, h->sc, h->stream);
+    h->launches += 1;
+  }
+  int rows = h->rows_used;
   if (!h->is_sub) {
     CKR(read_scalars(h));
+    rows = h->sc_host->band1 + 1;
     bem_ctx* sub = nullptr;
     CKR(pick_sub(h, &sub));
     if (sub) return fixed_cg_in_box<T>(h, sub, tol, max_iter, pcrit, so);
   }
-  if (!pf.cg_graph[0]) CKR(capture_chunk<T>(h, false, false, &pf.cg_graph[0]));
-  if (h->timing && !pf.cg_graph[1]) CKR(capture_chunk<T>(h, false, true, &pf.cg_graph[1]));
-  const size_t n = (size_t)h->nx * h->ny;
-  launch_mask_field<T>(pf.p, h->S, n, h->stream);
-  launch_mask_field<T>(pf.t, h->S, n, h->stream);
-  PassArgs<T> a = make_args<T>(h);
-  a.f.src = pf.p;
-  launch_pass_a<T>(a, A_PLAIN, h->stream);
-  launch_pass_b<T>(a, B_CONV, h->stream);
-  launch_pass_c<T>(a, C_CG_G, h->stream);
-  h->launches += 5;
-  CKR(read_scalars(h));
-  if (!h->sc_host->done) {
-    CKR(run_loop(h, pf.cg_graph[0], pf.cg_graph[1], max_iter, false, (int)sizeof(T)));
-    if (h->sc_host->have_tau) {
-      Fields<T> f = a.f;
-      launch_cg_finish<T>(a.pl, f, h->sc, h->ew_ngrid, h->stream);
+  bool ran = false;
+  if (coop) CKR(run_coop(h, false, rows, &ran));
+  if (!ran && resident) {
+    CKR(run_resident(h, false));
+    ran = true;
+  }
+  if (ran) {
+    so->eps = h->sc_host->iter > 0 ? sqrt(std::max(h->sc_host->G, 0.0)) / h->sc_host->bnorm : h->sc_host->eps;
+  } else {
+    if (!boxed) {  // the passes work on the contact band
+      launch_box(plan_of<T>(h), h->S, h->sc, h->stream);
       h->launches += 1;
     }
-    so->eps = sqrt(std::max(h->sc_host->G, 0.0)) / h->sc_host->bnorm;
-  } else {
-    so->eps = h->sc_host->eps;
+    if (!pf.cg_graph[0]) CKR(capture_chunk<T>(h, false, false, &pf.cg_graph[0]));
+    if (h->timing && !pf.cg_graph[1]) CKR(capture_chunk<T>(h, false, true, &pf.cg_graph[1]));
+    const size_t n = (size_t)h->nx * h->ny;
+    launch_mask_field<T>(pf.p, h->S, n, h->stream);
+    launch_mask_field<T>(pf.t, h->S, n, h->stream);
+    PassArgs<T> a = make_args<T>(h);
+    a.f.src = pf.p;
+    launch_pass_a<T>(a, A_PLAIN, h->stream);
+    launch_pass_b<T>(a, B_CONV, h->stream);
+    launch_pass_c<T>(a, C_CG_G, h->stream);
+    h->launches += 5;
+    CKR(read_scalars(h));
+    if (!h->sc_host->done) {
+      CKR(run_loop(h, pf.cg_graph[0], pf.cg_graph[1], max_iter, false, (int)sizeof(T)));
+      if (h->sc_host->have_tau) {
+        Fields<T> f = a.f;
+        launch_cg_finish<T>(a.pl, f, h->sc, h->ew_ngrid, h->stream);
+        h->launches += 1;
+      }
+      so->eps = sqrt(std::max(h->sc_host->G, 0.0)) / h->sc_host->bnorm;
+    } else {
+      so->eps = h->sc_host->eps;
+    }
   }
   so->iterations += h->sc_host->iter;
   if (h->sc_host->status != SC_OK) so->status = map_status(h->sc_host->status);
@@ -1202,6 +1334,7 @@ int refine(bem_ctx* h, double d, bool adhesive, int sweeps, double tol64, double
                                 sub->nx, sub->ny, h->stream);
       launch_box_copy64(h->h64, h->nx, h->ny, x0, y0, sub->h64, sub->nx, sub->ny, 1.0e6, h->stream);
       sub->timing = h->timing;
+      sub->rows_used = b1 - b0 + 1;
       CKR(refine_here(sub, d, adhesive, sweeps, tol64, tol32, so, 0, b1 - b0));
       launch_box_scatter<double>(sub->io64, h->io64, h->nx, h->ny, x0, y0, sub->nx, sub->ny, h->stream);
       h->launches += 3;
@@ -1510,7 +1643,7 @@ extern "C" void bem_destroy(bem_handle h) {
     for (int j = 0; j < 4; ++j)
       if (h->ev[i][j]) cudaEventDestroy(h->ev[i][j]);
   if (h->ev_ready) cudaEventDestroy(h->ev_ready);
-  fr(h->tmw);
+  fr(h->tmw); fr(h->coop);
   fr(h->kq64); fr(h->geo); fr(h->tw64); fr(h->tw32); fr(h->twfx); fr(h->fxe); fr(h->khat64); fr(h->khat32); fr(h->W); fr(h->h64); fr(h->io64); fr(h->io64b);
   fr(h->S); fr(h->part); fr(h->partC); fr(h->partE); fr(h->stats); fr(h->sc);
   fr(h->f32.p); fr(h->f32.g); fr(h->f32.t); fr(h->f32.r); fr(h->f32.c);
