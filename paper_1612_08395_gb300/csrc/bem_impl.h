@@ -82,7 +82,8 @@ enum PassAMode {
   A_PK_P = 1,   // Polonsky-Keer update of p (steps 7-8), partials sum|dp|, sum p, #overlap
   A_PK_T = 2,   // t = (p > 0) ? g + beta t : 0
   A_CG_T = 3,   // fixed-set CG: p -= tau t, g -= tau r (the previous step, if any), t = S ? g + beta t : 0
-  A_TORUS = 4   // x = K on the even torus (spectrum set-up, FP64)
+  A_TORUS = 4,  // x = K on the even torus (spectrum set-up, FP64)
+  A_PLAIN64 = 5 // FP32: x = src64 (a field of doubles)
 };
 // Pass C (row complex-to-real FFT) epilogue modes.
 enum PassCMode {
@@ -91,7 +92,8 @@ enum PassCMode {
   C_PK_R = 2,   // partials sum_{p>0} g t, sum_{p>0} r t; last block: tau
   C_CG_R = 3,   // r = S ? u : 0 (stored); partials t.r, g.r, r.r, g.g; last block: stop test, tau, beta
   C_CG_G = 4,   // g = S ? u + c : 0; partials sum g^2, sum_S c^2; last block: G, bnorm
-  C_GAP = 5     // g = u + c (no mask) -- FP64 residual of the refinement
+  C_GAP = 5,    // g = u + c (no mask) -- FP64 residual of the refinement
+  C_PLAIN64 = 6 // FP32: dst64 = u (a field of doubles)
 };
 enum PassBMode { B_CONV = 0, B_SPECTRUM = 1 };
 
@@ -105,6 +107,8 @@ struct Fields {
   uint8_t* S;  // fixed contact set (adhesive / refinement)
   const T* src;  // A_PLAIN source
   T* dst;        // C_PLAIN destination
+  const double* src64;  // A_PLAIN64 source
+  double* dst64;        // C_PLAIN64 destination
 };
 
 template <typename T>
@@ -243,7 +247,6 @@ template <typename T> void launch_detach(const Plan& pl, Fields<T> f, double* pa
 template <typename T> void launch_stats(const Plan& pl, const T* p, const T* g, const uint8_t* S,
                                         int use_set, double* part, double* out, int ngrid,
                                         cudaStream_t s);
-template <typename T> void launch_convert_in(const double* src, T* dst, size_t n, cudaStream_t s);
 template <typename T> void launch_convert_out(const T* src, double* dst, size_t n, cudaStream_t s);
 template <typename T> void launch_offset(const double* h64, double d, T* c, size_t n, cudaStream_t s);
 template <typename T> void launch_set_from_p(const T* p, uint8_t* S, size_t n, cudaStream_t s);

@@ -173,6 +173,8 @@ template <typename T, int MODE>
 __device__ __forceinline__ void pro_gather(const PassArgs<T>& a, size_t i, PIn<T>& x) {
   if (MODE == A_PLAIN) {
     x.p = __ldg(a.f.src + i);
+  } else if (MODE == A_PLAIN64) {
+    x.p = (T)__ldg(a.f.src64 + i);
   } else if (MODE == A_PK_P) {
     x.p = a.f.p[i]; x.t = a.f.t[i]; x.g = a.f.g[i];
   } else if (MODE == A_PK_T) {
@@ -199,7 +201,7 @@ __device__ __forceinline__ T* pro_out(const PassArgs<T>& a) {
 // mode also stores back into pro_out), without the store.
 template <typename T, int MODE>
 __device__ __forceinline__ T pro_value(PIn<T>& x, bool upd, T tau, T beta, T* acc) {
-  if (MODE == A_PLAIN) {
+  if (MODE == A_PLAIN || MODE == A_PLAIN64) {
     return x.p;
   } else if (MODE == A_PK_P) {
     T q = x.p;
@@ -227,7 +229,7 @@ __device__ __forceinline__ T pro_value(PIn<T>& x, bool upd, T tau, T beta, T* ac
 template <typename T, int MODE>
 __device__ __forceinline__ T pro_apply(const PassArgs<T>& a, size_t i, const PIn<T>& x, bool upd,
                                        T tau, T beta, T* acc) {
-  if (MODE == A_PLAIN) {
+  if (MODE == A_PLAIN || MODE == A_PLAIN64) {
     return x.p;
   } else if (MODE == A_PK_P) {
     // Polonsky-Keer steps 7-8: p <- max(p - tau t, 0) on the contact set,
@@ -368,7 +370,7 @@ __global__ void BEM_ROW_BOUNDS(LOGL) k_pass_a(PassArgs<T> a) {
   __shared__ double red[3 * 32];
   Cx* sm = reinterpret_cast<Cx*>(smem_raw);
   Scalars* sc = a.sc;
-  if (MODE != A_PLAIN && MODE != A_TORUS) {
+  if (MODE != A_PLAIN && MODE != A_PLAIN64 && MODE != A_TORUS) {
     if (sc->done) return;
   }
   const int nb = a.pl.nbA, lognb = a.pl.lognbA, rs = a.pl.gA.rs;
@@ -450,32 +452,38 @@ __global__ void BEM_ROW_BOUNDS(LOGL) k_pass_a(PassArgs<T> a) {
 // shared memory as bulk copies (one per field row).  Used when rows are
 // multiples of 16 elements and the fields are 16-byte aligned.
 template <int MODE> struct ProStage {
-  static constexpr int nT = (MODE == A_PK_P || MODE == A_PK_T) ? 3 : (MODE == A_CG_T ? 4 : (MODE == A_PLAIN ? 1 : 0));
+  static constexpr int nT = (MODE == A_PK_P || MODE == A_PK_T) ? 3
+                            : MODE == A_CG_T ? 4 : (MODE == A_PLAIN || MODE == A_PLAIN64) ? 1 : 0;
   static constexpr bool S = MODE == A_CG_T;
 };
+// Type of the staged field rows: doubles for A_PLAIN64.
+template <typename T, int MODE> struct StageT { using type = T; };
+template <typename T> struct StageT<T, A_PLAIN64> { using type = double; };
+template <typename T, int MODE> using ST = typename StageT<T, MODE>::type;
 template <typename T, int MODE>
 __host__ __device__ constexpr size_t pro_stage_bytes(int nb, int nx) {
-  return ((size_t)ProStage<MODE>::nT * sizeof(T) + (ProStage<MODE>::S ? 1 : 0)) * (size_t)nb * nx;
+  return ((size_t)ProStage<MODE>::nT * sizeof(ST<T, MODE>) + (ProStage<MODE>::S ? 1 : 0)) * (size_t)nb * nx;
 }
 template <typename T, int MODE>
-__device__ __forceinline__ const T* pro_field(const PassArgs<T>& a, int f) {
-  if (MODE == A_PLAIN) return a.f.src;
-  if (MODE == A_CG_T) return f == 0 ? a.f.t : (f == 1 ? a.f.g : (f == 2 ? a.f.p : a.f.r));
-  return f == 0 ? a.f.p : (f == 1 ? a.f.t : a.f.g);
+__device__ __forceinline__ const ST<T, MODE>* pro_field(const PassArgs<T>& a, int f) {
+  if constexpr (MODE == A_PLAIN64) return a.f.src64;
+  else if constexpr (MODE == A_PLAIN) return a.f.src;
+  else if constexpr (MODE == A_CG_T) return f == 0 ? a.f.t : (f == 1 ? a.f.g : (f == 2 ? a.f.p : a.f.r));
+  else return f == 0 ? a.f.p : (f == 1 ? a.f.t : a.f.g);
 }
 // Thread 0 stages the prologue fields of rows row0 .. row0+rows-1 into shared
 // memory: one bulk copy per field row, completing on `bar` (16-byte aligned
 // rows: the persistent launch requires nx % 16 == 0 and aligned fields).
 template <typename T, int MODE>
-__device__ __forceinline__ void pro_prefetch(const PassArgs<T>& a, T* st, uint8_t* ss, int row0, int rows,
+__device__ __forceinline__ void pro_prefetch(const PassArgs<T>& a, ST<T, MODE>* st, uint8_t* ss, int row0, int rows,
                                              int nx, int nb, unsigned long long* bar) {
   if (threadIdx.x != 0) return;
-  const unsigned rb = (unsigned)(nx * (int)sizeof(T));
+  const unsigned rb = (unsigned)(nx * (int)sizeof(ST<T, MODE>));
   fence_proxy_async_smem();
   mbar_expect_tx(bar, (unsigned)rows * (ProStage<MODE>::nT * rb + (ProStage<MODE>::S ? (unsigned)nx : 0u)));
 #pragma unroll
   for (int f = 0; f < ProStage<MODE>::nT; ++f) {
-    const T* src = pro_field<T, MODE>(a, f);
+    const ST<T, MODE>* src = pro_field<T, MODE>(a, f);
     for (int bb = 0; bb < rows; ++bb)
       bulk_g2s(st + ((size_t)f * nb + bb) * nx, src + (size_t)(row0 + bb) * nx, rb, bar);
   }
@@ -486,15 +494,15 @@ __device__ __forceinline__ void pro_prefetch(const PassArgs<T>& a, T* st, uint8_
 }
 // Both elements of an even column pair (col, col+1) from the staging area.
 template <typename T, int MODE>
-__device__ __forceinline__ void pro_gather_pair_staged(const T* st, const uint8_t* ss, int b, int col, int nx,
-                                                       int nb, PIn<T>& x0, PIn<T>& x1) {
+__device__ __forceinline__ void pro_gather_pair_staged(const ST<T, MODE>* st, const uint8_t* ss, int b, int col,
+                                                       int nx, int nb, PIn<T>& x0, PIn<T>& x1) {
   const size_t j = (size_t)b * nx + col, plane = (size_t)nb * nx;
-  const V2<T>* s2 = reinterpret_cast<const V2<T>*>(st + j);
+  const V2<ST<T, MODE>>* s2 = reinterpret_cast<const V2<ST<T, MODE>>*>(st + j);
   const size_t p2 = plane / 2;
-  if (MODE == A_PLAIN) {
-    const V2<T> v = s2[0];
-    x0.p = v.x; x1.p = v.y;
-  } else if (MODE == A_CG_T) {
+  if constexpr (MODE == A_PLAIN || MODE == A_PLAIN64) {
+    const V2<ST<T, MODE>> v = s2[0];
+    x0.p = (T)v.x; x1.p = (T)v.y;
+  } else if constexpr (MODE == A_CG_T) {
     const V2<T> vt = s2[0], vg = s2[p2], vp = s2[2 * p2], vr = s2[3 * p2];
     const uchar2 vs = *reinterpret_cast<const uchar2*>(ss + j);
     x0.t = vt.x; x1.t = vt.y; x0.g = vg.x; x1.g = vg.y; x0.s = vs.x; x1.s = vs.y;
@@ -503,17 +511,6 @@ __device__ __forceinline__ void pro_gather_pair_staged(const T* st, const uint8_
     const V2<T> vp = s2[0], vt = s2[p2], vg = s2[2 * p2];
     x0.p = vp.x; x1.p = vp.y; x0.t = vt.x; x1.t = vt.y; x0.g = vg.x; x1.g = vg.y;
   }
-}
-
-template <typename T, int MODE>
-__device__ __forceinline__ void pro_gather_staged(const T* st, const uint8_t* ss, int b, int col, int nx,
-                                                  int nb, PIn<T>& x) {
-  const size_t j = (size_t)b * nx + col, plane = (size_t)nb * nx;
-  if (MODE == A_PLAIN) { x.p = st[j]; }
-  else if (MODE == A_CG_T) {
-    x.t = st[j]; x.g = st[plane + j]; x.p = st[2 * plane + j]; x.r = st[3 * plane + j]; x.s = ss[j];
-  }
-  else { x.p = st[j]; x.t = st[plane + j]; x.g = st[2 * plane + j]; }
 }
 
 #ifndef BEM_ROWP_MIN_BLOCKS
@@ -530,7 +527,7 @@ __device__ __forceinline__ void pass_ap_body(const PassArgs<T>& a) {
   __shared__ double red[3 * 32];
   Cx* sm = reinterpret_cast<Cx*>(smem_raw);
   Scalars* sc = a.sc;
-  if (MODE != A_PLAIN) {
+  if (MODE != A_PLAIN && MODE != A_PLAIN64) {
     if (sc->done) return;
   }
   const int nb = a.pl.nbA, lognb = a.pl.lognbA, rs = a.pl.gA.rs;
@@ -540,8 +537,8 @@ __device__ __forceinline__ void pass_ap_body(const PassArgs<T>& a) {
   const int half = (ncols + 1) >> 1;
   const int G = (nrows + nb - 1) / nb;
   Cx* buf = sm + b * rs;
-  T* st = reinterpret_cast<T*>(smem_raw + ((sizeof(Cx) * (size_t)nb * rs + 15) & ~(size_t)15));
-  uint8_t* ss = reinterpret_cast<uint8_t*>(st) + (size_t)ProStage<MODE>::nT * sizeof(T) * nb * ncols;
+  ST<T, MODE>* st = reinterpret_cast<ST<T, MODE>*>(smem_raw + ((sizeof(Cx) * (size_t)nb * rs + 15) & ~(size_t)15));
+  uint8_t* ss = reinterpret_cast<uint8_t*>(st) + (size_t)ProStage<MODE>::nT * sizeof(ST<T, MODE>) * nb * ncols;
   const Cx* tw = reinterpret_cast<const Cx*>(a.twA);
   const Cx* tws = reinterpret_cast<const Cx*>(a.twS);
   const int* sp = a.spA;
@@ -581,7 +578,7 @@ __device__ __forceinline__ void pass_ap_body(const PassArgs<T>& a) {
     // of the first CG-loop launch waits (bounded) on a barrier nothing
     // completes; every copy it issued has already landed, so it gives up like a
     // lost copy would.  (A_PLAIN launches carry no scalars.)
-    if (MODE != A_PLAIN && sc != nullptr && g == g0 && blockIdx.x == 0) {
+    if (MODE != A_PLAIN && MODE != A_PLAIN64 && sc != nullptr && g == g0 && blockIdx.x == 0) {
       __shared__ unsigned long long never;
       __shared__ int inj;
       if (tid == 0) {
@@ -617,7 +614,7 @@ __device__ __forceinline__ void pass_ap_body(const PassArgs<T>& a) {
       if (act && n < half) {
         const T x0 = pro_value<T, MODE>(in[e][0], upd, tau, beta, acc);
         const T x1 = pro_value<T, MODE>(in[e][1], upd, tau, beta, acc);
-        if (MODE != A_PLAIN) {
+        if (MODE != A_PLAIN && MODE != A_PLAIN64) {
           V2<T> o;
           o.x = x0; o.y = x1;
           *reinterpret_cast<V2<T>*>(out + rowoff + 2 * n) = o;
@@ -1042,7 +1039,7 @@ __device__ __forceinline__ T* epi_out(const PassArgs<T>& a) {
 }
 template <typename T, int MODE>
 __device__ __forceinline__ T epi_value(T u, const EIn<T>& x, T* acc) {
-  if (MODE == C_PLAIN) {
+  if (MODE == C_PLAIN || MODE == C_PLAIN64) {
     return u;
   } else if (MODE == C_PK_G) {
     const T gv = u + x.c;
@@ -1096,6 +1093,8 @@ template <typename T, int MODE>
 __device__ __forceinline__ void epi_apply(const PassArgs<T>& a, size_t i, T u, const EIn<T>& x, T* acc) {
   if (MODE == C_PLAIN) {
     a.f.dst[i] = u;
+  } else if (MODE == C_PLAIN64) {
+    a.f.dst64[i] = (double)u;
   } else if (MODE == C_PK_G) {
     const T gv = u + x.c;
     a.f.g[i] = gv;
@@ -1276,7 +1275,7 @@ __global__ void BEM_ROW_BOUNDS(LOGL) k_pass_c(PassArgs<T> a) {
   __shared__ int lastflag;
   Cx* sm = reinterpret_cast<Cx*>(smem_raw);
   Scalars* sc = a.sc;
-  if (MODE != C_PLAIN && MODE != C_GAP) {
+  if (MODE != C_PLAIN && MODE != C_PLAIN64 && MODE != C_GAP) {
     if (sc->done) return;
   }
   __shared__ CgPre pre;
@@ -1386,7 +1385,7 @@ __global__ void BEM_ROW_BOUNDS(LOGL) k_pass_c(PassArgs<T> a) {
         if (act && n < half && 2 * n + h < nx)
           epi_gather_staged<T, MODE>(st, ss, b, 2 * n + h, nx, nb, ein[e][h]);
     }
-  } else if (MODE != C_PLAIN) {
+  } else if (MODE != C_PLAIN && MODE != C_PLAIN64) {
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       if (!F::first_half(e)) continue;
@@ -1409,7 +1408,7 @@ __global__ void BEM_ROW_BOUNDS(LOGL) k_pass_c(PassArgs<T> a) {
       if (act && n < half && 2 * n + h < nx)
         epi_apply<T, MODE>(a, rowoff + 2 * n + h, us * (h ? v[e].y : v[e].x), ein[e][h], acc);
   }
-  if (MODE == C_PLAIN || MODE == C_GAP) return;
+  if (MODE == C_PLAIN || MODE == C_PLAIN64 || MODE == C_GAP) return;
   constexpr int NQ = MODE == C_CG_R ? 4 : 2;
   block_partials<T, NQ>(acc, a.partC + 4 * blockIdx.x, red);
   if (!last_block_arrival(MODE == C_PK_G ? &sc->cnt_c : &sc->cnt_a, &lastflag)) return;
@@ -1436,7 +1435,7 @@ __device__ __forceinline__ void pass_cp_body(const PassArgs<T>& a) {
   __shared__ int lastflag;
   Cx* sm = reinterpret_cast<Cx*>(smem_raw);
   Scalars* sc = a.sc;
-  if (MODE != C_PLAIN && MODE != C_GAP) {
+  if (MODE != C_PLAIN && MODE != C_PLAIN64 && MODE != C_GAP) {
     if (sc->done) return;
   }
   __shared__ CgPre pre;
@@ -1589,7 +1588,7 @@ __device__ __forceinline__ void pass_cp_body(const PassArgs<T>& a) {
     const size_t rowoff = (size_t)row * nx;
     // nx is a multiple of 16 here: column pairs (2n, 2n+1) are whole
     EIn<T> ein[8][2];
-    if (MODE != C_PLAIN) {
+    if (MODE != C_PLAIN && MODE != C_PLAIN64) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         if (!F::first_half(e)) continue;
@@ -1617,14 +1616,18 @@ __device__ __forceinline__ void pass_cp_body(const PassArgs<T>& a) {
         V2<T> o;
         o.x = epi_value<T, MODE>(us * v[e].x, ein[e][0], acc);
         o.y = epi_value<T, MODE>(us * v[e].y, ein[e][1], acc);
-        if (MODE != C_PK_R) *reinterpret_cast<V2<T>*>(out + rowoff + 2 * n) = o;
+        if constexpr (MODE == C_PLAIN64) {
+          *reinterpret_cast<double2*>(a.f.dst64 + rowoff + 2 * n) = make_double2((double)o.x, (double)o.y);
+        } else if (MODE != C_PK_R) {
+          *reinterpret_cast<V2<T>*>(out + rowoff + 2 * n) = o;
+        }
       }
     }
     __syncthreads();  // epilogue staging and transform rows consumed
     if (gn < gend && EpiStage<MODE>::any) prefetch_e(gn);
   }
   cp_async_wait_all();
-  if (MODE == C_PLAIN || MODE == C_GAP) return;
+  if (MODE == C_PLAIN || MODE == C_PLAIN64 || MODE == C_GAP) return;
   constexpr int NQ = MODE == C_CG_R ? 4 : 2;
   block_partials<T, NQ>(acc, a.partC + 4 * blockIdx.x, red);
   if (!last_block_arrival(MODE == C_PK_G ? &sc->cnt_c : &sc->cnt_a, &lastflag)) return;
@@ -1787,11 +1790,6 @@ __global__ void k_stats(int n, const T* p, const T* g, const uint8_t* S, int use
 }
 
 template <typename T>
-__global__ void k_convert_in(const double* src, T* dst, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    dst[i] = (T)src[i];
-}
-template <typename T>
 __global__ void k_convert_out(const T* src, double* dst, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     dst[i] = (double)src[i];
@@ -1847,13 +1845,14 @@ inline bool aligned16(const void* p) { return p == nullptr || (reinterpret_cast<
 template <typename T, int MODE>
 bool pro_fields_aligned(const PassArgs<T>& a) {
   if (MODE == A_PLAIN) return aligned16(a.f.src);
+  if (MODE == A_PLAIN64) return aligned16(a.f.src64);
   return aligned16(a.f.p) && aligned16(a.f.t) && aligned16(a.f.g) && aligned16(a.f.S) &&
          (MODE != A_CG_T || aligned16(a.f.r));
 }
 template <typename T>
 bool epi_fields_aligned(const PassArgs<T>& a) {
   return aligned16(a.f.c) && aligned16(a.f.p) && aligned16(a.f.t) && aligned16(a.f.S) && aligned16(a.W) &&
-         aligned16(a.f.dst) && aligned16(a.f.g) && aligned16(a.f.r);
+         aligned16(a.f.dst) && aligned16(a.f.dst64) && aligned16(a.f.g) && aligned16(a.f.r);
 }
 
 template <typename T, int MODE>
@@ -2020,6 +2019,7 @@ void launch_pass_a(const PassArgs<T>& a, int mode, cudaStream_t s) {
   } else {
     switch (mode) {
       case A_PLAIN: launch_a_mode<T, A_PLAIN>(a, s); break;
+      case A_PLAIN64: launch_a_mode<T, A_PLAIN64>(a, s); break;
       case A_PK_P: launch_a_mode<T, A_PK_P>(a, s); break;
       case A_PK_T: launch_a_mode<T, A_PK_T>(a, s); break;
       case A_CG_T: launch_a_mode<T, A_CG_T>(a, s); break;
@@ -2046,6 +2046,7 @@ void launch_pass_c(const PassArgs<T>& a, int mode, cudaStream_t s) {
   } else {
     switch (mode) {
       case C_PLAIN: launch_c_mode<T, C_PLAIN>(a, s); break;
+      case C_PLAIN64: launch_c_mode<T, C_PLAIN64>(a, s); break;
       case C_PK_G: launch_c_mode<T, C_PK_G>(a, s); break;
       case C_PK_R: launch_c_mode<T, C_PK_R>(a, s); break;
       case C_CG_R: launch_c_mode<T, C_CG_R>(a, s); break;
@@ -2078,10 +2079,12 @@ cudaError_t set_smem_attrs_a(int bytes) {
   } else {
 #define BEM_CASE(LG)                          \
   BEM_ATTR((k_pass_a<T, A_PLAIN, LG>))        \
+  BEM_ATTR((k_pass_a<T, A_PLAIN64, LG>))      \
   BEM_ATTR((k_pass_a<T, A_PK_P, LG>))         \
   BEM_ATTR((k_pass_a<T, A_PK_T, LG>))         \
   BEM_ATTR((k_pass_a<T, A_CG_T, LG>))         \
   BEM_ATTR((k_pass_ap<T, A_PLAIN, LG>))       \
+  BEM_ATTR((k_pass_ap<T, A_PLAIN64, LG>))     \
   BEM_ATTR((k_pass_ap<T, A_PK_P, LG>))        \
   BEM_ATTR((k_pass_ap<T, A_PK_T, LG>))        \
   BEM_ATTR((k_pass_ap<T, A_CG_T, LG>))        \
@@ -2115,12 +2118,14 @@ cudaError_t set_smem_attrs_c(int bytes) {
   cudaError_t e = cudaSuccess, r;
 #define BEM_CASE(LG)                          \
   BEM_ATTR((k_pass_c<T, C_PLAIN, LG>))        \
+  BEM_ATTR((k_pass_c<T, C_PLAIN64, LG>))      \
   BEM_ATTR((k_pass_c<T, C_PK_G, LG>))         \
   BEM_ATTR((k_pass_c<T, C_PK_R, LG>))         \
   BEM_ATTR((k_pass_c<T, C_CG_R, LG>))         \
   BEM_ATTR((k_pass_c<T, C_CG_G, LG>))         \
   BEM_ATTR((k_pass_c<T, C_GAP, LG>))          \
   BEM_ATTR((k_pass_cp<T, C_PLAIN, LG>))       \
+  BEM_ATTR((k_pass_cp<T, C_PLAIN64, LG>))     \
   BEM_ATTR((k_pass_cp<T, C_PK_G, LG>))        \
   BEM_ATTR((k_pass_cp<T, C_PK_R, LG>))        \
   BEM_ATTR((k_pass_cp<T, C_CG_R, LG>))        \
@@ -2178,10 +2183,6 @@ void launch_stats(const Plan& pl, const T* p, const T* g, const uint8_t* S, int 
   k_stats<T><<<ngrid, 256, 0, s>>>(pl.nx * pl.ny, p, g, S, use_set, part, counter, out);
 }
 template <typename T>
-void launch_convert_in(const double* src, T* dst, size_t n, cudaStream_t s) {
-  k_convert_in<T><<<ew_grid(n), 256, 0, s>>>(src, dst, n);
-}
-template <typename T>
 void launch_convert_out(const T* src, double* dst, size_t n, cudaStream_t s) {
   k_convert_out<T><<<ew_grid(n), 256, 0, s>>>(src, dst, n);
 }
@@ -2220,7 +2221,6 @@ void launch_mask_field(T* x, const uint8_t* S, size_t n, cudaStream_t s) {
   template void launch_cg_finish<T>(const Plan&, Fields<T>, const Scalars*, int, cudaStream_t); \
   template void launch_stats<T>(const Plan&, const T*, const T*, const uint8_t*, int, double*, \
                                 double*, int, cudaStream_t);                                   \
-  template void launch_convert_in<T>(const double*, T*, size_t, cudaStream_t);                \
   template void launch_convert_out<T>(const T*, double*, size_t, cudaStream_t);               \
   template void launch_offset<T>(const double*, double, T*, size_t, cudaStream_t);            \
   template void launch_set_from_p<T>(const T*, uint8_t*, size_t, cudaStream_t);               \
