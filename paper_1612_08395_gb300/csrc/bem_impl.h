@@ -21,7 +21,21 @@ struct Geo {
 //   so[ls * 8 + r] = swz(r << ls), ls = 0..13     (112 entries)
 //   sp[k]          = swz(dig_pos(k)), k < 2^logL  (digit-reversed, swizzled)
 constexpr int kSoEntries = 112;
-void launch_geo_tables(int* so, int* sp, Geo g, int esize, cudaStream_t s);
+
+// Every table of a context, made by one launch: twiddles as [length-M stages |
+// length-Py stages | real-FFT split | radix-16 length-Py stages (FP32 only)] in
+// FP64, FP32 and as fixed-point limbs, and up to four index tables, so then sp
+// (null pointers: not made).
+struct TableArgs {
+  int logM, logP;
+  double2* t64;
+  float2* t32;
+  int4* fx;
+  int* geo[4];
+  Geo g[4];
+  int esize[4];
+};
+void launch_tables(const TableArgs& a, cudaStream_t s);
 
 // Launch geometry of the three convolution passes for one handle.
 //   ny, nx: field rows and columns;  Px, Py: torus sides (powers of two
@@ -116,8 +130,8 @@ struct PassArgs {
   Plan pl;
   Fields<T> f;
   void* W;              // C<T>[(M+1) * rows_w]
-  int rows_w;           // row length of W (= ny, or Py for the spectrum)
-  int nrows_in;         // rows fed to pass A (= ny, or Py for the torus)
+  int rows_w;           // row length of W (= ny, or Py/2 + 1 for the spectrum)
+  int nrows_in;         // rows fed to pass A (= ny, or Py/2 + 1 for the torus)
   int ncols_in;         // columns fed to pass A (= nx, or Px for the torus)
   const double* kq64;   // A_TORUS: influence quarter, (Py/2+1) x (M+1)
   const T* khat;        // B_CONV: spectrum quarter, transposed: [kx][ky], ky <= Py/2
@@ -176,7 +190,6 @@ void launch_fx_c(const PassArgs<double>& a, int mode, const PassArgs<double>* ar
 cudaError_t set_smem_attrs_fx_a(int bytes);
 cudaError_t set_smem_attrs_fx_b(int bytes);
 cudaError_t set_smem_attrs_fx_c(int bytes);
-void launch_fx_tables(const double2* w, int4* out, int n, cudaStream_t s);
 
 // CG loops of small grids in one thread-block cluster (resident.cuh): lm = log2 M
 // in 4..8, lp = log2 Py in 5..9, n instances.
@@ -284,11 +297,6 @@ void batcher_stats(LoopBatcher* b, long long* launches, long long* instances);
 // Record `msg` as the thread's last error and return `code`.
 int set_error(int code, const char* msg);
 
-// Twiddle tables of one FFT length (stage tables, 2^logL entries reserved) and
-// of the real-FFT split (M+1 entries), FP64 and FP32 copies.
-void launch_twiddles(double2* t64, float2* t32, int logL, cudaStream_t s);
-void launch_split_twiddles(double2* t64, float2* t32, int M, cudaStream_t s);
-void launch_twiddles16(double2* t64, float2* t32, int logL, cudaStream_t s);
 // Geometry (swizzle, first-stage radix, row stride) of a length-2^logL
 // transform with `rows` transforms per CTA, for elements of esize bytes.
 Geo make_geo(int logL, int rows, int esize);

@@ -394,8 +394,8 @@ __global__ void BEM_ROW_BOUNDS(LOGL) k_pass_a(PassArgs<T> a) {
   Cx v[8];
   if (MODE == A_TORUS) {
     // K on the even Px x Py torus (spectrum set-up, FP64, all columns)
-    const int py = a.pl.py, px = a.pl.px;
-    const int ry = row < py - row ? row : py - row;
+    // (rows 0..Py/2: the others repeat them)
+    const int px = a.pl.px, ry = row;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const int n = F::n0(t, e);
@@ -695,7 +695,8 @@ __device__ __forceinline__ void pass_b_body(const PassArgs<T>& a) {
     v[e] = mk<T>(0, 0);
     if (HALF && !F::first_half(e)) continue;
     const int y = F::n0(t, e);
-    if (act && y >= ylo && y <= yhi && bem_check(coff + y < (size_t)(M + 1) * rin, a.kerr)) v[e] = W[coff + y];
+    const int yw = MODE == B_SPECTRUM ? min(y, L - y) : y;  // the torus is even: rows 0..L/2 stand for all
+    if (act && yw >= ylo && yw <= yhi && bem_check(coff + yw < (size_t)(M + 1) * rin, a.kerr)) v[e] = W[coff + yw];
   }
   F::stage0_fwd(v, t, tw);
 #pragma unroll

@@ -13,7 +13,16 @@
 // analytic on the element and tensor Gauss-Legendre rules are used directly,
 // with fewer points the farther the element; the distance is counted in units
 // of the element's longer side, so elongated elements near the singularity
-// take the corner formula.
+// take the corner formula.  From SERIES sides on the element's mean is its
+// Taylor series to sixth order in the sides (the eighth-order term is below
+// 0.01 SERIES^-8 = 6e-17 of it), one power instead of sixteen: all but a corner
+// of a large table.  Bound by FP64 instructions throughout.
+//
+// The corner formula takes a CTA per element and a thread per quadrature node,
+// the tensor rules a warp per element: one thread evaluating an element's eight
+// rays took 1.8 ms and its 256 nodes 0.6 ms, which every table, however small,
+// had to wait for.  Square elements need half the table: K(di, dj) = K(dj, di).
+// Together (GB300): 65^2 table 1.84 -> 0.04 ms, 1025^2 3.5 -> 0.1 ms.
 #include <math.h>
 #include <cuda_runtime.h>
 
@@ -24,10 +33,10 @@ namespace bem {
 namespace {
 constexpr int NG16 = 16;
 constexpr int NEAR = 4;
+constexpr int SERIES = 60;
 __constant__ double c_x16[16], c_w16[16];
 __constant__ double c_x10[10], c_w10[10];
 __constant__ double c_x6[6], c_w6[6];
-__constant__ double c_x4[4], c_w4[4];
 
 // Gauss-Legendre rule on [-1, 1]: roots of P_n by Newton's method, starting
 // from the Tricomi approximation; P_n and P_n' from the Bonnet recurrence.
@@ -66,88 +75,139 @@ int influence_init_nodes() {
   legendre_rule(6, x, w);
   if (cudaMemcpyToSymbol(c_x6, x, sizeof(double) * 6) != cudaSuccess) return -1;
   if (cudaMemcpyToSymbol(c_w6, w, sizeof(double) * 6) != cudaSuccess) return -1;
-  legendre_rule(4, x, w);
-  if (cudaMemcpyToSymbol(c_x4, x, sizeof(double) * 4) != cudaSuccess) return -1;
-  if (cudaMemcpyToSymbol(c_w4, w, sizeof(double) * 4) != cudaSuccess) return -1;
   return 0;
 }
 
-// G(U) = int_0^{asinh U} cosh(s)^-k ds, composite 16-point Gauss-Legendre
-// with panels no longer than 0.5.
-__device__ double g_ray(double U, double k) {
-  const double S = asinh(U);
-  int np = (int)ceil(S / 0.5);
-  if (np < 1) np = 1;
-  const double hp = S / np;
-  double sum = 0.0;
-  for (int q = 0; q < np; ++q) {
-    const double mid = (q + 0.5) * hp;
-    double s = 0.0;
-#pragma unroll 4
-    for (int i = 0; i < NG16; ++i) {
-      const double x = mid + 0.5 * hp * c_x16[i];
-      s += c_w16[i] * exp(-k * log(cosh(x)));
+// distance class of the element: its index distance, but for elongated
+// elements never more than its physical distance from the singularity in
+// units of its longer side (a long element can reach close to the origin)
+__device__ __forceinline__ double distance_class(int di, int dj, double dx, double dy) {
+  const double ea = fmax(0.0, (di - 0.5) * dx), eb = fmax(0.0, (dj - 0.5) * dy);
+  const double phys = sqrt(ea * ea + eb * eb) / fmax(dx, dy) + 0.5;
+  return fmin((double)(di > dj ? di : dj), phys);
+}
+
+// The corner formula: K = F(a1, b1) - F(a0, b1) - F(a1, b0) + F(a0, b0), with
+// F(x, y) = [ |x|^(1-k) G(|y/x|) + |y|^(1-k) G(|x/y|) ] / (1-k), odd in x and y,
+// and G(U) = int_0^{asinh U} cosh(s)^-k ds by composite 16-point Gauss-Legendre
+// with panels no longer than 0.5.  Thread t: corner t / 32, ray (t / 16) % 2,
+// node t % 16 of every panel.
+__global__ void __launch_bounds__(128) k_influence_near(double* Kq, int hx, int hy, double dx, double dy, double k) {
+  const int di = blockIdx.x, dj = blockIdx.y;
+  if (di >= hx || dj >= hy || distance_class(di, dj, dx, dy) > NEAR) return;
+  __shared__ double part[8];
+  const int c = threadIdx.x >> 5, ray = (threadIdx.x >> 4) & 1, i = threadIdx.x & 15;
+  const double x = (di + (c & 1 ? 0.5 : -0.5)) * dx, y = (dj + (c & 2 ? 0.5 : -0.5)) * dy;
+  const double p = fabs(ray ? y : x), q = fabs(ray ? x : y);
+  double g = 0.0, hp = 0.0;
+  if (p > 0.0 && q > 0.0) {
+    const double S = asinh(q / p);
+    const int np = max(1, (int)ceil(S / 0.5));
+    hp = S / np;
+    for (int m = 0; m < np; ++m) {
+      const double s = (m + 0.5) * hp + 0.5 * hp * c_x16[i];
+      g += exp(-k * log(cosh(s)));
     }
-    sum += s;
+    g *= c_w16[i];
   }
-  return sum * 0.5 * hp;
-}
-
-// F(x, y): integral over [0, x] x [0, y], odd in x and in y.
-__device__ double f_corner(double x, double y, double k) {
-  if (x == 0.0 || y == 0.0) return 0.0;
-  const double ax = fabs(x), ay = fabs(y);
-  const double v = (pow(ax, 1.0 - k) * g_ray(ay / ax, k) + pow(ay, 1.0 - k) * g_ray(ax / ay, k)) / (1.0 - k);
-  return ((x < 0.0) != (y < 0.0)) ? -v : v;
-}
-
-template <int NP>
-__device__ double tensor_gl(const double* xs, const double* ws, double a0, double a1, double b0,
-                            double b1, double expo) {
-  const double ca = 0.5 * (a0 + a1), ha = 0.5 * (a1 - a0);
-  const double cb = 0.5 * (b0 + b1), hb = 0.5 * (b1 - b0);
-  double s = 0.0;
-#pragma unroll 1
-  for (int i = 0; i < NP; ++i) {
-    const double a = ca + ha * xs[i];
-    const double a2 = a * a;
-    double si = 0.0;
 #pragma unroll
-    for (int j = 0; j < NP; ++j) {
-      const double b = cb + hb * xs[j];
-      si += ws[j] * exp(expo * log(a2 + b * b));
-    }
-    s += ws[i] * si;
+  for (int o = 8; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+  if (i == 0) {
+    double v = p > 0.0 && q > 0.0 ? pow(p, 1.0 - k) * (g * 0.5 * hp) / (1.0 - k) : 0.0;
+    if ((x < 0.0) != (y < 0.0)) v = -v;
+    part[threadIdx.x >> 4] = v;
   }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double F00 = part[0] + part[1], F10 = part[2] + part[3], F01 = part[4] + part[5], F11 = part[6] + part[7];
+    Kq[(size_t)dj * hx + di] = F11 - F01 - F10 + F00;
+  }
+}
+
+// Mean over the element of (x^2+y^2)^-a, a = (1+k)/2, times its area, by the
+// Taylor series at its centre: with q = x^2+y^2, X = x^2/q, Y = y^2/q and
+// c_n = a (a+1) ... (a+n-1), the derivative of order (2m, 2n) is q^-(a+m+n) times
+// sum over j, i of (-1)^(m-j+n-i) A(m,j) A(n,i) c_(m+n+j+i) X^j Y^i,
+// A(m,j) = 4^j (2m)! / ((m-j)! (2j)!); the mean takes it with
+// (hx/2)^(2m) (hy/2)^(2n) / ((2m+1)! (2n+1)!).  Beyond 400 sides the sixth-order
+// terms are below 3e-17 and left out.
+__device__ __forceinline__ double series_mean(double x, double y, double hx, double hy, double k, bool sixth) {
+  const double a = 0.5 * (1.0 + k);
+  const double c1 = a, c2 = c1 * (a + 1.0), c3 = c2 * (a + 2.0), c4 = c3 * (a + 3.0), c5 = c4 * (a + 4.0),
+               c6 = c5 * (a + 5.0);
+  const double q = x * x + y * y, rq = 1.0 / q, X = x * x * rq, Y = y * y * rq;
+  const double u = 0.25 * hx * hx * rq, v = 0.25 * hy * hy * rq;  // squared half sides over q
+  const double xx = -2.0 * c1 + 4.0 * c2 * X, yy = -2.0 * c1 + 4.0 * c2 * Y;
+  const double x4 = 12.0 * c2 + X * (-48.0 * c3 + 16.0 * c4 * X), y4 = 12.0 * c2 + Y * (-48.0 * c3 + 16.0 * c4 * Y);
+  const double x2y2 = 4.0 * c2 - 8.0 * c3 + 16.0 * c4 * X * Y;
+  const double s2 = (u * xx + v * yy) * (1.0 / 6.0);
+  const double s4 = (u * u * x4 + v * v * y4) * (1.0 / 120.0) + u * v * x2y2 * (1.0 / 36.0);
+  double s6 = 0.0;
+  if (sixth) {
+    const double x6 = -120.0 * c3 + X * (720.0 * c4 + X * (-480.0 * c5 + 64.0 * c6 * X));
+    const double y6 = -120.0 * c3 + Y * (720.0 * c4 + Y * (-480.0 * c5 + 64.0 * c6 * Y));
+    const double x4y2 = -24.0 * c3 + 48.0 * c4 * Y + X * (96.0 * c4 - 192.0 * c5 * Y + X * (-32.0 * c5 + 64.0 * c6 * Y));
+    const double y4x2 = -24.0 * c3 + 48.0 * c4 * X + Y * (96.0 * c4 - 192.0 * c5 * X + Y * (-32.0 * c5 + 64.0 * c6 * X));
+    s6 = (u * u * u * x6 + v * v * v * y6) * (1.0 / 5040.0) + u * v * (u * x4y2 + v * y4x2) * (1.0 / 720.0);
+  }
+  return hx * hy * exp(-a * log(q)) * (1.0 + (s2 + (s4 + s6)));
+}
+
+// One warp's sum of an element's NP x NP Gauss-Legendre nodes, in every lane.
+template <int NP>
+__device__ __forceinline__ double tensor_gl(const double* xs, const double* ws, double ca, double ha, double cb,
+                                            double hb, double expo) {
+  double s = 0.0;
+  for (int q = threadIdx.x & 31; q < NP * NP; q += 32) {
+    const int i = q / NP, j = q - i * NP;
+    const double a = ca + ha * xs[i], b = cb + hb * xs[j];
+    s += ws[i] * ws[j] * exp(expo * log(a * a + b * b));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s * ha * hb;
+}
+// Elements between the corner formula's and the series': a warp each, eight
+// elements of one row per CTA.
+__global__ void __launch_bounds__(256) k_influence_mid(double* Kq, int hx, int hy, double dx, double dy, double k) {
+  const int di = blockIdx.x * 8 + (threadIdx.x >> 5), dj = blockIdx.y;
+  if (di >= hx || dj >= hy) return;
+  const double far = distance_class(di, dj, dx, dy);
+  if (far <= NEAR || far > SERIES) return;
+  const double expo = -0.5 * (1.0 + k);
+  double v;
+  if (far <= 12) v = tensor_gl<16>(c_x16, c_w16, di * dx, 0.5 * dx, dj * dy, 0.5 * dy, expo);
+  else if (far <= 40) v = tensor_gl<10>(c_x10, c_w10, di * dx, 0.5 * dx, dj * dy, 0.5 * dy, expo);
+  else v = tensor_gl<6>(c_x6, c_w6, di * dx, 0.5 * dx, dj * dy, 0.5 * dy, expo);
+  if ((threadIdx.x & 31) == 0) Kq[(size_t)dj * hx + di] = v;
 }
 
 __global__ void k_influence(double* Kq, int hx, int hy, double dx, double dy, double k) {
   const int di = blockIdx.x * blockDim.x + threadIdx.x;
   const int dj = blockIdx.y;
   if (di >= hx || dj >= hy) return;
-  const double a0 = (di - 0.5) * dx, a1 = (di + 0.5) * dx;
-  const double b0 = (dj - 0.5) * dy, b1 = (dj + 0.5) * dy;
-  // distance class of the element: its index distance, but for elongated
-  // elements never more than its physical distance from the singularity in
-  // units of its longer side (a long element can reach close to the origin)
-  const double ea = fmax(0.0, a0), eb = fmax(0.0, b0), side = fmax(dx, dy);
-  const double phys = sqrt(ea * ea + eb * eb) / side + 0.5;
-  const double far = fmin((double)(di > dj ? di : dj), phys);
-  double v;
-  if (far <= NEAR) {
-    v = f_corner(a1, b1, k) - f_corner(a0, b1, k) - f_corner(a1, b0, k) + f_corner(a0, b0, k);
-  } else {
-    const double expo = -0.5 * (1.0 + k);
-    if (far <= 12) v = tensor_gl<16>(c_x16, c_w16, a0, a1, b0, b1, expo);
-    else if (far <= 40) v = tensor_gl<10>(c_x10, c_w10, a0, a1, b0, b1, expo);
-    else if (far <= 200) v = tensor_gl<6>(c_x6, c_w6, a0, a1, b0, b1, expo);
-    else v = tensor_gl<4>(c_x4, c_w4, a0, a1, b0, b1, expo);
-  }
+  const bool square = dx == dy;
+  if (square && di < dj && dj < hx) return;  // written by the mirror element (its column dj is in the table)
+  const double far = distance_class(di, dj, dx, dy);
+  if (far <= SERIES) return;  // k_influence_near, k_influence_mid
+  const double v = series_mean(di * dx, dj * dy, dx, dy, k, far <= 400.0);
   Kq[(size_t)dj * hx + di] = v;
+  if (square && di > dj && di < hy) Kq[(size_t)di * hx + dj] = v;
+}
+
+// Elements whose distance class can be at most `far` along an axis of step d.
+static int reach(double far, double side, double d, int n) {
+  const double e = (far - 0.5) * side / d + 1.5;  // (i - 1/2) d <= (far - 1/2) side
+  return e < n ? (int)e + 1 : n;
 }
 
 void launch_influence(double* Kq, int hx, int hy, double dx, double dy, double k, cudaStream_t s) {
+  const double side = dx > dy ? dx : dy;
+  const int nx = reach(NEAR, side, dx, hx), ny = reach(NEAR, side, dy, hy);
+  k_influence_near<<<dim3(nx, ny), 128, 0, s>>>(Kq, hx, hy, dx, dy, k);
+  const int mx = reach(SERIES, side, dx, hx), my = reach(SERIES, side, dy, hy);
+  k_influence_mid<<<dim3((mx + 7) / 8, my), 256, 0, s>>>(Kq, hx, hy, dx, dy, k);
+  if (mx == hx && my == hy && hx <= SERIES && hy <= SERIES) return;  // nothing farther
   const dim3 block(128), grid((hx + 127) / 128, hy);
   k_influence<<<grid, block, 0, s>>>(Kq, hx, hy, dx, dy, k);
 }

@@ -37,99 +37,112 @@ void launch_to_f32(const double* src, float* dst, size_t n, cudaStream_t s) {
   k_to_f32<<<ew_grid(n), 256, 0, s>>>(src, dst, n);
 }
 
-// Stage twiddle tables of a length 2^logL transform, stages in DIF order,
-// tables concatenated.  FP32: the table of stage (R, s) holds
-// exp(-2 pi i o/(R s)) for o < s (the radix-8 offsets are tw_off8); the
-// butterflies form the powers they need.  FP64: the table of stage (R, s)
-// holds every power, exp(-2 pi i o q/(R s)) at (q-1) s + o for q = 1..R-1
-// (offsets FftC::pow_off; fewer than 2^logL entries in all).  Computed in FP64.
-__global__ void k_twiddles(double2* t64, float2* t32, int logL) {
+// ---------------------------------------------------------------------------
+// All tables of a context in one launch, one entry per thread.  An entry costs
+// one FP64 sincospi, a few hundred issue slots of the FP64 pipe for a warp:
+// spread over the chip the tables of a 4096-point torus take a few microseconds
+// (as a few CTAs looping over them, 62 us per length).
+//
+// Stage twiddles of a length 2^logL transform, stages in DIF order, tables
+// concatenated.  FP64 and fixed point: the table of stage (R, s) holds every
+// power, exp(-2 pi i o q/(R s)) at (q-1) s + o for q = 1..R-1 (offsets
+// FftC::pow_off; fewer than 2^logL entries in all).  FP32: exp(-2 pi i o/(R s))
+// for o < s (radix-8 offsets tw_off8); the butterflies form the powers.
+__device__ __forceinline__ int4 fx_limbs(double2 v) {  // w 2^60 = h 2^30 + l (fx_kernels.cuh)
+  const long long x = __double2ll_rn(v.x * 1152921504606846976.0), y = __double2ll_rn(v.y * 1152921504606846976.0);
+  int4 q;
+  q.y = ((int)x << 2) >> 2;
+  q.x = (int)((x - q.y) >> 30);
+  q.w = ((int)y << 2) >> 2;
+  q.z = (int)((y - q.w) >> 30);
+  return q;
+}
+__device__ __forceinline__ double2 unit(double turns) {  // exp(2 pi i turns)
+  double sn, cs;
+  sincospi(2.0 * turns, &sn, &cs);
+  return make_double2(cs, sn);
+}
+__device__ void stage_entry(int i, int logL, double2* t64, float2* t32, int4* fx) {
   const int r0 = logL % 3;
-  const int L = 1 << logL;
-  int off = 0, off64 = 0;
-  int R = r0 ? (1 << r0) : 8;
-  int s = L / R;
-  for (;;) {
-    for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < s; o += gridDim.x * blockDim.x) {
-      double sn, cs;
-      sincospi(-2.0 * (double)o / ((double)R * (double)s), &sn, &cs);
-      t32[off + o] = make_float2((float)cs, (float)sn);
-      for (int q = 1; q < R; ++q) {  // o q < R s: the argument stays in (-2, 0]
-        sincospi(-2.0 * (double)(o * q) / ((double)R * (double)s), &sn, &cs);
-        t64[off64 + (q - 1) * s + o] = make_double2(cs, sn);
-      }
-    }
-    if (s == 1) break;
+  int R = r0 ? (1 << r0) : 8, s = (1 << logL) / R, off = 0, off64 = 0;
+  while (i - off64 >= (R - 1) * s) {  // the stage of entry i
+    if (s == 1) return;
     off += s;
     off64 += (R - 1) * s;
     R = 8;
     s /= 8;
   }
+  const int q = (i - off64) / s + 1, o = (i - off64) - (q - 1) * s;  // o q < R s
+  const double2 w = unit(-(double)(o * q) / ((double)R * (double)s));
+  if (t64) t64[i] = w;
+  if (fx) fx[i] = fx_limbs(w);
+  if (t32 && q == 1) t32[off + o] = make_float2((float)w.x, (float)w.y);
 }
-void launch_twiddles(double2* t64, float2* t32, int logL, cudaStream_t s) {
-  k_twiddles<<<64, 256, 0, s>>>(t64, t32, logL);
-}
-
-// Stage twiddle tables of the radix-16 column pass of length 2^logL (9 <= logL
-// <= 13; other lengths have no such pass and get no table): a leading stage
-// of radix R0 = 2^(logL mod 4) (16 if that is 1) and stride s = 2^logL/R0,
-// then radix-16 stages; the table of stage (R, s) holds exp(-2 pi i o/(R s))
-// for o < s, tables concatenated in DIF order.  Computed in FP64.
-__global__ void k_twiddles16(double2* t64, float2* t32, int logL) {
+// FP32 stage tables of the radix-16 column pass of length 2^logL (9 <= logL <=
+// 13; other lengths have none): a leading stage of radix 2^(logL mod 4) (16 if
+// that is 1), then radix-16 stages; stage (R, s) holds exp(-2 pi i o/(R s)), o < s.
+__device__ void stage16_entry(int i, int logL, float2* t32) {
   if (logL < 9 || logL > 13) return;
   const int rb = logL & 3;
-  int R = rb ? 1 << rb : 16;
-  int s = (1 << logL) / R;
-  int off = 0;
+  int R = rb ? 1 << rb : 16, s = (1 << logL) / R, off = 0;
   while (s > 1) {
-    for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < s; o += gridDim.x * blockDim.x) {
-      double sn, cs;
-      sincospi(-2.0 * (double)o / ((double)R * (double)s), &sn, &cs);
-      t64[off + o] = make_double2(cs, sn);
-      t32[off + o] = make_float2((float)cs, (float)sn);
+    if (i < off + s) {
+      const double2 w = unit(-(double)(i - off) / ((double)R * (double)s));
+      t32[i] = make_float2((float)w.x, (float)w.y);
+      return;
     }
     off += s;
     R = 16;
     s /= 16;
   }
 }
-void launch_twiddles16(double2* t64, float2* t32, int logL, cudaStream_t s) {
-  k_twiddles16<<<64, 256, 0, s>>>(t64, t32, logL);
-}
-
-// exp(-i pi k / M), k = 0..M: the real-FFT split of a length-2M real transform.
-__global__ void k_split_twiddles(double2* t64, float2* t32, int M) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k <= M; k += gridDim.x * blockDim.x) {
-    double sn, cs;
-    sincospi(-(double)k / (double)M, &sn, &cs);
-    t64[k] = make_double2(cs, sn);
-    t32[k] = make_float2((float)cs, (float)sn);
-  }
-}
-void launch_split_twiddles(double2* t64, float2* t32, int M, cudaStream_t s) {
-  k_split_twiddles<<<64, 256, 0, s>>>(t64, t32, M);
-}
-
 // Index tables of one transform length: so[ls*8 + r] = swz(r << ls) and
 // sp[k] = swz(dig_pos(k)) (see Geo).
-__global__ void k_geo_tables(int* so, int* sp, Geo g, int esize) {
+__device__ void geo_entry(int i, int* so, const Geo& g, int esize) {
   const Swz z{g.sa, g.sb, g.sc, g.sd};
-  const int L = 1 << g.logL;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kSoEntries + L; i += gridDim.x * blockDim.x) {
-    int x;
-    if (i < kSoEntries) {
-      const int ls = i >> 3, r = i & 7;
-      x = (r << ls) < L ? (r << ls) : 0;
-    } else {
-      x = dig_pos(i - kSoEntries, g.logL, g.r0);
-    }
-    const int v = esize == 4 ? swz<float>(x, z) : swz<double>(x, z);
-    if (i < kSoEntries) so[i] = v;
-    else sp[i - kSoEntries] = v;
+  int x;
+  if (i < kSoEntries) {
+    const int ls = i >> 3, r = i & 7;
+    x = (r << ls) < (1 << g.logL) ? (r << ls) : 0;
+  } else {
+    x = dig_pos(i - kSoEntries, g.logL, g.r0);
+  }
+  so[i] = esize == 4 ? swz<float>(x, z) : swz<double>(x, z);
+}
+__global__ void k_tables(TableArgs a) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int M = 1 << a.logM, P = 1 << a.logP;
+  if (i < M) return stage_entry(i, a.logM, a.t64, a.t32, a.fx);
+  i -= M;
+  if (i < P)
+    return stage_entry(i, a.logP, a.t64 ? a.t64 + M : nullptr, a.t32 ? a.t32 + M : nullptr, a.fx ? a.fx + M : nullptr);
+  i -= P;
+  if (i <= M) {  // exp(-i pi k / M): the real-FFT split
+    const double2 w = unit(-0.5 * (double)i / (double)M);
+    if (a.t64) a.t64[M + P + i] = w;
+    if (a.t32) a.t32[M + P + i] = make_float2((float)w.x, (float)w.y);
+    if (a.fx) a.fx[M + P + i] = fx_limbs(w);
+    return;
+  }
+  i -= M + 1;
+  if (a.t32) {
+    if (i < P) return stage16_entry(i, a.logP, a.t32 + M + P + M + 1);
+    i -= P;
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    if (!a.geo[t]) continue;
+    const int n = kSoEntries + (1 << a.g[t].logL);
+    if (i < n) return geo_entry(i, a.geo[t], a.g[t], a.esize[t]);
+    i -= n;
   }
 }
-void launch_geo_tables(int* so, int* sp, Geo g, int esize, cudaStream_t s) {
-  k_geo_tables<<<32, 256, 0, s>>>(so, sp, g, esize);
+void launch_tables(const TableArgs& a, cudaStream_t s) {
+  const int M = 1 << a.logM, P = 1 << a.logP;
+  int n = M + P + M + 1 + (a.t32 ? P : 0);
+  for (int t = 0; t < 4; ++t)
+    if (a.geo[t]) n += kSoEntries + (1 << a.g[t].logL);
+  k_tables<<<(n + 63) / 64, 64, 0, s>>>(a);
 }
 
 // Bounding box of the contact set: first/last row and column holding an

@@ -1,4 +1,4 @@
-// Pass B of the FP64 path (64-bit block fixed point), and its tables.
+// Pass B of the FP64 path (64-bit block fixed point).
 #include "fx_kernels.cuh"
 
 namespace bem {
@@ -25,22 +25,6 @@ cudaError_t set_smem_attrs_fx_b(int bytes) {
 #undef BEM_CASE
 #undef BEM_ATTR
   return e;
-}
-
-// Twiddles as two 30-bit limbs per component (fx_kernels.cuh) from their FP64
-// values: w 2^60 = h 2^30 + l, l in [-2^29, 2^29).
-__global__ void k_fx_tables(const double2* __restrict__ w, int4* __restrict__ out, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double2 v = w[i];
-    int4 q;
-    const ll x = __double2ll_rn(v.x * 1152921504606846976.0), y = __double2ll_rn(v.y * 1152921504606846976.0);
-    fsplit(x, q.x, q.y);
-    fsplit(y, q.z, q.w);
-    out[i] = q;
-  }
-}
-void launch_fx_tables(const double2* w, int4* out, int n, cudaStream_t s) {
-  k_fx_tables<<<std::min((n + 255) / 256, 128), 256, 0, s>>>(w, out, n);
 }
 
 }  // namespace bem

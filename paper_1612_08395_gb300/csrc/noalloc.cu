@@ -42,10 +42,15 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 std::mutex g_setup_mu;
 void* g_scratch_dev[kMaxDevices] = {};
 
-__global__ void k_transpose_spectrum(const double* src, double* dst, int hx, int hyq) {
-  // src[ky * hx + kx] (as bem_spectrum writes it) -> dst[kx * hyq + ky]
-  const int kx = blockIdx.x * blockDim.x + threadIdx.x, ky = blockIdx.y;
-  if (kx < hx && ky < hyq) dst[(size_t)kx * hyq + ky] = src[(size_t)ky * hx + kx];
+// src[ky * hx + kx] (as bem_spectrum writes it) -> dst[kx * hyq + ky], by 32 x 32 tiles.
+__global__ void k_transpose_spectrum(const double* __restrict__ src, double* __restrict__ dst, int hx, int hyq) {
+  __shared__ double tile[32][33];
+  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
+  for (int j = threadIdx.y; j < 32; j += 8)
+    if (x0 + (int)threadIdx.x < hx && y0 + j < hyq) tile[j][threadIdx.x] = src[(size_t)(y0 + j) * hx + x0 + threadIdx.x];
+  __syncthreads();
+  for (int j = threadIdx.y; j < 32; j += 8)
+    if (y0 + (int)threadIdx.x < hyq && x0 + j < hx) dst[(size_t)(x0 + j) * hyq + y0 + threadIdx.x] = tile[threadIdx.x][j];
 }
 
 int pow2_at_least(int v) {
@@ -101,15 +106,12 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   const int px = pow2_at_least(2 * Nx < 32 ? 32 : 2 * Nx);
   const int py = pow2_at_least(2 * Ny < 32 ? 32 : 2 * Ny);
   const int M = px / 2, hx = M + 1, hyq = py / 2 + 1;
-  // scratch layout: W | transposed spectrum | twiddles (FP64, FP32, fixed point) |
-  // exponents | index tables
+  // scratch layout: W | transposed spectrum | twiddles | exponents | index tables
   const size_t ntw = (size_t)M + py + M + 1;
   const size_t w_bytes = sizeof(double) * 2 * (size_t)hx * Ny;
   const size_t k_off = (w_bytes + 255) & ~(size_t)255;
   const size_t t_off = (k_off + sizeof(double) * (size_t)hx * hyq + 255) & ~(size_t)255;
-  const size_t t32_off = (t_off + sizeof(double2) * ntw + 255) & ~(size_t)255;
-  const size_t tfx_off = (t32_off + sizeof(float2) * ntw + 255) & ~(size_t)255;
-  const size_t e_off = (tfx_off + sizeof(int4) * ntw + 255) & ~(size_t)255;
+  const size_t e_off = (t_off + sizeof(int4) * ntw + 255) & ~(size_t)255;
   const size_t g_off = (e_off + sizeof(int) * ((size_t)Ny + hx) + 255) & ~(size_t)255;
   const size_t g_ints = 2 * bem::kSoEntries + (size_t)M + py;
   if (g_off + sizeof(int) * g_ints > kScratchBytes)
@@ -127,18 +129,16 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   cudaStream_t s = (cudaStream_t)stream;
   unsigned char* scratch = static_cast<unsigned char*>(base);
   double* khat_t = reinterpret_cast<double*>(scratch + k_off);
-  double2* tw64 = reinterpret_cast<double2*>(scratch + t_off);
-  float2* tw32 = reinterpret_cast<float2*>(scratch + t32_off);
-  int4* twfx = reinterpret_cast<int4*>(scratch + tfx_off);
+  int4* twfx = reinterpret_cast<int4*>(scratch + t_off);
   int* geo = reinterpret_cast<int*>(scratch + g_off);
-  bem::launch_geo_tables(geo, geo + bem::kSoEntries, pl.gA, 8, s);
-  bem::launch_geo_tables(geo + bem::kSoEntries + M, geo + 2 * bem::kSoEntries + M, pl.gB, 8, s);
-  k_transpose_spectrum<<<dim3((hx + 127) / 128, hyq), 128, 0, s>>>(khat, khat_t, hx, hyq);
-  bem::launch_twiddles(tw64, tw32, ilog2i(M), s);
-  bem::launch_twiddles(tw64 + M, tw32 + M, ilog2i(py), s);
-  bem::launch_split_twiddles(tw64 + M + py, tw32 + M + py, M, s);
-
-  bem::launch_fx_tables(tw64, twfx, (int)ntw, s);
+  bem::TableArgs t{};
+  t.logM = ilog2i(M);
+  t.logP = ilog2i(py);
+  t.fx = twfx;
+  t.geo[0] = geo; t.g[0] = pl.gA; t.esize[0] = 8;
+  t.geo[1] = geo + bem::kSoEntries + M; t.g[1] = pl.gB; t.esize[1] = 8;
+  bem::launch_tables(t, s);
+  k_transpose_spectrum<<<dim3((hx + 31) / 32, (hyq + 31) / 32), dim3(32, 8), 0, s>>>(khat, khat_t, hx, hyq);
 
   bem::PassArgs<double> a{};
   a.pl = pl;
@@ -149,9 +149,6 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   a.nrows_in = Ny;
   a.ncols_in = Nx;
   a.khat = khat_t;
-  a.twA = tw64;
-  a.twB = tw64 + M;
-  a.twS = tw64 + M + py;
   a.fxA = twfx;
   a.fxB = twfx + M;
   a.fxS = twfx + M + py;

@@ -54,7 +54,7 @@ size_t footprint(int nx, int ny) {
   b += 16 * (M + 1) * ny;               // W (FP64 size)
   b += 3 * 8 * n + n;                   // profile, two FP64 staging fields, contact set
   b += 5 * 4 * n + 5 * 8 * n;           // FP32 and FP64 CG fields
-  b += 16 * (M + 1) * py;               // spectrum set-up workspace
+  b += 16 * (M + 1) * hyq;              // spectrum set-up workspace
   b += 1 << 20;                         // partial sums, statistics, scalars
   b += b / 3;                           // contact-box sub-contexts (tori of 1/4, 1/16, ... the area)
   return b;

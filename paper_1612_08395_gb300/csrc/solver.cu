@@ -408,7 +408,7 @@ PassArgs<T> make_args(bem_ctx* h) {
   a.khat = khat_of<T>(h);
   const size_t M = h->px / 2, P = h->py;
   if constexpr (sizeof(T) == 8) {
-    a.twA = h->tw64; a.twB = h->tw64 + M; a.twS = h->tw64 + M + P; a.twB16 = h->tw64 + M + P + M + 1;
+    a.twA = h->tw64; a.twB = h->tw64 + M; a.twS = h->tw64 + M + P;
   } else {
     a.twA = h->tw32; a.twB = h->tw32 + M; a.twS = h->tw32 + M + P; a.twB16 = h->tw32 + M + P + M + 1;
   }
@@ -1386,10 +1386,7 @@ std::map<ShapeKey, Tuned> g_tuned;
 int set_plan32(bem_ctx* h, const Plan& pl) {
   h->plan32 = pl;
   CKR(update_w_map(h, pl.nbA));
-  int* g32 = h->geo;
-  const int M = h->px / 2;
-  launch_geo_tables(g32, g32 + kSoEntries, pl.gA, 4, h->stream);
-  launch_geo_tables(g32 + kSoEntries + M, g32 + 2 * kSoEntries + M, pl.gB, 4, h->stream);
+  // the index tables depend on the lengths only (the row pads enter through rs)
   return BEM_OK;
 }
 
@@ -1562,7 +1559,7 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
   if ((rc = dmalloc(h, (void**)&h->kq64, sizeof(double) * (size_t)hyq * (M + 1)))) return cleanup(rc);
   // [length-M stages | length-Py stages | split | radix-16 length-Py stages]
   const size_t ntw = (size_t)M + h->py + M + 1 + h->py;
-  if ((rc = dmalloc(h, (void**)&h->tw64, sizeof(double2) * ntw))) return cleanup(rc);
+  if ((rc = dmalloc(h, (void**)&h->tw64, sizeof(double2) * (ntw - h->py)))) return cleanup(rc);
   if ((rc = dmalloc(h, (void**)&h->tw32, sizeof(float2) * ntw))) return cleanup(rc);
   if ((rc = dmalloc(h, (void**)&h->twfx, sizeof(int4) * (ntw - h->py)))) return cleanup(rc);
   if ((rc = dmalloc(h, (void**)&h->fxe, sizeof(int) * ((size_t)Ny + M + 1)))) return cleanup(rc);
@@ -1594,18 +1591,20 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
     return cleanup(fail(BEM_ECUDA, "memset failed"));
 
   {
+    TableArgs t{};
+    t.logM = ilog2(M);
+    t.logP = ilog2(h->py);
+    t.t64 = h->tw64;
+    t.t32 = h->tw32;
+    t.fx = h->twfx;
     int* g32 = h->geo;
     int* g64 = h->geo + 2 * kSoEntries + M + h->py;
-    launch_geo_tables(g32, g32 + kSoEntries, h->plan32.gA, 4, h->stream);
-    launch_geo_tables(g32 + kSoEntries + M, g32 + 2 * kSoEntries + M, h->plan32.gB, 4, h->stream);
-    launch_geo_tables(g64, g64 + kSoEntries, h->plan64.gA, 8, h->stream);
-    launch_geo_tables(g64 + kSoEntries + M, g64 + 2 * kSoEntries + M, h->plan64.gB, 8, h->stream);
+    t.geo[0] = g32; t.g[0] = h->plan32.gA; t.esize[0] = 4;
+    t.geo[1] = g32 + kSoEntries + M; t.g[1] = h->plan32.gB; t.esize[1] = 4;
+    t.geo[2] = g64; t.g[2] = h->plan64.gA; t.esize[2] = 8;
+    t.geo[3] = g64 + kSoEntries + M; t.g[3] = h->plan64.gB; t.esize[3] = 8;
+    launch_tables(t, h->stream);
   }
-  launch_twiddles(h->tw64, h->tw32, ilog2(M), h->stream);
-  launch_twiddles(h->tw64 + M, h->tw32 + M, ilog2(h->py), h->stream);
-  launch_split_twiddles(h->tw64 + M + h->py, h->tw32 + M + h->py, M, h->stream);
-  launch_fx_tables(h->tw64, h->twfx, (int)(ntw - h->py), h->stream);
-  launch_twiddles16(h->tw64 + M + h->py + M + 1, h->tw32 + M + h->py + M + 1, ilog2(h->py), h->stream);
   // a1: influence coefficients on the offsets 0..Px/2, 0..Py/2 (Eq. 9)
   if (parent) {
     const size_t pw = (size_t)parent->px / 2 + 1;
@@ -1618,7 +1617,7 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
   // spectrum of the even torus extension (Eq. 13: FFT(K)), FP64, once
   {
     void* Wspec = nullptr;
-    if (cudaMalloc(&Wspec, sizeof(double) * 2 * (size_t)(M + 1) * h->py) != cudaSuccess)
+    if (cudaMalloc(&Wspec, sizeof(double) * 2 * (size_t)(M + 1) * hyq) != cudaSuccess)
       return cleanup(fail(BEM_ENOMEM, "spectrum workspace allocation failed"));
     PassArgs<double> a{};
     a.pl = h->plan64;
@@ -1627,8 +1626,8 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
     a.soA = g64; a.spA = g64 + kSoEntries;
     a.soB = g64 + kSoEntries + M; a.spB = g64 + 2 * kSoEntries + M;
     a.W = Wspec;
-    a.rows_w = h->py;
-    a.nrows_in = h->py;
+    a.rows_w = hyq;  // K is even: rows 0..Py/2 of the torus hold all
+    a.nrows_in = hyq;
     a.ncols_in = h->px;
     a.kq64 = h->kq64;
     a.khat64_out = h->khat64;
