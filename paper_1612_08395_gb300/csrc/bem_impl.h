@@ -214,6 +214,7 @@ struct CoopArgs {
   int resume, max_launch;  // as ResArgs
 };
 size_t coop_shared_bytes();
+int coop_ctas(int lm, int lp, int nsm);  // CTAs of a launch, 0 where these lengths have no kernel
 cudaError_t launch_coop_cg(const CoopArgs& r, int lm, int lp, cudaStream_t s);
 cudaError_t launch_coop_pk(const CoopArgs& r, int lm, int lp, cudaStream_t s);
 cudaError_t coop_setup_cg();  // once per device
@@ -255,7 +256,7 @@ template <typename T> void launch_box_gather(const T* p, const T* c, const uint8
                                              int y0, T* bp, T* bc, uint8_t* bS, int bx, int by, cudaStream_t s);
 template <typename T> void launch_box_scatter(const T* bp, T* p, int nx, int ny, int x0, int y0, int bx, int by,
                                               cudaStream_t s);
-template <typename T> void launch_detach(const Plan& pl, Fields<T> f, double* part, Scalars* sc,
+template <typename T> void launch_detach(const Plan& pl, Fields<T> f, double pcrit, double* part, Scalars* sc,
                                          int ngrid, cudaStream_t s);
 template <typename T> void launch_stats(const Plan& pl, const T* p, const T* g, const uint8_t* S,
                                         int use_set, double* part, double* out, int ngrid,
@@ -267,7 +268,10 @@ template <typename T> void launch_mask_field(T* x, const uint8_t* S, size_t n, c
 void launch_refine_apply(double* p64, const float* dp, double dscale, const uint8_t* S, int project,
                          size_t n, cudaStream_t s);
 void launch_to_f32(const double* src, float* dst, size_t n, cudaStream_t s);
-void launch_to_f32_scaled(const double* src, double scale, float* dst, size_t n, cudaStream_t s);
+void launch_refine_rhs(const double* g, double scale, float* c, float* p, float* t, size_t n, cudaStream_t s);
+void launch_max_abs2(const double* a, const double* b, const uint8_t* S, size_t n, unsigned long long* acc,
+                     unsigned int* counter, double* out, cudaStream_t s);
+void launch_set_scalars(const Scalars& v, Scalars* sc, cudaStream_t s);
 // S = (p > 0) or (g < 0): active set of the refinement sweep.
 void launch_active_set(const double* p, const double* g, uint8_t* S, size_t n, cudaStream_t s);
 

@@ -1714,10 +1714,10 @@ __global__ void k_batch_ctl(const PassArgs<T>* __restrict__ arr, int n, unsigned
 
 // Detach every element of S with tensile stress -p > p_crit (Eq. 24).
 template <typename T>
-__global__ void k_detach(int n, Fields<T> f, double* part, Scalars* sc) {
+__global__ void k_detach(int n, Fields<T> f, double pcrit, double* part, Scalars* sc) {
   __shared__ double red[3 * 32];
   __shared__ int lastflag;
-  const T pc = (T)sc->pcrit;
+  const T pc = (T)pcrit;
   T cnt = 0, ns = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     if (f.S[i]) {
@@ -1737,55 +1737,99 @@ __global__ void k_detach(int n, Fields<T> f, double* part, Scalars* sc) {
   sc->n_ic = s[1];
 }
 
+// Bits of |x| as an integer that orders like it; 0 for NaN (as fmax would skip it).
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  const unsigned long long v = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+  return v > 0x7ff0000000000000ull ? 0 : v;
+}
+// Largest value over the CTA, in thread 0 (red: one word per warp).
+__device__ __forceinline__ unsigned long long block_max(unsigned long long v, unsigned long long* red) {
+  const unsigned hi = (unsigned)(v >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)v : 0u);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ((unsigned long long)mh << 32) | ml;
+  __syncthreads();
+  unsigned long long m = 0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, red[w]);
+  return m;
+}
+
 // Final statistics: out[0] = sum p, out[1] = #contact, out[2] = max |g| on
 // contact, out[3] = max(-g) off contact.  Contact = S if use_set else p > 0.
+// FP64 arithmetic is what this kernel would be bound by (27 us for 1024^2
+// elements with FP64 counts, comparisons and maxima): counts and maxima are
+// integers, and zero pressures are not added.
 template <typename T>
 __global__ void k_stats(int n, const T* p, const T* g, const uint8_t* S, int use_set, double* part,
                         unsigned int* counter, double* out) {
   __shared__ double red[3 * 32];
-  __shared__ double redm[2][32];
+  __shared__ unsigned long long redm[32];
   __shared__ int lastflag;
-  double sp = 0, cnt = 0, m1 = 0, m2 = 0;
+  double sp = 0;
+  int cnt = 0;
+  unsigned long long m1 = 0, m2 = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double pv = (double)p[i];
-    const bool in = use_set ? (S[i] != 0) : (pv > 0.0);
-    sp += pv;
-    if (in) { cnt += 1.0; if (g) m1 = fmax(m1, fabs((double)g[i])); }
-    else if (g) m2 = fmax(m2, -(double)g[i]);
+    const T pv = p[i];
+    bool zero, pos;
+    if constexpr (sizeof(T) == 8) {
+      const long long b = __double_as_longlong(pv);
+      zero = (b << 1) == 0;
+      pos = b > 0 && b <= 0x7ff0000000000000ll;
+    } else {
+      zero = pv == (T)0;
+      pos = pv > (T)0;
+    }
+    if (!zero) sp += (double)pv;
+    const bool in = use_set ? (S[i] != 0) : pos;
+    cnt += in;
+    if (g) {
+      const T gv = g[i];
+      unsigned long long b;
+      bool neg;
+      if constexpr (sizeof(T) == 8) {
+        b = abs_bits(gv);
+        neg = __double_as_longlong(gv) < 0;
+      } else {  // ordered as FP32, widened once at the end
+        const unsigned f = __float_as_uint(gv) & 0x7fffffffu;
+        b = f > 0x7f800000u ? 0 : f;
+        neg = gv < (T)0;
+      }
+      if (in) m1 = max(m1, b);
+      else if (neg) m2 = max(m2, b);
+    }
   }
-  double v[2] = {sp, cnt};
-  // max reductions
-  for (int o = 16; o > 0; o >>= 1) {
-    m1 = fmax(m1, __shfl_down_sync(0xffffffffu, m1, o));
-    m2 = fmax(m2, __shfl_down_sync(0xffffffffu, m2, o));
-  }
-  if ((threadIdx.x & 31) == 0) { redm[0][threadIdx.x >> 5] = m1; redm[1][threadIdx.x >> 5] = m2; }
+  double v[2] = {sp, (double)cnt};
   block_sum<2>(v, red);
+  m1 = block_max(m1, redm);
+  m2 = block_max(m2, redm);
   if (threadIdx.x == 0) {
-    double a1 = 0, a2 = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { a1 = fmax(a1, redm[0][w]); a2 = fmax(a2, redm[1][w]); }
     double* pp = part + 4 * blockIdx.x;
-    pp[0] = v[0]; pp[1] = v[1]; pp[2] = a1; pp[3] = a2;
+    pp[0] = v[0]; pp[1] = v[1];
+    pp[2] = __longlong_as_double((long long)m1); pp[3] = __longlong_as_double((long long)m2);
   }
   if (!last_block_arrival(counter, &lastflag)) return;
   // fixed-order parallel reduction of the per-CTA partials
-  double s0 = 0, s1 = 0, x1 = 0, x2 = 0;
+  double s0 = 0, s1 = 0;
+  unsigned long long x1 = 0, x2 = 0;
   for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
     s0 += __ldcg(part + 4 * b); s1 += __ldcg(part + 4 * b + 1);
-    x1 = fmax(x1, __ldcg(part + 4 * b + 2)); x2 = fmax(x2, __ldcg(part + 4 * b + 3));
+    x1 = max(x1, (unsigned long long)__double_as_longlong(__ldcg(part + 4 * b + 2)));
+    x2 = max(x2, (unsigned long long)__double_as_longlong(__ldcg(part + 4 * b + 3)));
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    x1 = fmax(x1, __shfl_down_sync(0xffffffffu, x1, o));
-    x2 = fmax(x2, __shfl_down_sync(0xffffffffu, x2, o));
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) { redm[0][threadIdx.x >> 5] = x1; redm[1][threadIdx.x >> 5] = x2; }
   double v2[2] = {s0, s1};
   block_sum<2>(v2, red);
+  x1 = block_max(x1, redm);
+  x2 = block_max(x2, redm);
   if (threadIdx.x == 0) {
-    double a1 = 0, a2 = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { a1 = fmax(a1, redm[0][w]); a2 = fmax(a2, redm[1][w]); }
-    out[0] = v2[0]; out[1] = v2[1]; out[2] = a1; out[3] = a2;
+    out[0] = v2[0]; out[1] = v2[1];
+    if constexpr (sizeof(T) == 8) {
+      out[2] = __longlong_as_double((long long)x1);
+      out[3] = __longlong_as_double((long long)x2);
+    } else {
+      out[2] = (double)__uint_as_float((unsigned)x1);
+      out[3] = (double)__uint_as_float((unsigned)x2);
+    }
     *counter = 0;
   }
 }
@@ -2172,9 +2216,9 @@ void launch_cg_finish(const Plan& pl, Fields<T> f, const Scalars* sc, int ngrid,
   k_cg_finish<T><<<ngrid, 256, 0, s>>>(pl.nx, f, sc);
 }
 template <typename T>
-void launch_detach(const Plan& pl, Fields<T> f, double* part, Scalars* sc, int ngrid,
+void launch_detach(const Plan& pl, Fields<T> f, double pcrit, double* part, Scalars* sc, int ngrid,
                    cudaStream_t s) {
-  k_detach<T><<<ngrid, 256, 0, s>>>(pl.nx * pl.ny, f, part, sc);
+  k_detach<T><<<ngrid, 256, 0, s>>>(pl.nx * pl.ny, f, pcrit, part, sc);
 }
 template <typename T>
 void launch_stats(const Plan& pl, const T* p, const T* g, const uint8_t* S, int use_set,
@@ -2218,7 +2262,7 @@ void launch_mask_field(T* x, const uint8_t* S, size_t n, cudaStream_t s) {
   template void launch_box_gather<T>(const T*, const T*, const uint8_t*, int, int, int, int, T*, T*, \
                                      uint8_t*, int, int, cudaStream_t);                         \
   template void launch_box_scatter<T>(const T*, T*, int, int, int, int, int, int, cudaStream_t); \
-  template void launch_detach<T>(const Plan&, Fields<T>, double*, Scalars*, int, cudaStream_t); \
+  template void launch_detach<T>(const Plan&, Fields<T>, double, double*, Scalars*, int, cudaStream_t); \
   template void launch_cg_finish<T>(const Plan&, Fields<T>, const Scalars*, int, cudaStream_t); \
   template void launch_stats<T>(const Plan&, const T*, const T*, const uint8_t*, int, double*, \
                                 double*, int, cudaStream_t);                                   \

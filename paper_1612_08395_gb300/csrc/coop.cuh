@@ -35,12 +35,37 @@ struct CoopGeo {
 };
 
 // State of the grid barrier and the partial sums (device memory of the handle).
+constexpr int kCoopMaxCtas = 256;
 struct CoopShared {
-  unsigned int count, fail;
-  unsigned int pad[30];
-  float2 part[2][256 * 8];  // alternating between consecutive sums
+  unsigned int count, pad[31];           // arrivals at the grid barrier
+  float2 part[2][kCoopMaxCtas * 8];      // alternating between consecutive sums
 };
-size_t coop_shared_bytes();
+
+// Grid barrier: every CTA's earlier global writes are visible to every CTA
+// afterwards (read with L2 loads).  One counter, polled by one thread per CTA: a
+// word per CTA polled by everybody's first warp keeps the L2 busy with the polls
+// (a fixed-set iteration of 129 CTAs took 29 us instead of 14).  False: the wait
+// ran out (about a second).
+__device__ __forceinline__ bool coop_grid_sync(CoopShared* cs, int nb, unsigned* target, int* bad) {
+  *target += nb;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned v;
+    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(&cs->count) : "memory");
+    ++v;
+    unsigned long long t0 = 0;
+    for (int i = 0; (int)(v - *target) < 0; ++i) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&cs->count) : "memory");
+      if ((i & 1023) == 1023) {
+        const unsigned long long t = global_ns();
+        if (!t0) t0 = t;
+        else if (t - t0 > kMbarMaxNs) { *bad = 1; break; }
+      }
+    }
+  }
+  __syncthreads();
+  return *bad == 0;
+}
 
 template <int LM, int LP>
 struct Coop {
@@ -61,32 +86,13 @@ struct Coop {
     CoopShared* cs;
     float2* work;
     int R, rows, nb, blk;  // rows per CTA, rows in all, CTAs, this CTA
-    unsigned target;       // barrier count of the next barrier
+    unsigned target;       // barrier count after the last barrier
     int* bad;              // shared: a wait ran out
     int magic;             // ceil(65536 / (R / 2))
   };
 
-  // Every CTA's earlier global writes are visible to every CTA afterwards (read
-  // with L2 loads).  False: the wait ran out.
   static __device__ __forceinline__ bool grid_sync(Ctx& c) {
-    __syncthreads();
-    c.target += c.nb;
-    if (threadIdx.x == 0) {
-      unsigned old;
-      asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(&c.cs->count) : "memory");
-      unsigned v = old + 1;
-      unsigned long long t0 = 0;
-      for (int i = 0; (int)(v - c.target) < 0; ++i) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&c.cs->count) : "memory");
-        if ((i & 1023) == 1023) {
-          const unsigned long long t = global_ns();
-          if (!t0) t0 = t;
-          else if (t - t0 > kMbarMaxNs) { *c.bad = 1; break; }
-        }
-      }
-    }
-    __syncthreads();
-    return *c.bad == 0;
+    return coop_grid_sync(c.cs, c.nb, &c.target, c.bad);
   }
 
   // Rows: transform input x(row slot, element pair index) -> W.
@@ -304,7 +310,7 @@ struct Coop {
     if (wid == 0) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) v[q] = lane < ns ? red[q * 32 + lane] : make_float2(0.f, 0.f);
-      warp_sum_ff<NQ>(v);
+      warp_sum_all<NQ>(v);
     }
     return true;
   }
@@ -375,170 +381,118 @@ struct Coop {
     }
     __syncthreads();
     bool ok = true;
-    float2 v5[5];
-    if (!PK && !ca.resume) {  // the initial residual
-      phase_a(c, [&](int sl, int t_, float2* v) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          v[e] = FR::first_half(e) ? fp[sl * (M / 2) + FR::n0(t_, e)] : make_float2(0.f, 0.f);
-      });
-      ok = grid_sync(c);
-      if (ok) { phase_b(c); ok = grid_sync(c); }
-      float acc[2] = {0.f, 0.f};
-      if (ok) {
-        phase_c(c, [&](int sl, int t_, float2* v) {
-          const unsigned Sr = S >> (8 * (sl / Gm::RPR));
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            if (!FR::first_half(e)) continue;
-            const int i = sl * (M / 2) + FR::n0(t_, e);
-            const float2 cv = fx[i];
-            float2 gv;
-            gv.x = Sr >> (2 * slot(e)) & 1 ? us * v[e].x + cv.x : 0.f;
-            gv.y = Sr >> (2 * slot(e) + 1) & 1 ? us * v[e].y + cv.y : 0.f;
-            acc[0] += gv.x * gv.x + gv.y * gv.y;
-            acc[1] += cv.x * cv.x + cv.y * cv.y;
-            fg[i] = gv;
-            fx[i] = make_float2(0.f, 0.f);
-          }
-        });
-        ok = sum<2>(c, acc, red, &par, v5);
-        if (ok && tid < 32) finalize_cg_g(&sc, v5);
-        __syncthreads();
-      }
-    }
-    for (int it = 0; ok && it < ca.max_launch && !sc.done; ++it) {
+    // one transform per pass of this loop, whatever it is for (see resident.cuh)
+    enum { kP, kT, kG };
+    int step = PK ? kP : ca.resume ? kT : kG;
+    for (int it = 0; it < ca.max_launch && !sc.done;) {
       const bool upd = sc.have_tau != 0;
-      const float tau = (float)sc.tau;
-      if (PK) {
-        float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        phase_a(c, [&](int sl, int t_, float2* v) {
-          const unsigned onr = on >> (8 * (sl / Gm::RPR));
+      const float tau = (float)sc.tau, beta = (float)sc.beta;
+      float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+      float2 v5[5];
+      phase_a(c, [&](int sl, int t_, float2* v) {
+        const int rd = 8 * (sl / Gm::RPR);
+        const unsigned onr = on >> rd, Sr = S >> rd;
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            v[e] = make_float2(0.f, 0.f);
-            if (!FR::first_half(e)) continue;
-            const int i = sl * (M / 2) + FR::n0(t_, e);
-            float2 pv = fp[i];
-            const float2 tv = ft[i], gv = fg[i];
-            PIn<float> q;
-            if (onr >> (2 * slot(e)) & 1) {
-              q.p = pv.x; q.t = tv.x; q.g = gv.x;
-              pv.x = pro_value<float, A_PK_P>(q, upd, tau, 0.f, acc);
-            }
-            if (onr >> (2 * slot(e) + 1) & 1) {
-              q.p = pv.y; q.t = tv.y; q.g = gv.y;
-              pv.y = pro_value<float, A_PK_P>(q, upd, tau, 0.f, acc);
-            }
-            if (upd) fp[i] = pv;
-            v[e] = pv;
-          }
-        });
-        if (!(ok = grid_sync(c))) break;
-        phase_b(c);
-        if (!(ok = grid_sync(c))) break;
-        phase_c(c, [&](int sl, int t_, float2* v) {
-          const unsigned onr = on >> (8 * (sl / Gm::RPR));
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            if (!FR::first_half(e)) continue;
-            const int i = sl * (M / 2) + FR::n0(t_, e);
-            const float2 cv = fx[i], pv = fp[i];
-            float2 gv = make_float2(0.f, 0.f);
-            if (onr >> (2 * slot(e)) & 1) {
-              gv.x = us * v[e].x + cv.x;
-              if (pv.x > 0.f) { acc[3] += gv.x * gv.x; acc[4] += 1.f; }
-            }
-            if (onr >> (2 * slot(e) + 1) & 1) {
-              gv.y = us * v[e].y + cv.y;
-              if (pv.y > 0.f) { acc[3] += gv.y * gv.y; acc[4] += 1.f; }
-            }
-            fg[i] = gv;
-          }
-        });
-        if (!(ok = sum<5>(c, acc, red, &par, v5))) break;
-        if (tid < 32) finalize_pk_g(&sc, v5);
-        __syncthreads();
-        if (sc.done) break;
-        const float beta = (float)sc.beta;
-        phase_a(c, [&](int sl, int t_, float2* v) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            v[e] = make_float2(0.f, 0.f);
-            if (!FR::first_half(e)) continue;
-            const int i = sl * (M / 2) + FR::n0(t_, e);
-            const float2 pv = fp[i], gv = fg[i];
-            float2 tv = ft[i];
-            tv.x = pv.x > 0.f ? gv.x + beta * tv.x : 0.f;
-            tv.y = pv.y > 0.f ? gv.y + beta * tv.y : 0.f;
-            ft[i] = tv;
-            v[e] = tv;
-          }
-        });
-        if (!(ok = grid_sync(c))) break;
-        phase_b(c);
-        if (!(ok = grid_sync(c))) break;
-        float ac2[2] = {0.f, 0.f};
-        phase_c(c, [&](int sl, int t_, float2* v) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            if (!FR::first_half(e)) continue;
-            const int i = sl * (M / 2) + FR::n0(t_, e);
-            const float2 pv = fp[i], gv = fg[i], tv = ft[i];
-            if (pv.x > 0.f) { ac2[0] += gv.x * tv.x; ac2[1] += us * v[e].x * tv.x; }
-            if (pv.y > 0.f) { ac2[0] += gv.y * tv.y; ac2[1] += us * v[e].y * tv.y; }
-          }
-        });
-        if (!(ok = sum<2>(c, ac2, red, &par, v5))) break;
-        if (tid < 32) finalize_pk_r(&sc, v5);
-        __syncthreads();
-      } else {
-        const float beta = (float)sc.beta;
-        phase_a(c, [&](int sl, int t_, float2* v) {
-          const unsigned Sr = S >> (8 * (sl / Gm::RPR));
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            v[e] = make_float2(0.f, 0.f);
-            if (!FR::first_half(e)) continue;
-            const int i = sl * (M / 2) + FR::n0(t_, e);
+        for (int e = 0; e < 8; ++e) {
+          v[e] = make_float2(0.f, 0.f);
+          if (!FR::first_half(e)) continue;
+          const int i = sl * (M / 2) + FR::n0(t_, e);
+          float2 pv = fp[i];
+          if (step == kT) {
             float2 gv = fg[i], tv = ft[i];
-            if (upd) {
+            if (!PK && upd) {
               const float2 xv = fx[i];
-              float2 pv = fp[i];
               pv.x -= tau * tv.x; pv.y -= tau * tv.y;
               gv.x -= tau * xv.x; gv.y -= tau * xv.y;
               fp[i] = pv;
               fg[i] = gv;
             }
-            tv.x = Sr >> (2 * slot(e)) & 1 ? gv.x + beta * tv.x : 0.f;
-            tv.y = Sr >> (2 * slot(e) + 1) & 1 ? gv.y + beta * tv.y : 0.f;
+            const bool in0 = PK ? pv.x > 0.f : (Sr >> (2 * slot(e)) & 1) != 0;
+            const bool in1 = PK ? pv.y > 0.f : (Sr >> (2 * slot(e) + 1) & 1) != 0;
+            tv.x = in0 ? gv.x + beta * tv.x : 0.f;
+            tv.y = in1 ? gv.y + beta * tv.y : 0.f;
             ft[i] = tv;
             v[e] = tv;
+          } else {
+            if (PK) {
+              const float2 tv = ft[i], gv = fg[i];
+              PIn<float> q;
+              if (onr >> (2 * slot(e)) & 1) {
+                q.p = pv.x; q.t = tv.x; q.g = gv.x;
+                pv.x = pro_value<float, A_PK_P>(q, upd, tau, 0.f, acc);
+              }
+              if (onr >> (2 * slot(e) + 1) & 1) {
+                q.p = pv.y; q.t = tv.y; q.g = gv.y;
+                pv.y = pro_value<float, A_PK_P>(q, upd, tau, 0.f, acc);
+              }
+              if (upd) fp[i] = pv;
+            }
+            v[e] = pv;
           }
-        });
-        if (!(ok = grid_sync(c))) break;
-        phase_b(c);
-        if (!(ok = grid_sync(c))) break;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        phase_c(c, [&](int sl, int t_, float2* v) {
-          const unsigned Sr = S >> (8 * (sl / Gm::RPR));
+        }
+      });
+      if (!(ok = grid_sync(c))) break;
+      phase_b(c);
+      if (!(ok = grid_sync(c))) break;
+      phase_c(c, [&](int sl, int t_, float2* v) {
+        const int rd = 8 * (sl / Gm::RPR);
+        const unsigned onr = on >> rd, Sr = S >> rd;
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            if (!FR::first_half(e)) continue;
-            const int i = sl * (M / 2) + FR::n0(t_, e);
-            const float2 gv = fg[i], tv = ft[i];
-            float2 rv;
-            rv.x = Sr >> (2 * slot(e)) & 1 ? us * v[e].x : 0.f;
-            rv.y = Sr >> (2 * slot(e) + 1) & 1 ? us * v[e].y : 0.f;
-            fx[i] = rv;
-            acc[0] += rv.x * tv.x; acc[1] += rv.x * gv.x; acc[2] += rv.x * rv.x; acc[3] += gv.x * gv.x;
-            acc[0] += rv.y * tv.y; acc[1] += rv.y * gv.y; acc[2] += rv.y * rv.y; acc[3] += gv.y * gv.y;
+        for (int e = 0; e < 8; ++e) {
+          if (!FR::first_half(e)) continue;
+          const int i = sl * (M / 2) + FR::n0(t_, e);
+          const float2 w = make_float2(us * v[e].x, us * v[e].y);
+          if (PK) {
+            const float2 pv = fp[i];
+            if (step == kT) {
+              const float2 gv = fg[i], tv = ft[i];
+              if (pv.x > 0.f) { acc[0] += gv.x * tv.x; acc[1] += w.x * tv.x; }
+              if (pv.y > 0.f) { acc[0] += gv.y * tv.y; acc[1] += w.y * tv.y; }
+            } else {
+              const float2 cv = fx[i];
+              float2 gv = make_float2(0.f, 0.f);
+              if (onr >> (2 * slot(e)) & 1) {
+                gv.x = w.x + cv.x;
+                if (pv.x > 0.f) { acc[3] += gv.x * gv.x; acc[4] += 1.f; }
+              }
+              if (onr >> (2 * slot(e) + 1) & 1) {
+                gv.y = w.y + cv.y;
+                if (pv.y > 0.f) { acc[3] += gv.y * gv.y; acc[4] += 1.f; }
+              }
+              fg[i] = gv;
+            }
+          } else {
+            const bool in0 = Sr >> (2 * slot(e)) & 1, in1 = Sr >> (2 * slot(e) + 1) & 1;
+            if (step == kT) {
+              const float2 gv = fg[i], tv = ft[i];
+              const float2 rv = make_float2(in0 ? w.x : 0.f, in1 ? w.y : 0.f);
+              fx[i] = rv;
+              acc[0] += rv.x * tv.x; acc[1] += rv.x * gv.x; acc[2] += rv.x * rv.x; acc[3] += gv.x * gv.x;
+              acc[0] += rv.y * tv.y; acc[1] += rv.y * gv.y; acc[2] += rv.y * rv.y; acc[3] += gv.y * gv.y;
+            } else {
+              const float2 cv = fx[i];
+              const float2 gv = make_float2(in0 ? w.x + cv.x : 0.f, in1 ? w.y + cv.y : 0.f);
+              acc[0] += gv.x * gv.x + gv.y * gv.y;
+              acc[1] += cv.x * cv.x + cv.y * cv.y;
+              fg[i] = gv;
+              fx[i] = make_float2(0.f, 0.f);
+            }
           }
-        });
-        if (!(ok = sum<4>(c, acc, red, &par, v5))) break;
-        if (tid < 32) finalize_cg_r(&sc, v5);
-        __syncthreads();
+        }
+      });
+      if (!(ok = sum<PK ? 5 : 4>(c, acc, red, &par, v5))) break;
+      if (tid < 32) {
+        if (PK) {
+          if (step == kP) finalize_pk_g(&sc, v5);
+          else finalize_pk_r(&sc, v5);
+        } else {
+          if (step == kG) finalize_cg_g(&sc, v5);
+          else finalize_cg_r(&sc, v5);
+        }
       }
+      __syncthreads();
+      if (step == kT) ++it;
+      step = PK && step == kT ? kP : kT;
     }
     if (!ok) {  // a wait ran out: give up together
       if (tid == 0 && a.kerr) atomicOr(a.kerr, 1u);
@@ -602,7 +556,7 @@ constexpr size_t coop_smem(int R) { return 8 * (size_t)CoopGeo<LM, LP>::work + 1
 template <int LM, int LP>
 inline void coop_shape(int rows, int nsm, int* nb, int* R) {
   using Gm = CoopGeo<LM, LP>;
-  *nb = std::min(std::min(nsm, 256), (Gm::M + 1 + Gm::CPR - 1) / Gm::CPR);
+  *nb = std::min(std::min(nsm, kCoopMaxCtas), (Gm::M + 1 + Gm::CPR - 1) / Gm::CPR);
   *R = 2 * std::max(1, (rows + 2 * *nb - 1) / (2 * *nb));
 }
 
@@ -616,7 +570,7 @@ cudaError_t launch_coop_kind(CoopArgs r, int lm, int lp, cudaStream_t s) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   // a fresh barrier for every launch
-  cudaError_t e = cudaMemsetAsync(r.shared, 0, 2 * sizeof(unsigned int), s);
+  cudaError_t e = cudaMemsetAsync(r.shared, 0, sizeof(unsigned int), s);
   if (e != cudaSuccess) return e;
   switch (lm * 16 + lp) {
 #define BEM_CASE(LM, LP)                                                     \

@@ -21,13 +21,55 @@ void launch_refine_apply(double* p64, const float* dp, double dscale, const uint
   k_refine_apply<<<ew_grid(n), 256, 0, s>>>(p64, dp, dscale, S, project, n);
 }
 
-__global__ void k_to_f32_scaled(const double* src, double scale, float* dst, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    dst[i] = (float)(scale * src[i]);
+// The correction's data: c = scale g, p = t = 0.
+__global__ void k_refine_rhs(const double* g, double scale, float* c, float* p, float* t, size_t n) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    c[i] = (float)(scale * g[i]);
+    p[i] = 0.f;
+    t[i] = 0.f;
+  }
 }
-void launch_to_f32_scaled(const double* src, double scale, float* dst, size_t n, cudaStream_t s) {
-  k_to_f32_scaled<<<ew_grid(n), 256, 0, s>>>(src, scale, dst, n);
+void launch_refine_rhs(const double* g, double scale, float* c, float* p, float* t, size_t n, cudaStream_t s) {
+  k_refine_rhs<<<ew_grid(n), 256, 0, s>>>(g, scale, c, p, t, n);
 }
+
+// out[0] = max |a|, out[1] = max |b| over S (NaN skipped), as FP64; acc: two
+// words and a counter, zero before and after.
+__global__ void k_max_abs2(const double* __restrict__ a, const double* __restrict__ b, const uint8_t* __restrict__ S,
+                           size_t n, unsigned long long* acc, unsigned int* counter, double* out) {
+  __shared__ unsigned long long red[32];
+  __shared__ int lastflag;
+  unsigned long long ma = 0, mb = 0;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    if (!S[i]) continue;
+    ma = max(ma, abs_bits(a[i]));
+    mb = max(mb, abs_bits(b[i]));
+  }
+  ma = block_max(ma, red);
+  mb = block_max(mb, red);
+  if (threadIdx.x == 0) {
+    if (ma) atomicMax(acc, ma);
+    if (mb) atomicMax(acc + 1, mb);
+  }
+  if (!last_block_arrival(counter, &lastflag)) return;
+  if (threadIdx.x == 0) {
+    out[0] = __longlong_as_double((long long)atomicExch(acc, 0ull));
+    out[1] = __longlong_as_double((long long)atomicExch(acc + 1, 0ull));
+    *counter = 0;
+  }
+}
+void launch_max_abs2(const double* a, const double* b, const uint8_t* S, size_t n, unsigned long long* acc,
+                     unsigned int* counter, double* out, cudaStream_t s) {
+  k_max_abs2<<<std::min(ew_grid(n), 304), 256, 0, s>>>(a, b, S, n, acc, counter, out);
+}
+
+// The solve's scalars, all but the sticky error word: by kernel argument, so no
+// copy engine, pinned staging or host wait is involved.
+__global__ void k_set_scalars(Scalars v, Scalars* sc) {
+  for (int i = threadIdx.x; i < (int)(offsetof(Scalars, kerr) / 4); i += blockDim.x)
+    reinterpret_cast<int*>(sc)[i] = reinterpret_cast<const int*>(&v)[i];
+}
+void launch_set_scalars(const Scalars& v, Scalars* sc, cudaStream_t s) { k_set_scalars<<<1, 32, 0, s>>>(v, sc); }
 
 __global__ void k_to_f32(const double* src, float* dst, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)

@@ -81,13 +81,14 @@ __device__ __forceinline__ void cl_st4(unsigned addr, float2 v, float2 w) {
 __device__ __forceinline__ float2 ff_xor(float2 v, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
+
 // Sums of NQ (2, 4 or 5) float-float values over the lanes of a warp.  The first
 // levels scatter: a lane passes on half of its values and keeps the other half,
-// so that two or four sums take six additions a lane instead of ten or twenty
-// (a float-float addition is ten instructions, and every warp of the CTA forms
-// these sums).  The totals are returned in v of every lane; with `mine`, only
-// the lane's own one, of quantity warp_sum_q(lane) (a fifth one comes in v[4] of
-// every lane), in v[0].  ff_add is commutative, so all lanes hold the same bits.
+// so that two or four sums take six additions a lane instead of ten or twenty (a
+// float-float addition is ten instructions, and every warp of the CTA forms
+// these sums).  The lane's own quantity, warp_sum_q(lane), is
+// returned in v[0], a fifth one in v[4] of every lane; the additions commute, so
+// all lanes of a quantity hold the same bits.
 template <int NQ>
 __device__ __forceinline__ int warp_sum_q(int lane) { return NQ == 2 ? lane >> 4 : lane >> 3; }
 template <int NQ>
@@ -99,7 +100,7 @@ __device__ __forceinline__ void warp_sum_mine(float2* v) {
     for (int o = 16; o > 0; o >>= 1) v[NQ - 1] = ff_add(v[NQ - 1], ff_xor(v[NQ - 1], o));
   }
   float2 a;
-  if (NQ == 2) {
+  if constexpr (NQ == 2) {
     a = ff_add(h4 ? v[1] : v[0], ff_xor(h4 ? v[0] : v[1], 16));
     a = ff_add(a, ff_xor(a, 8));
   } else {
@@ -111,23 +112,23 @@ __device__ __forceinline__ void warp_sum_mine(float2* v) {
   for (int o = 4; o > 0; o >>= 1) a = ff_add(a, ff_xor(a, o));
   v[0] = a;
 }
+// ... the totals in every lane
 template <int NQ>
-__device__ __forceinline__ void warp_sum_ff(float2* v) {
+__device__ __forceinline__ void warp_sum_all(float2* v) {
   warp_sum_mine<NQ>(v);
   const float2 a = v[0];
   constexpr int W = NQ == 2 ? 16 : 8, N = NQ == 2 ? 2 : 4;
 #pragma unroll
-  for (int q = 0; q < N; ++q)
-    v[q] = make_float2(__shfl_sync(0xffffffffu, a.x, q * W), __shfl_sync(0xffffffffu, a.y, q * W));
+  for (int q = 0; q < N; ++q) v[q] = make_float2(__shfl_sync(0xffffffffu, a.x, q * W), __shfl_sync(0xffffffffu, a.y, q * W));
 }
-// One warp's sums into red[q * stride + i] (leading lanes write).
+// ... one warp's sums into red[q * stride + i] (leading lanes write)
 template <int NQ>
 __device__ __forceinline__ void warp_sum_store(float2* v, float2* red, int stride, int i) {
   warp_sum_mine<NQ>(v);
   const int lane = threadIdx.x & 31;
   constexpr int W = NQ == 2 ? 16 : 8;
   if ((lane & (W - 1)) == 0) red[warp_sum_q<NQ>(lane) * stride + i] = v[0];
-  if (NQ == 5 && lane == 1) red[4 * stride + i] = v[4];
+  if (NQ == 5 && lane == 1) red[4 * stride + i] = v[NQ - 1];
 }
 
 // The scalar decisions of pass_c_finalize taken by one warp on sums that every
@@ -434,7 +435,7 @@ struct Resident {
     if (wid == 0) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) v[q] = lane < nw ? red[q * nw + lane] : make_float2(0.f, 0.f);
-      warp_sum_ff<NQ>(v);
+      warp_sum_all<NQ>(v);
       if (lane < CS) {
 #pragma unroll
         for (int q = 0; q < NQ; ++q) cl_st2(cl_map(slots + rank * 8 + q, lane), v[q]);
@@ -444,7 +445,7 @@ struct Resident {
     if (wid == 0) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) v[q] = lane < CS ? slots[lane * 8 + q] : make_float2(0.f, 0.f);
-      warp_sum_ff<NQ>(v);
+      warp_sum_all<NQ>(v);
     }
   }
 
@@ -508,78 +509,68 @@ struct Resident {
       }
     }
     cl_sync();  // every CTA's buffers are cleared before anyone stores into them
-    float2 v5[5];
-    if (!PK && !ra_.resume) {  // the initial residual
-      conv(a, sm, rank, ny, p, u, us);
-      float acc[2] = {0.f, 0.f};
+    // One transform per pass of this loop, whatever it is for, so that its code
+    // exists once (the loop's instructions are fetched for a few warps only).
+    //   PK: kP updates p and forms the gap, kT the direction and its transform;
+    //   CG: kG forms the initial residual, kT is an iteration.
+    enum { kP, kT, kG };
+    int step = PK ? kP : ra_.resume ? kT : kG;
+    for (int it = 0; it < ra_.max_launch && !sc.done;) {
+      const bool upd = sc.have_tau != 0;
+      const float tau = (float)sc.tau, beta = (float)sc.beta;
+      float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, y[8];
+      float2 v5[5];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        g[i] = S >> i & 1 ? u[i] + x[i] : 0.f;
-        acc[0] += g[i] * g[i];
-        acc[1] += x[i] * x[i];
-        x[i] = 0.f;
-      }
-      sum<2>(acc, red, slots, rank, v5);
-      if (tid < 32) finalize_cg_g(&sc, v5);
-      __syncthreads();
-    }
-    for (int it = 0; it < ra_.max_launch && !sc.done; ++it) {
-      const bool upd = sc.have_tau != 0;
-      const float tau = (float)sc.tau;
-      if (PK) {
-        float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (on >> i & 1) {
+        if (step == kT) {
+          if (!PK && upd) { p[i] -= tau * tt[i]; g[i] -= tau * x[i]; }
+          tt[i] = (PK ? p[i] > 0.f : (S >> i & 1) != 0) ? g[i] + beta * tt[i] : 0.f;
+          y[i] = tt[i];
+        } else {
+          if (PK && (on >> i & 1)) {
             PIn<float> q;
             q.p = p[i]; q.t = tt[i]; q.g = g[i];
             p[i] = pro_value<float, A_PK_P>(q, upd, tau, 0.f, acc);
           }
+          y[i] = p[i];
         }
-        conv(a, sm, rank, ny, p, u, us);
+      }
+      conv(a, sm, rank, ny, y, u, us);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (on >> i & 1) {
+      for (int i = 0; i < 8; ++i) {
+        if (PK) {
+          if (step == kT) {
+            if (p[i] > 0.f) { acc[0] += g[i] * tt[i]; acc[1] += u[i] * tt[i]; }
+          } else if (on >> i & 1) {
             g[i] = u[i] + x[i];
             if (p[i] > 0.f) { acc[3] += g[i] * g[i]; acc[4] += 1.f; }
           }
-        }
-        sum<5>(acc, red, slots, rank, v5);
-        if (tid < 32) finalize_pk_g(&sc, v5);
-        __syncthreads();
-        if (sc.done) break;
-        const float beta = (float)sc.beta;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) tt[i] = p[i] > 0.f ? g[i] + beta * tt[i] : 0.f;
-        conv(a, sm, rank, ny, tt, u, us);
-        float ac2[2] = {0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-          if (p[i] > 0.f) { ac2[0] += g[i] * tt[i]; ac2[1] += u[i] * tt[i]; }
-        sum<2>(ac2, red, slots, rank, v5);
-        if (tid < 32) finalize_pk_r(&sc, v5);
-        __syncthreads();
-      } else {
-        const float beta = (float)sc.beta;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (upd) { p[i] -= tau * tt[i]; g[i] -= tau * x[i]; }
-          tt[i] = S >> i & 1 ? g[i] + beta * tt[i] : 0.f;
-        }
-        conv(a, sm, rank, ny, tt, u, us);
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        } else if (step == kT) {
           x[i] = S >> i & 1 ? u[i] : 0.f;
           acc[0] += x[i] * tt[i];
           acc[1] += x[i] * g[i];
           acc[2] += x[i] * x[i];
           acc[3] += g[i] * g[i];
+        } else {
+          g[i] = S >> i & 1 ? u[i] + x[i] : 0.f;
+          acc[0] += g[i] * g[i];
+          acc[1] += x[i] * x[i];
+          x[i] = 0.f;
         }
-        sum<4>(acc, red, slots, rank, v5);
-        if (tid < 32) finalize_cg_r(&sc, v5);
-        __syncthreads();
       }
+      sum<PK ? 5 : 4>(acc, red, slots, rank, v5);
+      if (tid < 32) {
+        if (PK) {
+          if (step == kP) finalize_pk_g(&sc, v5);
+          else finalize_pk_r(&sc, v5);
+        } else {
+          if (step == kG) finalize_cg_g(&sc, v5);
+          else finalize_cg_r(&sc, v5);
+        }
+      }
+      __syncthreads();
+      if (step == kT) ++it;
+      step = PK && step == kT ? kP : kT;
     }
     // a fixed-set solve may end with its last update pending
     const bool fin = !PK && sc.done && sc.have_tau;

@@ -15,6 +15,7 @@
 #include <mutex>
 #include <vector>
 #include <string>
+#include <type_traits>
 
 #include <cuda.h>  // CUtensorMap (the encoder comes from the driver entry point)
 
@@ -203,10 +204,17 @@ bool plan_fits(const Plan& pl, int esize) { return shape_fits(pl, esize); }
 
 // Devices whose clusters hold the resident loops (set once by device_setup).
 static bool g_resident[64] = {};
-// ... and whether it takes cooperative launches; one cooperative loop runs on a
-// device at a time (its CTAs wait for one another and fill the SMs).
+// ... and whether it takes cooperative launches.  The CTAs of one wait for one
+// another, so all of them must be resident at once: solves of several threads
+// share a budget of one CTA per SM, in order of arrival.
 static bool g_coop[64] = {};
-static std::mutex g_coop_mu[64];
+struct CoopGate {
+  std::mutex mu;
+  std::condition_variable cv;
+  int used = 0;
+  unsigned long long next = 0, serving = 0;
+};
+static CoopGate g_coop_gate[64];
 
 // Once per device and process, with that device current: opt every pass kernel
 // into the shared memory it may ask for, and upload the quadrature nodes.
@@ -287,6 +295,7 @@ struct bem_ctx {
   bem::LoopBatcher* batcher = nullptr;
   cudaEvent_t ev_ready = nullptr;  // this context's work before its batched loop
   void* coop = nullptr;  // barrier and partial sums of the cooperative CG loop
+  int box[4] = {0, -1, 0, -1};  // first/last row and column of the last held or overlap set
   int rows_used = 0;     // sub-contexts: rows of the box (pressure lies in rows 0 .. rows_used - 1)
   // Tensor map of W (FP32) for pass C's TMA staging, with the plan's rows per
   // CTA (device memory; null where TMA does not apply)
@@ -500,10 +509,7 @@ int init_scalars(bem_ctx* h, double tol, int max_iter, double pcrit) {
   s.inject = inj && inj[0] == '1';
 #endif
   *h->sc_host = s;
-  // every member but the sticky error word
-  CK(cudaMemcpyAsync(h->sc, h->sc_host, offsetof(Scalars, kerr), cudaMemcpyHostToDevice, h->stream));
-  // the host copy is reused for reads; make sure the upload has consumed it
-  CK(cudaStreamSynchronize(h->stream));
+  launch_set_scalars(s, h->sc, h->stream);
   return BEM_OK;
 }
 
@@ -929,22 +935,53 @@ cudaError_t launch_resident(const ResArgs& r, const bem_ctx* h, bool pk, int n, 
   return pk ? launch_resident_pk(r, lm, lp, n, s) : launch_resident_cg(r, lm, lp, n, s);
 }
 
-// Whether the loop may run as one cooperative launch over the chip (coop.cuh):
-// FP32, row transforms of 256 to 1024 points and columns of 512 to 2048, the
-// sizes at which the passes' starts and tails cost as much as their work.  The
-// server's loops share launches instead.
-bool coop_applies(const bem_ctx* h, int es) {
-  return es == 4 && h->px >= 512 && h->px <= 2048 && h->py >= 512 && h->py <= 2048 && (h->ny & 1) == 0 &&
-         !h->timing && !h->batcher && g_coop[h->device];
+// Cooperative launches of `ctas` CTAs on this handle's stream may run until the
+// hold ends, which waits for them.
+struct CoopHold {
+  bem_ctx* h = nullptr;
+  int ctas = 0;
+  void acquire(bem_ctx* ctx, int n) {
+    if (ctas >= n) return;  // the stream's launches follow one another
+    release();
+    CoopGate& g = g_coop_gate[ctx->device];
+    std::unique_lock<std::mutex> lk(g.mu);
+    const unsigned long long my = g.next++;
+    g.cv.wait(lk, [&] { return g.serving == my && g.used + n <= ctx->plan32.nsm; });
+    g.serving++;
+    g.used += n;
+    h = ctx;
+    ctas = n;
+    g.cv.notify_all();
+  }
+  void release() {
+    if (!ctas) return;
+    cudaStreamSynchronize(h->stream);
+    CoopGate& g = g_coop_gate[h->device];
+    {
+      std::lock_guard<std::mutex> lk(g.mu);
+      g.used -= ctas;
+    }
+    ctas = 0;
+    g.cv.notify_all();
+  }
+  ~CoopHold() { release(); }
+};
+
+// CTAs of the cooperative launch over the chip (coop.cuh) that this context's CG
+// loops in precision es run as, 0: not.  FP32, row transforms of 256 to 1024
+// points and columns of 512 to 2048, the sizes at which the passes' starts and
+// tails cost as much as their work.  Pass timing needs the separate passes, and
+// the server's loops share launches instead.
+int coop_applies(const bem_ctx* h, int es) {
+  if (es != 4 || h->timing || h->batcher || !g_coop[h->device] || (h->ny & 1)) return 0;
+  return coop_ctas(ilog2(h->px / 2), ilog2(h->py), h->plan32.nsm);
 }
 
-// The whole CG loop over `rows` grid rows as cooperative launches.  *ran = false:
-// another one is running on this device; the caller takes the passes.
-int run_coop(bem_ctx* h, bool pk, int rows, bool* ran) {
-  std::unique_lock<std::mutex> lk(g_coop_mu[h->device], std::try_to_lock);
-  *ran = lk.owns_lock();
-  if (!*ran) return BEM_OK;
+// The whole CG loop over `rows` grid rows as cooperative launches of nb CTAs.
+int run_coop(bem_ctx* h, bool pk, int rows, int nb) {
   if (!h->coop) CKR(dmalloc(h, &h->coop, coop_shared_bytes()));
+  CoopHold hold;
+  hold.acquire(h, nb);
   CoopArgs r{};
   r.one = make_args<float>(h);
   r.shared = h->coop;
@@ -1000,6 +1037,13 @@ int map_status(int sc_status) {
 }
 
 int pick_sub(bem_ctx* h, bem_ctx** out);
+// The box that k_box or k_box_overlap has collected.
+int read_box(bem_ctx* h) {
+  CKR(read_scalars(h));
+  const Scalars& s = *h->sc_host;
+  h->box[0] = s.band0; h->box[1] = s.band1; h->box[2] = s.col0; h->box[3] = s.col1;
+  return BEM_OK;
+}
 template <typename T>
 int pk_in_box(bem_ctx* h, bem_ctx* sub, double d, double tol, int max_iter, bool warm, StepOut* so);
 
@@ -1012,7 +1056,7 @@ int run_pk(bem_ctx* h, double d, double tol, int max_iter, bool warm, StepOut* s
     CKR(init_scalars(h, tol, max_iter, 0.0));
     launch_box_overlap(plan_of<T>(h), h->h64, d, h->sc, h->stream);
     h->launches += 1;
-    CKR(read_scalars(h));
+    CKR(read_box(h));
     bem_ctx* sub = nullptr;
     CKR(pick_sub(h, &sub));
     if (sub) return pk_in_box<T>(h, sub, d, tol, max_iter, warm, so);
@@ -1020,13 +1064,11 @@ int run_pk(bem_ctx* h, double d, double tol, int max_iter, bool warm, StepOut* s
   launch_pk_init<T>(plan_of<T>(h), h->h64, d, pf.c, pf.p, pf.t, warm ? 1 : 0, h->ew_ngrid, h->stream);
   h->launches += 1;
   CKR(init_scalars(h, tol, max_iter, 0.0));
-  bool ran = false;
-  if (coop_applies(h, (int)sizeof(T))) CKR(run_coop(h, true, h->is_sub ? h->rows_used : h->ny, &ran));
-  if (!ran && resident_applies(h, (int)sizeof(T))) {
+  if (const int nb = coop_applies(h, (int)sizeof(T))) {
+    CKR(run_coop(h, true, h->is_sub ? h->rows_used : h->ny, nb));
+  } else if (resident_applies(h, (int)sizeof(T))) {
     CKR(run_resident(h, true));
-    ran = true;
-  }
-  if (!ran) {
+  } else {
     if (!pf.pk_graph[0]) CKR(capture_chunk<T>(h, true, false, &pf.pk_graph[0]));
     if (h->timing && !pf.pk_graph[1]) CKR(capture_chunk<T>(h, true, true, &pf.pk_graph[1]));
     CKR(run_loop(h, pf.pk_graph[0], pf.pk_graph[1], max_iter, true, (int)sizeof(T)));
@@ -1046,9 +1088,8 @@ int run_pk(bem_ctx* h, double d, double tol, int max_iter, bool warm, StepOut* s
 // (they depend only on the element offsets), its spectrum is its own.
 int pick_sub(bem_ctx* h, bem_ctx** out) {
   *out = nullptr;
-  const Scalars& s = *h->sc_host;
-  if (s.band1 < s.band0 || s.col1 < s.col0) return BEM_OK;
-  const int bw = s.col1 - s.col0 + 1, bh = s.band1 - s.band0 + 1;
+  if (h->box[1] < h->box[0] || h->box[3] < h->box[2]) return BEM_OK;
+  const int bw = h->box[3] - h->box[2] + 1, bh = h->box[1] - h->box[0] + 1;
   const int qx = pow2_at_least(2 * bw < 32 ? 32 : 2 * bw), qy = pow2_at_least(2 * bh < 32 ? 32 : 2 * bh);
   if (qx > h->px || qy > h->py || (size_t)qx * qy >= (size_t)h->px * h->py) return BEM_OK;
   for (bem_ctx* c : h->subs)
@@ -1107,8 +1148,8 @@ void absorb_sub(bem_ctx* h, bem_ctx* sub) {
 // the whole grid is formed with one full transform.
 template <typename T>
 int pk_in_box(bem_ctx* h, bem_ctx* sub, double d, double tol, int max_iter, bool warm, StepOut* so) {
-  const int x0 = h->sc_host->col0, y0 = h->sc_host->band0;
-  sub->rows_used = h->sc_host->band1 - y0 + 1;
+  const int x0 = h->box[2], y0 = h->box[0];
+  sub->rows_used = h->box[1] - y0 + 1;
   const size_t n = (size_t)h->nx * h->ny;
   PrecFields<T>& pf = fields_of<T>(h);
   CKR(ensure_fields<T>(sub));
@@ -1143,8 +1184,8 @@ int pk_in_box(bem_ctx* h, bem_ctx* sub, double d, double tol, int max_iter, bool
 // same result as solving on the whole grid.  p outside S is zero either way.
 template <typename T>
 int fixed_cg_in_box(bem_ctx* h, bem_ctx* sub, double tol, int max_iter, double pcrit, StepOut* so) {
-  const int x0 = h->sc_host->col0, y0 = h->sc_host->band0;
-  sub->rows_used = h->sc_host->band1 - y0 + 1;
+  const int x0 = h->box[2], y0 = h->box[0];
+  sub->rows_used = h->box[1] - y0 + 1;
   PrecFields<T>& pf = fields_of<T>(h);
   CKR(ensure_fields<T>(sub));
   PrecFields<T>& bf = fields_of<T>(sub);
@@ -1170,33 +1211,25 @@ int run_fixed_cg(bem_ctx* h, double tol, int max_iter, double pcrit, StepOut* so
   CKR(ensure_fields<T>(h));
   PrecFields<T>& pf = fields_of<T>(h);
   CKR(init_scalars(h, tol, max_iter, pcrit));
-  const bool coop = coop_applies(h, (int)sizeof(T)), resident = resident_applies(h, (int)sizeof(T));
-  bool boxed = !h->is_sub || !(coop || resident);
-  if (boxed) {
+  const int coop = coop_applies(h, (int)sizeof(T));
+  const bool resident = resident_applies(h, (int)sizeof(T));
+  if (!h->is_sub || !(coop || resident)) {  // the passes work on the contact band
     launch_box(plan_of<T>(h), h->S, h->sc, h->stream);
     h->launches += 1;
   }
   int rows = h->rows_used;
   if (!h->is_sub) {
-    CKR(read_scalars(h));
-    rows = h->sc_host->band1 + 1;
+    CKR(read_box(h));
+    rows = h->box[1] + 1;
     bem_ctx* sub = nullptr;
     CKR(pick_sub(h, &sub));
     if (sub) return fixed_cg_in_box<T>(h, sub, tol, max_iter, pcrit, so);
   }
-  bool ran = false;
-  if (coop) CKR(run_coop(h, false, rows, &ran));
-  if (!ran && resident) {
-    CKR(run_resident(h, false));
-    ran = true;
-  }
-  if (ran) {
+  if (coop || resident) {
+    if (coop) CKR(run_coop(h, false, rows, coop));
+    else CKR(run_resident(h, false));
     so->eps = h->sc_host->iter > 0 ? sqrt(std::max(h->sc_host->G, 0.0)) / h->sc_host->bnorm : h->sc_host->eps;
   } else {
-    if (!boxed) {  // the passes work on the contact band
-      launch_box(plan_of<T>(h), h->S, h->sc, h->stream);
-      h->launches += 1;
-    }
     if (!pf.cg_graph[0]) CKR(capture_chunk<T>(h, false, false, &pf.cg_graph[0]));
     if (h->timing && !pf.cg_graph[1]) CKR(capture_chunk<T>(h, false, true, &pf.cg_graph[1]));
     const size_t n = (size_t)h->nx * h->ny;
@@ -1233,9 +1266,7 @@ int detach(bem_ctx* h, double pcrit, double* ndetached) {
   Fields<T> f{};
   f.p = pf.p;
   f.S = h->S;
-  h->sc_host->pcrit = pcrit;
-  CK(cudaMemcpyAsync(&h->sc->pcrit, &pcrit, sizeof(double), cudaMemcpyHostToDevice, h->stream));
-  launch_detach<T>(plan_of<T>(h), f, h->partE, h->sc, h->ew_ngrid, h->stream);
+  launch_detach<T>(plan_of<T>(h), f, pcrit, h->partE, h->sc, h->ew_ngrid, h->stream);
   h->launches += 1;
   CKR(read_scalars(h));
   *ndetached = h->sc_host->n_ol;
@@ -1284,11 +1315,19 @@ int gap64(bem_ctx* h, double d, int band_lo = 0, int band_hi = -1) {
   return BEM_OK;
 }
 
-// Largest |x| over S (use_set) -- via the statistics kernel.
-int max_abs_on_set(bem_ctx* h, const double* x, double* out) {
-  bem_result tmp{};
-  CKR(collect<double>(h, h->io64, x, 1, &tmp));
-  *out = h->stats_host[2];
+// Largest |a| and |b| over S, one launch and one wait.
+int max_abs_on_set(bem_ctx* h, const double* a, const double* b, double* ma, double* mb) {
+  // the accumulators follow the statistics' partials and counter
+  double* acc = h->stats + 8 + 4 * (size_t)h->stats_ngrid + 2;
+  launch_max_abs2(a, b, h->S, (size_t)h->nx * h->ny, reinterpret_cast<unsigned long long*>(acc),
+                  reinterpret_cast<unsigned int*>(acc + 2), h->stats + 4, h->stream);
+  h->launches += 1;
+  CK(cudaMemcpyAsync(h->stats_host + 4, h->stats + 4, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaMemcpyAsync(&h->sc_host->kerr, &h->sc->kerr, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  if (h->sc_host->kerr) return device_error(h);
+  *ma = h->stats_host[4];
+  *mb = h->stats_host[5];
   return BEM_OK;
 }
 
@@ -1308,14 +1347,11 @@ int refine_here(bem_ctx* h, double d, bool adhesive, int sweeps, double tol64, d
     else CKR(gap64(h, d));
     if (!adhesive) { launch_active_set(h->io64, h->f64.g, h->S, n, h->stream); h->launches += 1; }
     double res = 0, scale = 0;
-    CKR(max_abs_on_set(h, h->f64.g, &res));
-    CKR(max_abs_on_set(h, h->f64.c, &scale));
+    CKR(max_abs_on_set(h, h->f64.g, h->f64.c, &res, &scale));
     if (res <= tol64 * scale || !(res > 0)) break;
     // the FP32 correction solves for dp / res so its data are O(1) in FP32
-    launch_to_f32_scaled(h->f64.g, 1.0 / res, h->f32.c, n, h->stream);
+    launch_refine_rhs(h->f64.g, 1.0 / res, h->f32.c, h->f32.p, h->f32.t, n, h->stream);
     h->launches += 1;
-    CK(cudaMemsetAsync(h->f32.p, 0, n * sizeof(float), h->stream));
-    CK(cudaMemsetAsync(h->f32.t, 0, n * sizeof(float), h->stream));
     StepOut cg;
     CKR(run_fixed_cg<float>(h, tol32, 2000, 0.0, &cg));
     so->iterations += cg.iterations;
@@ -1334,17 +1370,13 @@ int refine_here(bem_ctx* h, double d, bool adhesive, int sweeps, double tol64, d
 // are gathered into the sub-context and the pressure is scattered back.
 int refine(bem_ctx* h, double d, bool adhesive, int sweeps, double tol64, double tol32, StepOut* so) {
   if (!h->is_sub) {
-    CKR(init_scalars(h, 0.0, 0, 0.0));  // an empty box to collect into
-    if (adhesive) launch_box(h->plan64, h->S, h->sc, h->stream);
-    else launch_box_overlap(h->plan64, h->h64, d, h->sc, h->stream);
-    h->launches += 1;
-    CKR(read_scalars(h));
-    // rows of the held set (adhesive): its box, in this grid and at the sub-grid's origin
-    const int b0 = h->sc_host->band0, b1 = h->sc_host->band1;
+    // the box of the set: the solve before the refinement has collected it (the held
+    // set, unchanged since, or the overlap set at this depth)
+    const int b0 = h->box[0], b1 = h->box[1];
     bem_ctx* sub = nullptr;
     CKR(pick_sub(h, &sub));
     if (sub) {
-      const int x0 = h->sc_host->col0, y0 = h->sc_host->band0;
+      const int x0 = h->box[2], y0 = h->box[0];
       CKR(ensure_fields<double>(sub));
       CKR(ensure_fields<float>(sub));
       launch_box_gather<double>(h->io64, h->io64, h->S, h->nx, h->ny, x0, y0, sub->io64, sub->io64b, sub->S,
