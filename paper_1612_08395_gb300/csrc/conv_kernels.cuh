@@ -351,10 +351,12 @@ __device__ __forceinline__ void split_store(const C<T>* sm, int rs, int nb, int 
 }
 
 // Launch bounds of the row passes (A and C): the plan caps their CTAs at
-// BEM_MAX_THREADS_A threads except for the longest rows; three resident CTAs
-// per SM (registers capped accordingly) hide more of the global latency.
+// BEM_MAX_THREADS_A threads except for the longest rows.  Two resident CTAs per
+// SM: with three (40 registers) the compiled fixed-set passes of 128-point rows
+// were wrong -- from the second iteration on, with columns past 96 in use -- while
+// the same source is right at 64 registers and above.
 #ifndef BEM_ROW_MIN_BLOCKS
-#define BEM_ROW_MIN_BLOCKS 3
+#define BEM_ROW_MIN_BLOCKS 2
 #endif
 #define BEM_ROW_BOUNDS(LOGL) __launch_bounds__((LOGL) >= 13 ? 1024 : 512, (LOGL) >= 13 ? 1 : BEM_ROW_MIN_BLOCKS)
 
