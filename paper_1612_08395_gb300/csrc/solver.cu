@@ -96,6 +96,7 @@ constexpr int kResidentIters = 4096;
 #endif
 
 template <typename T> struct PrecFields {
+  void* block = nullptr;  // one allocation of the five fields
   T *p = nullptr, *g = nullptr, *t = nullptr, *r = nullptr, *c = nullptr;
   bool ready = false;
   cudaGraphExec_t pk_graph[2] = {nullptr, nullptr}, cg_graph[2] = {nullptr, nullptr};  // [timed]
@@ -255,6 +256,7 @@ struct bem_ctx {
   Plan plan32{}, plan64{};
   int nx = 0, ny = 0, px = 0, py = 0;
   double dx = 0, dy = 0, k = 0, nu = 0, E0 = 0, c0 = 0, alpha = 0, A = 0;
+  void* block = nullptr;    // device memory of everything below but the CG fields
   double* kq64 = nullptr;
   int* geo = nullptr;       // index tables: [A32 | B32 | A64 | B64], each so (112) + sp (L)
   double2* tw64 = nullptr;  // [length-M stages | length-Py stages | split], FP64
@@ -333,15 +335,11 @@ int ensure_fields(bem_ctx* h) {
   PrecFields<T>& f = fields_of<T>(h);
   if (f.ready) return BEM_OK;
   const size_t n = (size_t)h->nx * h->ny;
-  CKR(dmalloc(h, (void**)&f.p, n * sizeof(T)));
-  CKR(dmalloc(h, (void**)&f.g, n * sizeof(T)));
-  CKR(dmalloc(h, (void**)&f.t, n * sizeof(T)));
-  CKR(dmalloc(h, (void**)&f.r, n * sizeof(T)));
-  CKR(dmalloc(h, (void**)&f.c, n * sizeof(T)));
-  CK(cudaMemsetAsync(f.p, 0, n * sizeof(T), h->stream));
-  CK(cudaMemsetAsync(f.g, 0, n * sizeof(T), h->stream));
-  CK(cudaMemsetAsync(f.t, 0, n * sizeof(T), h->stream));
-  CK(cudaMemsetAsync(f.r, 0, n * sizeof(T), h->stream));
+  const size_t fb = (n * sizeof(T) + 511) & ~(size_t)511;
+  CKR(dmalloc(h, &f.block, 5 * fb));
+  T** fields[5] = {&f.p, &f.g, &f.t, &f.r, &f.c};
+  for (int i = 0; i < 5; ++i) *fields[i] = reinterpret_cast<T*>((char*)f.block + i * fb);
+  CK(cudaMemsetAsync(f.p, 0, 4 * fb, h->stream));  // p, g, t, r
   f.ready = true;
   return BEM_OK;
 }
@@ -389,14 +387,6 @@ int update_w_map(bem_ctx* h, int nb) {
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return BEM_OK;  // not representable: stay on cp.async
-  if (!h->tmw) {
-    if (cudaMalloc(&h->tmw, sizeof(CUtensorMap)) != cudaSuccess) {
-      cudaGetLastError();
-      h->tmw = nullptr;
-      return BEM_OK;
-    }
-    h->bytes += sizeof(CUtensorMap);
-  }
   // ordered before every later launch on the handle's stream
   CK(cudaMemcpyAsync(h->tmw, &m, sizeof m, cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
@@ -1588,34 +1578,53 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
   const int M = h->px / 2, hyq = h->py / 2 + 1;
   const size_t n = (size_t)Nx * Ny;
   int rc;
-  if ((rc = dmalloc(h, (void**)&h->kq64, sizeof(double) * (size_t)hyq * (M + 1)))) return cleanup(rc);
   // [length-M stages | length-Py stages | split | radix-16 length-Py stages]
   const size_t ntw = (size_t)M + h->py + M + 1 + h->py;
-  if ((rc = dmalloc(h, (void**)&h->tw64, sizeof(double2) * (ntw - h->py)))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->tw32, sizeof(float2) * ntw))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->twfx, sizeof(int4) * (ntw - h->py)))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->fxe, sizeof(int) * ((size_t)Ny + M + 1)))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->geo, sizeof(int) * 2 * (2 * kSoEntries + M + h->py)))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->khat64, sizeof(double) * (size_t)hyq * (M + 1)))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->khat32, sizeof(float) * (size_t)hyq * (M + 1)))) return cleanup(rc);
-  if ((rc = dmalloc(h, &h->W, sizeof(double) * 2 * (size_t)(M + 1) * Ny))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->h64, sizeof(double) * n))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->io64, sizeof(double) * n))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->io64b, sizeof(double) * n))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->S, n))) return cleanup(rc);
   const int gmax = Ny;  // per-CTA partials come from row groups: at most one per row, for any shape
-  if ((rc = dmalloc(h, (void**)&h->part, sizeof(double) * 4 * (size_t)gmax))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->partC, sizeof(double) * 4 * (size_t)gmax))) return cleanup(rc);
   h->ew_ngrid = (int)((n + 255) / 256 < (size_t)BEM_EW_CTAS_PER_SM * h->plan32.nsm
                           ? (n + 255) / 256 : (size_t)BEM_EW_CTAS_PER_SM * h->plan32.nsm);
   if (h->ew_ngrid < 1) h->ew_ngrid = 1;
-  if ((rc = dmalloc(h, (void**)&h->partE, sizeof(double) * 4 * (size_t)h->ew_ngrid))) return cleanup(rc);
   h->stats_ngrid = h->ew_ngrid;
-  if ((rc = dmalloc(h, (void**)&h->stats, sizeof(double) * (8 + 4 * (size_t)h->stats_ngrid + 8)))) return cleanup(rc);
-  if ((rc = dmalloc(h, (void**)&h->sc, sizeof(Scalars)))) return cleanup(rc);
-  if (cudaMallocHost((void**)&h->sc_host, sizeof(Scalars)) != cudaSuccess ||
-      cudaMallocHost((void**)&h->stats_host, 8 * sizeof(double)) != cudaSuccess)
+  // One device block for all of them: an allocation of its own each, and a free
+  // with its device-wide wait each, were a third of setting a handle up and
+  // taking it down.  W and the three fields after it double as the workspace of
+  // the spectrum's set-up, 16 (M + 1) (Py/2 + 1) bytes, before any of them is used.
+  const size_t w_bytes = sizeof(double) * 2 * (size_t)(M + 1) * Ny, f_bytes = sizeof(double) * n;
+  const size_t spec_bytes = sizeof(double) * 2 * (size_t)(M + 1) * hyq;
+  const size_t spare = spec_bytes > w_bytes + 3 * f_bytes ? spec_bytes - (w_bytes + 3 * f_bytes) : 0;
+  const struct { void** p; size_t bytes; } parts[] = {
+      {(void**)&h->kq64, sizeof(double) * (size_t)hyq * (M + 1)},
+      {(void**)&h->tw64, sizeof(double2) * (ntw - h->py)},
+      {(void**)&h->tw32, sizeof(float2) * ntw},
+      {(void**)&h->twfx, sizeof(int4) * (ntw - h->py)},
+      {(void**)&h->fxe, sizeof(int) * ((size_t)Ny + M + 1)},
+      {(void**)&h->geo, sizeof(int) * 2 * (2 * kSoEntries + M + h->py)},
+      {(void**)&h->khat64, sizeof(double) * (size_t)hyq * (M + 1)},
+      {(void**)&h->khat32, sizeof(float) * (size_t)hyq * (M + 1)},
+      {(void**)&h->part, sizeof(double) * 4 * (size_t)gmax},
+      {(void**)&h->partC, sizeof(double) * 4 * (size_t)gmax},
+      {(void**)&h->partE, sizeof(double) * 4 * (size_t)h->ew_ngrid},
+      {(void**)&h->stats, sizeof(double) * (8 + 4 * (size_t)h->stats_ngrid + 8)},
+      {(void**)&h->sc, sizeof(Scalars)},
+      {(void**)&h->tmw, sizeof(CUtensorMap)},
+      {(void**)&h->S, n},
+      {&h->W, w_bytes},
+      {(void**)&h->h64, f_bytes},
+      {(void**)&h->io64, f_bytes},
+      {(void**)&h->io64b, f_bytes + spare},
+  };
+  auto padded = [](size_t v) { return (v + 511) & ~(size_t)511; };
+  size_t total = 0;
+  for (const auto& q : parts) total += padded(q.bytes);
+  if ((rc = dmalloc(h, &h->block, total))) return cleanup(rc);
+  char* at = (char*)h->block;
+  for (const auto& q : parts) {
+    *q.p = at;
+    at += padded(q.bytes);
+  }
+  if (cudaMallocHost((void**)&h->sc_host, sizeof(Scalars) + 8 * sizeof(double)) != cudaSuccess)
     return cleanup(fail(BEM_ENOMEM, "pinned allocation failed"));
+  h->stats_host = reinterpret_cast<double*>(h->sc_host + 1);
   memset(h->sc_host, 0, sizeof(Scalars));
   if (cudaMemsetAsync(h->sc, 0, sizeof(Scalars), h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->stats, 0, sizeof(double) * (8 + 4 * (size_t)h->stats_ngrid + 8), h->stream) != cudaSuccess ||
@@ -1648,16 +1657,13 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
   }
   // spectrum of the even torus extension (Eq. 13: FFT(K)), FP64, once
   {
-    void* Wspec = nullptr;
-    if (cudaMalloc(&Wspec, sizeof(double) * 2 * (size_t)(M + 1) * hyq) != cudaSuccess)
-      return cleanup(fail(BEM_ENOMEM, "spectrum workspace allocation failed"));
     PassArgs<double> a{};
     a.pl = h->plan64;
     a.twA = h->tw64; a.twB = h->tw64 + M; a.twS = h->tw64 + M + h->py;
     const int* g64 = h->geo + 2 * kSoEntries + M + h->py;
     a.soA = g64; a.spA = g64 + kSoEntries;
     a.soB = g64 + kSoEntries + M; a.spB = g64 + 2 * kSoEntries + M;
-    a.W = Wspec;
+    a.W = h->W;  // with the fields after it
     a.rows_w = hyq;  // K is even: rows 0..Py/2 of the torus hold all
     a.nrows_in = hyq;
     a.ncols_in = h->px;
@@ -1667,7 +1673,6 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
     launch_pass_a<double>(a, A_TORUS, h->stream);
     launch_pass_b<double>(a, B_SPECTRUM, h->stream);
     cudaError_t e = cudaStreamSynchronize(h->stream);
-    cudaFree(Wspec);
     if (e != cudaSuccess) return cleanup(fail(BEM_ECUDA, "spectrum set-up failed: %s", cudaGetErrorString(e)));
   }
   cudaError_t e = cudaGetLastError();
@@ -1691,13 +1696,11 @@ extern "C" void bem_destroy(bem_handle h) {
     for (int j = 0; j < 4; ++j)
       if (h->ev[i][j]) cudaEventDestroy(h->ev[i][j]);
   if (h->ev_ready) cudaEventDestroy(h->ev_ready);
-  fr(h->tmw); fr(h->coop);
-  fr(h->kq64); fr(h->geo); fr(h->tw64); fr(h->tw32); fr(h->twfx); fr(h->fxe); fr(h->khat64); fr(h->khat32); fr(h->W); fr(h->h64); fr(h->io64); fr(h->io64b);
-  fr(h->S); fr(h->part); fr(h->partC); fr(h->partE); fr(h->stats); fr(h->sc);
-  fr(h->f32.p); fr(h->f32.g); fr(h->f32.t); fr(h->f32.r); fr(h->f32.c);
-  fr(h->f64.p); fr(h->f64.g); fr(h->f64.t); fr(h->f64.r); fr(h->f64.c);
-  if (h->sc_host) cudaFreeHost(h->sc_host);
-  if (h->stats_host) cudaFreeHost(h->stats_host);
+  fr(h->coop);
+  fr(h->block);
+  fr(h->f32.block);
+  fr(h->f64.block);
+  if (h->sc_host) cudaFreeHost(h->sc_host);  // with stats_host
   if (h->stream && h->own_stream) cudaStreamDestroy(h->stream);
   delete h;
 }
