@@ -27,7 +27,11 @@
 // the outputs that depend on it (all rows, as an FP64 FFT would) with NaN.
 //
 // Bound by the integer pipes: about 400 instructions per radix-8 butterfly and
-// stage, two thirds of them twiddle products.
+// stage, two thirds of them twiddle products.  Measured (GB300) against FP64
+// butterflies: the transform of a 1501 x 1100 grid 1,616 -> 390 us, of 64 x 64
+// 57 -> 37 us; there is no size at which FP64 butterflies are faster, so the CG
+// and plain modes have no FP64 kernels (the spectrum's set-up, whose result is
+// kept in FP64, does).
 #pragma once
 #include "conv_kernels.cuh"
 
@@ -245,11 +249,15 @@ __device__ __forceinline__ ll dfix(double x, int emax) {
 }
 
 // Threads per CTA of these kernels are capped as the plan caps them; registers
-// for eight complex integers and a product in flight.
-#ifndef BEM_FX_MIN_BLOCKS
-#define BEM_FX_MIN_BLOCKS 1
-#endif
-#define BEM_FX_BOUNDS(LOGL) __launch_bounds__((LOGL) >= 13 ? 1024 : 512, (LOGL) >= 13 ? 1 : BEM_FX_MIN_BLOCKS)
+// for eight complex integers and a product in flight (128).  Row passes of 2048
+// and 4096 points, whose CTAs have 512 threads, fit an SM twice at 64 registers:
+// they spill about as much as they hold, but one CTA's barriers, loads and
+// FP64 conversions are covered by the other's (transform of 2048 x 2048 555 -> 480
+// us, 4096 x 1000 529 -> 463, 1501 x 1100 423 -> 390).  Shorter rows, of which
+// several CTAs fit anyway, and the column pass only lose by the spills (200 x 251
+// 41 -> 47 us; the 4096-point column pass 3% either way by grid).
+#define BEM_FX_BOUNDS(LOGL) __launch_bounds__((LOGL) >= 13 ? 1024 : 512, 1)
+#define BEM_FX_ROW_BOUNDS(LOGL) __launch_bounds__((LOGL) >= 13 ? 1024 : 512, (LOGL) == 11 || (LOGL) == 12 ? 2 : 1)
 constexpr int kFxStages = 8;  // shared magnitude words
 
 // ---------------------------------------------------------------------------
@@ -724,9 +732,9 @@ __device__ __forceinline__ void fx_pass_c_body(const PassArgs<double>& a) {
 }
 
 template <int MODE, int LOGL>
-__global__ void BEM_FX_BOUNDS(LOGL) k_fx_a(PassArgs<double> a) { fx_pass_a_body<MODE, LOGL>(a); }
+__global__ void BEM_FX_ROW_BOUNDS(LOGL) k_fx_a(PassArgs<double> a) { fx_pass_a_body<MODE, LOGL>(a); }
 template <int MODE, int LOGL>
-__global__ void BEM_FX_BOUNDS(LOGL) k_fx_a_mi(const PassArgs<double>* __restrict__ arr) {
+__global__ void BEM_FX_ROW_BOUNDS(LOGL) k_fx_a_mi(const PassArgs<double>* __restrict__ arr) {
   fx_pass_a_body<MODE, LOGL>(arr[blockIdx.y]);
 }
 template <int LOGL>
@@ -736,9 +744,9 @@ __global__ void BEM_FX_BOUNDS(LOGL) k_fx_b_mi(const PassArgs<double>* __restrict
   fx_pass_b_body<LOGL>(arr[blockIdx.y]);
 }
 template <int MODE, int LOGL>
-__global__ void BEM_FX_BOUNDS(LOGL) k_fx_c(PassArgs<double> a) { fx_pass_c_body<MODE, LOGL>(a); }
+__global__ void BEM_FX_ROW_BOUNDS(LOGL) k_fx_c(PassArgs<double> a) { fx_pass_c_body<MODE, LOGL>(a); }
 template <int MODE, int LOGL>
-__global__ void BEM_FX_BOUNDS(LOGL) k_fx_c_mi(const PassArgs<double>* __restrict__ arr) {
+__global__ void BEM_FX_ROW_BOUNDS(LOGL) k_fx_c_mi(const PassArgs<double>* __restrict__ arr) {
   fx_pass_c_body<MODE, LOGL>(arr[blockIdx.y]);
 }
 
