@@ -180,11 +180,13 @@ int bem_contact_set(bem_handle h, unsigned char *S_out);
  *   time on one device share their CG loops: when a job's solve reaches its
  *   loop it joins the loops waiting at that moment (all jobs in flight, or
  *   those that arrived within 200 us), and the loops of one size class (grid,
- *   torus, launch shapes, precision and loop kind) run as one while-loop graph
- *   in which every transform pass is a single launch over all of them, each
- *   instance stopping at its own convergence (its CTAs return at once when it
- *   is done).  *launches = such graphs launched, *loops = the solves' loops they
- *   carried.  Results are bitwise those of the job run alone.
+ *   torus, launch shapes, precision and loop kind) run as one launch: FP32 loops
+ *   on a torus of at most 512 x 512 as one launch with a thread-block cluster
+ *   per solve, the others as one while-loop graph in which every transform pass
+ *   is a single launch over all of them, each instance stopping at its own
+ *   convergence.  *launches = such launches, *loops = the solves' loops they
+ *   carried.  Counts and statuses are those of the job run alone, forces and
+ *   pressures agree with it to rounding.
  *   BEM_BATCH_LOOPS=0 in the environment makes every job run its own loops.
  * bem_server_footprint: the bytes admission reserves for a job on an Nx x Ny
  *   grid (a handle after FP32 and FP64 solves plus its set-up workspace);
@@ -280,9 +282,11 @@ int bem_get_info(bem_handle h, bem_info *info);
 int bem_set_material(bem_handle h, double nu, double E0, double c0);
 
 /* Accumulated device time of the transform passes recorded under
- * BEM_FLAG_TIME_PASSES: ms[0..2] = total milliseconds of passes A (row FFT and
- * CG prologue), B (column FFT, spectrum multiply, inverse column FFT) and C
- * (inverse row FFT and CG epilogue), count[0] = number of timed iterations,
+ * BEM_FLAG_TIME_PASSES (under it every CG loop runs as separate passes, also
+ * those that one cooperative or cluster launch carries without it): ms[0..2] =
+ * total milliseconds of passes A (row FFT and CG prologue), B (column FFT,
+ * spectrum multiply, inverse column FFT) and C (inverse row FFT and CG
+ * epilogue), count[0] = number of timed iterations,
  * count[1] = of those, iterations of the fixed-set loop.  reset != 0 clears the
  * totals after reading.  Events are timed on the handle's stream, the stream
  * the passes run on. */

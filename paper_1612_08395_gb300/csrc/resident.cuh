@@ -17,7 +17,9 @@
 // The arithmetic is that of the passes (FftC stages, the same prologues and
 // epilogues); only the order of the partial sums differs.
 //
-// Bound by latency: about 12 barriers and 10 FFT stages per transform.
+// Bound by latency: about 12 barriers and 10 FFT stages per transform.  Measured
+// (GB300, per Polonsky-Keer iteration, two transforms): 32 x 32 10 us, 128 x 128
+// 15, 256 x 256 30, as passes 29, 34 and 36; a fixed-set iteration takes half.
 #pragma once
 #include "conv_kernels.cuh"
 

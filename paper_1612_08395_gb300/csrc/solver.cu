@@ -1,6 +1,7 @@
 // Host orchestration of the solver: handle set-up (influence table and
-// spectrum), the constrained and fixed-set conjugate-gradient loops as chunks
-// of captured CUDA graphs, the adhesive detach loop, the FP64 refinement
+// spectrum), the constrained and fixed-set conjugate-gradient loops (one launch
+// where the grid allows it, else chunks of captured CUDA graphs), the adhesive
+// detach loop, the FP64 refinement
 // sweep, load-unload sweeps, and the C ABI of include/bem.h.
 #include <math.h>
 #include <stddef.h>
@@ -911,8 +912,9 @@ int run_loop(bem_ctx* h, cudaGraphExec_t g, cudaGraphExec_t g_timed, int max_ite
 }
 
 // Whether this context's CG loops in precision es run inside one cluster: FP32,
-// grids of at most 256 x 256 (the cluster's sixteen SMs hold and transform them
-// faster than the chip-wide passes start and end; above that the passes win).
+// tori of at most 512 x 512, which the cluster's sixteen SMs hold and transform
+// faster than the chip-wide passes start and end (per Polonsky-Keer iteration
+// 10 to 30 us against 29 to 36; larger ones do not fit their shared memory).
 // Pass timing needs the separate passes.
 bool resident_applies(const bem_ctx* h, int es) {
   return es == 4 && h->px <= 512 && h->py <= 512 && !h->timing && g_resident[h->device];
@@ -960,14 +962,19 @@ struct CoopHold {
 // CTAs of the cooperative launch over the chip (coop.cuh) that this context's CG
 // loops in precision es run as, 0: not.  FP32, row transforms of 256 to 1024
 // points and columns of 512 to 2048, the sizes at which the passes' starts and
-// tails cost as much as their work.  Pass timing needs the separate passes, and
-// the server's loops share launches instead.
+// tails cost as much as their work: a fixed-set iteration takes 11 us against 15 in
+// a cluster at 256 x 256, 14 against 21 as passes at 512 x 512, 29 against 33 at
+// 1024 x 1024.  Below, a cluster's barriers are cheaper than the grid's (128 x 128:
+// 7.4 us in a cluster); above, an SM's share of the rows does not fit its shared
+// memory.  Pass timing needs the separate passes, and the server's loops share
+// launches instead.
 int coop_applies(const bem_ctx* h, int es) {
   if (es != 4 || h->timing || h->batcher || !g_coop[h->device] || (h->ny & 1)) return 0;
   return coop_ctas(ilog2(h->px / 2), ilog2(h->py), h->plan32.nsm);
 }
 
-// The whole CG loop over `rows` grid rows as cooperative launches of nb CTAs.
+// The whole CG loop over `rows` grid rows as cooperative launches of nb CTAs, each
+// of at most kResidentIters iterations.
 int run_coop(bem_ctx* h, bool pk, int rows, int nb) {
   if (!h->coop) CKR(dmalloc(h, &h->coop, coop_shared_bytes()));
   CoopHold hold;
