@@ -8,10 +8,10 @@
 // per CTA (block floating point):
 //   - pass A finds the largest exponent of its row group's inputs and converts
 //     them to integers below 2^57 (the fields stay FP64 in memory);
-//   - every stage records the highest magnitude bit it wrote (an OR over the
+//   - every stage records the largest magnitude it wrote (a maximum over the
 //     CTA, published by the barrier the stage needs anyway) and the next stage
-//     shifts its inputs right, rounding, just far enough that a radix-8
-//     butterfly stays below 2^61.  A value therefore always carries about 57
+//     shifts its inputs right, rounding, just far enough that what a radix-8
+//     butterfly multiplies stays below 2^61.  A value therefore always carries 57
 //     bits relative to the largest one of its transform, against FP64's 53, and
 //     additions are exact;
 //   - twiddle factors have 60 bits (two 30-bit limbs); a product is three
@@ -21,15 +21,15 @@
 //     column's rows, and pass C its row group's columns, to the largest.
 //   - the spectrum multiply keeps the spectrum's own exponents and renormalises
 //     by the largest product, so steep spectra lose nothing.
-// Against 64-bit references the transform's error is no larger than the FP64
-// butterflies' (about 1/2 to 1 times it; the input and output conversions are
-// what remains).  NaN and infinity in an input mark the exponent, which poisons
+// Against long-double sums the transform's error is 0.3 to 0.7 times the FP64
+// butterflies' for k >= 0 and 0.5 to 1.2 times for k < 0 (contact pressures, 64 to
+// 2048 a side).  NaN and infinity in an input mark the exponent, which poisons
 // the outputs that depend on it (all rows, as an FP64 FFT would) with NaN.
 //
 // Bound by the integer pipes: about 400 instructions per radix-8 butterfly and
 // stage, two thirds of them twiddle products.  Measured (GB300) against FP64
-// butterflies: the transform of a 1501 x 1100 grid 1,616 -> 390 us, of 64 x 64
-// 57 -> 37 us; there is no size at which FP64 butterflies are faster, so the CG
+// butterflies: the transform of a 1501 x 1100 grid 1,617 -> 400 us, of 64 x 64
+// 57 -> 38 us; there is no size at which FP64 butterflies are faster, so the CG
 // and plain modes have no FP64 kernels (the spectrum's set-up, whose result is
 // kept in FP64, does).
 #pragma once
@@ -40,7 +40,14 @@ namespace bem {
 using ll = long long;
 using fx2 = longlong2;  // a complex value: real and imaginary 64-bit integers
 
-constexpr int kFxBits = 57;             // component bits before a radix-8 butterfly
+// Component bits where values are brought to a common exponent: before a radix-8
+// butterfly, before a leading stage half of whose inputs are zero, and in W and
+// before pass C's split, which only adds pairs.
+constexpr int kFxBits = 57, kFxBitsHalf = 58, kFxBitsW = 59;
+// High words of components before a radix-8 stage stay below this (2^57.69): the
+// values it multiplies are then below (4 + 4 sqrt 2) 2^57.69 < 2^61 - 2^34, those
+// it stores below 2^61.3.  (A limit of 57 whole bits left up to 0.7 bit unused.)
+constexpr unsigned kFxLimit = 54000000u;
 constexpr int kFxPoison = 1 << 20;      // exponent of a group that met NaN or infinity
 constexpr int kFxZero = -(1 << 20);     // exponent of a group of zeros
 
@@ -103,18 +110,21 @@ __device__ __forceinline__ unsigned fmag(ll v) {
   const int hi = (int)(v >> 32);
   return (unsigned)(hi ^ (hi >> 31));
 }
-__device__ __forceinline__ unsigned fmag(fx2 v) { return fmag(v.x) | fmag(v.y); }
+__device__ __forceinline__ unsigned fmag(fx2 v) { return max(fmag(v.x), fmag(v.y)); }
 // Components are below 2^fbits(mag)
 __device__ __forceinline__ int fbits(unsigned mag) { return 64 - __clz((int)mag); }
-// Shift that brings components below 2^B
-template <int B>
-__device__ __forceinline__ int fshift(unsigned mag) { return max(0, fbits(mag) - B); }
+// Shift that brings high words below kFxLimit
+__device__ __forceinline__ int fshift(unsigned mag) {
+  if (mag < kFxLimit) return 0;
+  const int s = 6 - __clz((int)mag);  // mag >> s has 26 bits
+  return (mag >> s) < kFxLimit ? s : s + 1;
+}
 
-// OR / max over the CTA into a shared word, one atomic per warp; published by
-// the caller's next barrier.
-__device__ __forceinline__ void cta_or(unsigned* w, unsigned v) {
-  v = __reduce_or_sync(0xffffffffu, v);
-  if ((threadIdx.x & 31) == 0 && v) atomicOr(w, v);
+// Maximum over the CTA into a shared word, one atomic per warp; published by the
+// caller's next barrier.
+__device__ __forceinline__ void cta_max(unsigned* w, unsigned v) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0 && v) atomicMax(w, v);
 }
 __device__ __forceinline__ void cta_max(int* w, int v) {
   v = __reduce_max_sync(0xffffffffu, v);
@@ -228,7 +238,7 @@ struct FxFft {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       buf[sb ^ F::sw(q << ls)] = v[q];
-      m |= fmag(v[q]);
+      m = max(m, fmag(v[q]));
     }
     return m;
   }
@@ -239,12 +249,12 @@ __device__ __forceinline__ int dexp(double x) {
   const int hi = __double2hiint(x) & 0x7fffffff;
   return (hi | __double2loint(x)) == 0 ? 0 : max(hi >> 20, 1);
 }
-// x as an integer below 2^kFxBits in magnitude where the largest biased
-// exponent around is emax: x = result * 2^(emax - 1022 - kFxBits).
+// x as an integer below 2^kFxBitsHalf in magnitude where the largest biased
+// exponent around is emax: x = result * 2^(emax - 1022 - kFxBitsHalf).
 __device__ __forceinline__ ll dfix(double x, int emax) {
   const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
   const ll m = ((ll)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32) | (unsigned)__double2loint(x);
-  const ll q = falign(m, (emax - max(e, 1)) - (kFxBits - 53));
+  const ll q = falign(m, (emax - max(e, 1)) - (kFxBitsHalf - 53));
   return hi < 0 ? -q : q;
 }
 
@@ -344,26 +354,26 @@ __device__ __forceinline__ void fx_pass_a_body(const PassArgs<double>& a) {
     if (!F::first_half(e)) continue;
     if (emax > 0 && emax < 0x7ff) v[e] = fmk(dfix(x[e][0], emax), dfix(x[e][1], emax));
   }
-  int ex = emax == 0 ? kFxZero : emax == 0x7ff ? kFxPoison : emax - 1022 - kFxBits;
+  int ex = emax == 0 ? kFxZero : emax == 0x7ff ? kFxPoison : emax - 1022 - kFxBitsHalf;
   X::stage0_fwd(v, t, tw);
   unsigned m = 0;
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     buf[F::ix0(t, e)] = v[e];
-    m |= fmag(v[e]);
+    m = max(m, fmag(v[e]));
   }
-  cta_or(&mag[0], m);
+  cta_max(&mag[0], m);
   __syncthreads();
   int st = 0;
 #pragma unroll
   for (int ls = F::LS_TOP; ls >= 0; ls -= 3) {
-    const int s = fshift<kFxBits>(mag[st]);
+    const int s = fshift(mag[st]);
     ex += s;
     m = X::template stage<true>(buf, t, ls, tw, s);
-    cta_or(&mag[++st], m);
+    cta_max(&mag[++st], m);
     __syncthreads();
   }
-  const int s = fshift<kFxBits>(mag[st]);
+  const int s = max(0, fbits(mag[st]) - kFxBitsW);
   ex += s;
   if (MODE == A_PK_P) block_partials<double, 3>(acc, a.partA + 4 * blockIdx.x, red);
   // X[k] = (z[k] + conj z[M-k])/2 + w_k (z[k] - conj z[M-k])/(2i), twice that here:
@@ -452,7 +462,7 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
   __syncthreads();
   cta_max(&emx[0], em);
   __syncthreads();
-  int ex = emx[0] - kFxBits;
+  int ex = emx[0] - kFxBitsHalf;
   const bool poison = emx[0] >= kFxPoison / 2, zero = emx[0] <= kFxZero / 2;
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
@@ -466,17 +476,17 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     buf[F::ix0(t, e)] = v[e];
-    m |= fmag(v[e]);
+    m = max(m, fmag(v[e]));
   }
-  cta_or(&mag[0], m);
+  cta_max(&mag[0], m);
   __syncthreads();
   int st = 0;
 #pragma unroll
   for (int ls = F::LS_TOP; ls >= 3; ls -= 3) {
-    const int s = fshift<kFxBits>(mag[st]);
+    const int s = fshift(mag[st]);
     ex += s;
     m = X::template stage<true>(buf, t, ls, tw, s);
-    cta_or(&mag[++st], m);
+    cta_max(&mag[++st], m);
     __syncthreads();
   }
   // stride-1 stage, spectrum multiply, first inverse stage in registers: thread
@@ -492,7 +502,7 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
       const int kk = ky <= (L >> 1) ? ky : L - ky;
       kf[q] = act ? __ldg(kc + kk) : 0.0;
     }
-    const int s = fshift<kFxBits>(mag[st]);
+    const int s = fshift(mag[st]);
     ex += s;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -527,20 +537,20 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       buf[sp0 ^ r] = v[r];
-      m |= fmag(v[r]);
+      m = max(m, fmag(v[r]));
     }
-    cta_or(&mag[++st], m);
+    cta_max(&mag[++st], m);
   }
   __syncthreads();
 #pragma unroll
   for (int ls = 3; ls <= F::LS_TOP; ls += 3) {
-    const int s = fshift<kFxBits>(mag[st]);
+    const int s = fshift(mag[st]);
     ex += s;
     m = X::template stage<false>(buf, t, ls, tw, s);
-    cta_or(&mag[++st], m);
+    cta_max(&mag[++st], m);
     __syncthreads();
   }
-  const int s = fshift<kFxBits>(mag[st]);
+  const int s = fshift(mag[st]);
   ex += s;
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
@@ -639,7 +649,7 @@ __device__ __forceinline__ void fx_pass_c_body(const PassArgs<double>& a) {
     __syncthreads();
     const int e0 = emx;
     const bool poison = e0 >= kFxPoison / 2, zero = e0 <= kFxZero / 2;
-    int ex = e0 - kFxBits;
+    int ex = e0 - kFxBitsW;
     unsigned m = 0;
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
@@ -656,23 +666,23 @@ __device__ __forceinline__ void fx_pass_c_body(const PassArgs<double>& a) {
       const fx2 O = fcmul<true>(fmk(p.x - q.x, p.y + q.y), __ldg(a.fxS + k));
       const fx2 zk = fmk(E.x - O.y, E.y + O.x);
       z[__ldg(sp + k)] = zk;
-      m |= fmag(zk);
+      m = max(m, fmag(zk));
       if (k != 0 && k != M - k) {
         const fx2 zm = fmk(E.x + O.y, O.x - E.y);  // conj(E - i O)
         z[__ldg(sp + M - k)] = zm;
-        m |= fmag(zm);
+        m = max(m, fmag(zm));
       }
     }
-    cta_or(&mag[0], m);
+    cta_max(&mag[0], m);
     __syncthreads();
     fx2* buf = sm + b * rs;
     int st = 0;
 #pragma unroll
     for (int ls = 0; ls <= F::LS_TOP; ls += 3) {
-      const int s = fshift<kFxBits>(mag[st]);
+      const int s = fshift(mag[st]);
       ex += s;
       m = X::template stage<false>(buf, t, ls, tw, s);
-      cta_or(&mag[++st], m);
+      cta_max(&mag[++st], m);
       __syncthreads();
     }
     const int row = row0 + b;
@@ -690,7 +700,7 @@ __device__ __forceinline__ void fx_pass_c_body(const PassArgs<double>& a) {
           if (act && n < half && 2 * n + h < nx) epi_gather<double, MODE>(a, rowoff + 2 * n + h, ein[e][h]);
       }
     }
-    const int s = fshift<kFxBits>(mag[st]);
+    const int s = fshift(mag[st]);
     ex += s;
     fx2 v[8];
 #pragma unroll
