@@ -22,7 +22,7 @@
 //   - the spectrum multiply keeps the spectrum's own exponents and renormalises
 //     by the largest product, so steep spectra lose nothing.
 // Against long-double sums the transform's error is 0.3 to 0.7 times the FP64
-// butterflies' for k >= 0 and 0.5 to 1.2 times for k < 0 (contact pressures, 64 to
+// butterflies' for k >= 0 and 0.5 to 1.3 times for k < 0 (contact pressures, 64 to
 // 2048 a side).  NaN and infinity in an input mark the exponent, which poisons
 // the outputs that depend on it (all rows, as an FP64 FFT would) with NaN.
 //
