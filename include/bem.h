@@ -39,10 +39,12 @@ extern "C" {
                              BEM_DEBUG_CHECKS) a kernel's bounds check failed  */
 #define BEM_ECANCELED (-7) /* a server job was cancelled before it started       */
 
-/* Arithmetic of the transform and the fields.  BEM_PREC_FP64: everything in
- * FP64 (the plain path).  BEM_PREC_FP32: FFT passes and fields in FP32, CG
- * scalars and all reductions in FP64.  BEM_PREC_FP32_REFINE: FP32 solve, then
- * FP64-residual refinement sweeps on the final contact set. */
+/* Arithmetic of the transform and the fields.  BEM_PREC_FP64 (the plain path):
+ * fields, CG scalars and sums in FP64; inside a transform 64-bit integers with
+ * common exponents, whose rounding errors are below those of FP64 butterflies.
+ * BEM_PREC_FP32: FFT passes and fields in FP32, CG scalars and all reductions in
+ * FP64.  BEM_PREC_FP32_REFINE: FP32 solve, then FP64-residual refinement sweeps
+ * on the final contact set. */
 #define BEM_PREC_FP64 0
 #define BEM_PREC_FP32 1
 #define BEM_PREC_FP32_REFINE 2

@@ -139,7 +139,7 @@ struct PassArgs {
   const void* twB;      // stage twiddle tables, length Py (C<T>)
   const void* twB16;    // stage twiddle tables of the radix-16 column pass, length Py (C<T>)
   const void* twS;      // exp(-i pi k / M), k = 0..M (C<T>): real-FFT split
-  const int4* fxA;      // FP64 path: the tables twA, twB and twS as 30-bit limbs (fx_kernels.cuh)
+  const int4* fxA;      // FP64 path: the tables twA, twB and twS as fixed-point limbs (fx_kernels.cuh)
   const int4* fxB;
   const int4* fxS;
   int* fx_ea;           // FP64 path: exponents of W's row groups (pass A) ...

@@ -7,23 +7,26 @@
 // keep every value of a transform as a 64-bit integer with one common exponent
 // per CTA (block floating point):
 //   - pass A finds the largest exponent of its row group's inputs and converts
-//     them to integers below 2^57 (the fields stay FP64 in memory);
+//     them to integers below 2^59 (the fields stay FP64 in memory);
 //   - every stage records the largest magnitude it wrote (a maximum over the
 //     CTA, published by the barrier the stage needs anyway) and the next stage
-//     shifts its inputs right, rounding, just far enough that what a radix-8
-//     butterfly multiplies stays below 2^61.  A value therefore always carries 57
-//     bits relative to the largest one of its transform, against FP64's 53, and
-//     additions are exact;
-//   - twiddle factors have 60 bits (two 30-bit limbs); a product is three
+//     shifts its inputs right, rounding, just far enough that its products stay
+//     within their factors' range.  A value is therefore rounded 58 bits or more
+//     below the largest one of its CTA's rows or columns (which the other passes
+//     add up with it anyway), against FP64's 53 below itself, and additions are
+//     exact;
+//   - twiddle factors have 62 bits (two limbs); a product is three
 //     32 x 32 -> 64 bit multiply-adds per real factor;
 //   - W holds the integers; one exponent per row group (pass A) or per CTA of
 //     columns (pass B) goes to a small array beside it.  Pass B aligns its
 //     column's rows, and pass C its row group's columns, to the largest.
 //   - the spectrum multiply keeps the spectrum's own exponents and renormalises
 //     by the largest product, so steep spectra lose nothing.
-// Against long-double sums the transform's error is 0.3 to 0.7 times the FP64
-// butterflies' for k >= 0 and 0.5 to 1.3 times for k < 0 (contact pressures, 64 to
-// 2048 a side).  NaN and infinity in an input mark the exponent, which poisons
+// Against extended-precision transforms the error is 0.3 to 0.6 times the FP64
+// butterflies' for k >= 0 and 0.4 to 0.8 times for k < 0 (contact pressures, 64 to
+// 2048 a side; 1.7e-16 against 2.9e-16 of the field at 2048 x 2048, k = -0.5).  With
+// products of factors below 2^61 and one bit less everywhere (two before inverse
+// stages), at the same speed, it was up to 1.3 times theirs for k < 0.  NaN and infinity in an input mark the exponent, which poisons
 // the outputs that depend on it (all rows, as an FP64 FFT would) with NaN.
 //
 // Bound by the integer pipes: about 400 instructions per radix-8 butterfly and
@@ -40,14 +43,18 @@ namespace bem {
 using ll = long long;
 using fx2 = longlong2;  // a complex value: real and imaginary 64-bit integers
 
-// Component bits where values are brought to a common exponent: before a radix-8
-// butterfly, before a leading stage half of whose inputs are zero, and in W and
-// before pass C's split, which only adds pairs.
-constexpr int kFxBits = 57, kFxBitsHalf = 58, kFxBitsW = 59;
-// High words of components before a radix-8 stage stay below this (2^57.69): the
-// values it multiplies are then below (4 + 4 sqrt 2) 2^57.69 < 2^61 - 2^34, those
-// it stores below 2^61.3.  (A limit of 57 whole bits left up to 0.7 bit unused.)
-constexpr unsigned kFxLimit = 54000000u;
+// Products take factors below 2^62 - 2^30 (fsplit).  Components may hold
+//   before a forward stage (butterfly, then twiddles)   110e6 2^32 = 2^58.71: the
+//     butterfly's values are below (4 + 4 sqrt 2) of that, 2^62 - 2^55; stored 2^62.3
+//   before an inverse stage (twiddles, then butterfly)  2^59 - 2^32: its factors
+//     1/sqrt 2 meet 8 of that, 2^62 - 2^35; stored below 8 sqrt 2 2^59 = 2^62.5
+//   before a leading stage half of whose inputs are zero  2^59: (2 + 2 sqrt 2) of it
+//   in W, and before pass C's split (sums of two, one of them multiplied)  2^60
+//   before the inverse stage after the spectrum            2^58 (whole bits, rounded up)
+// and every bit counts: a value is rounded at its CTA's common exponent, which on a
+// steep spectrum is far above most bins.
+constexpr int kFxBitsProd = 58, kFxBitsHalf = 59, kFxBitsW = 60;
+constexpr unsigned kFxLimitFwd = 110000000u, kFxLimitInv = (1u << 27) - 1;  // high words
 constexpr int kFxPoison = 1 << 20;      // exponent of a group that met NaN or infinity
 constexpr int kFxZero = -(1 << 20);     // exponent of a group of zeros
 
@@ -66,21 +73,24 @@ __device__ __forceinline__ ll madw(int a, int b, ll c) {
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
   return r;
 }
-// v = h 2^30 + l with l in [-2^29, 2^29), |v| < 2^61
+// v = h 2^31 + l with l in [-2^30, 2^30), |v| < 2^62 - 2^30
 __device__ __forceinline__ void fsplit(ll v, int& h, int& l) {
   const int lo = (int)v, hi = (int)(v >> 32);
-  l = (lo << 2) >> 2;
-  h = (int)__funnelshift_l((unsigned)lo, (unsigned)hi, 2) + ((lo >> 29) & 1);
+  l = (lo << 1) >> 1;
+  h = (int)__funnelshift_l((unsigned)lo, (unsigned)hi, 1) + ((lo >> 30) & 1);
 }
-constexpr ll kFxHalf = 1ll << 29;
-// v w, w = (wh 2^30 + wl) / 2^60 with |w| <= 1 (the dropped low product is below one unit)
+constexpr ll kFxHalf = 1ll << 30;
+// v w, w = (wh 2^31 + wl) / 2^62 with |w| <= 1 (the dropped low product is below one unit)
 __device__ __forceinline__ ll frmul(ll v, int wh, int wl) {
   int h, l;
   fsplit(v, h, l);
   const ll mid = madw(l, wh, madw(h, wl, kFxHalf));
-  return madw(h, wh, mid >> 30);
+  return madw(h, wh, mid >> 31);
 }
-// Complex product with w (limbs {re h, re l, im h, im l}), or with conj w.
+// Complex product with w (limbs {re h, re l, im h, im l}), or with conj w.  The four
+// middle products stay below 2^63: a low limb is below 2^30 but where its component
+// is within 2^-31 of 1 (2^31 then), and a butterfly's value with one component near
+// 2^62 has the other below 0.61 2^62.
 template <bool CONJ>
 __device__ __forceinline__ fx2 fcmul(fx2 v, int4 w) {
   int xh, xl, yh, yl;
@@ -90,7 +100,7 @@ __device__ __forceinline__ fx2 fcmul(fx2 v, int4 w) {
   const int nh = CONJ ? w.z : -w.z, nl = CONJ ? w.w : -w.w;  // and their negatives
   const ll mr = madw(yl, nh, madw(yh, nl, madw(xl, w.x, madw(xh, w.y, kFxHalf))));
   const ll mi = madw(yl, w.x, madw(yh, w.y, madw(xl, ph, madw(xh, pl, kFxHalf))));
-  return fmk(madw(yh, nh, madw(xh, w.x, mr >> 30)), madw(yh, w.x, madw(xh, ph, mi >> 30)));
+  return fmk(madw(yh, nh, madw(xh, w.x, mr >> 31)), madw(yh, w.x, madw(xh, ph, mi >> 31)));
 }
 // Right shift, rounding to nearest even, s >= 0 (0 for s > 62).  The shifts are
 // a few bits, so ties are common, and a tie that always rounds up would bias
@@ -113,11 +123,12 @@ __device__ __forceinline__ unsigned fmag(ll v) {
 __device__ __forceinline__ unsigned fmag(fx2 v) { return max(fmag(v.x), fmag(v.y)); }
 // Components are below 2^fbits(mag)
 __device__ __forceinline__ int fbits(unsigned mag) { return 64 - __clz((int)mag); }
-// Shift that brings high words below kFxLimit
+// Shift that brings high words below LIMIT
+template <unsigned LIMIT>
 __device__ __forceinline__ int fshift(unsigned mag) {
-  if (mag < kFxLimit) return 0;
-  const int s = 6 - __clz((int)mag);  // mag >> s has 26 bits
-  return (mag >> s) < kFxLimit ? s : s + 1;
+  if (mag < LIMIT) return 0;
+  const int s = 5 - __clz((int)mag);  // mag >> s has 27 bits, as LIMIT
+  return (mag >> s) < LIMIT ? s : s + 1;
 }
 
 // Maximum over the CTA into a shared word, one atomic per warp; published by the
@@ -136,17 +147,16 @@ template <int S> __device__ __forceinline__ void fdft4(fx2& v0, fx2& v1, fx2& v2
   v0 = fadd(a0, a2); v2 = fsub(a0, a2);
   v1 = fadd_si<S>(a1, d); v3 = fsub_si<S>(a1, d);
 }
-constexpr int kR2h = 759250125, kR2l = -6429112;  // 2^60 / sqrt 2 = kR2h 2^30 + kR2l, rounded
+constexpr int kR2h = 1518500250, kR2l = -25716447;  // 2^62 / sqrt 2 = kR2h 2^31 + kR2l, rounded
+__device__ __forceinline__ ll frmul_r2(ll v) { return frmul(v, kR2h, kR2l); }
 template <int S> __device__ __forceinline__ void fdft8(fx2* v) {
   fx2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
   fx2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
   fdft4<S>(e0, e1, e2, e3);
   fdft4<S>(o0, o1, o2, o3);
   // w8 o1 = r (o1.x - S o1.y, o1.y + S o1.x); w8^3 o3 = -r (o3.x + S o3.y, o3.y - S o3.x)
-  const fx2 u1 = fmk(frmul(S > 0 ? o1.x - o1.y : o1.x + o1.y, kR2h, kR2l),
-                     frmul(S > 0 ? o1.y + o1.x : o1.y - o1.x, kR2h, kR2l));
-  const fx2 u3 = fmk(frmul(S > 0 ? o3.x + o3.y : o3.x - o3.y, kR2h, kR2l),
-                     frmul(S > 0 ? o3.y - o3.x : o3.y + o3.x, kR2h, kR2l));
+  const fx2 u1 = fmk(frmul_r2(S > 0 ? o1.x - o1.y : o1.x + o1.y), frmul_r2(S > 0 ? o1.y + o1.x : o1.y - o1.x));
+  const fx2 u3 = fmk(frmul_r2(S > 0 ? o3.x + o3.y : o3.x - o3.y), frmul_r2(S > 0 ? o3.y - o3.x : o3.y + o3.x));
   v[0] = fadd(e0, o0); v[4] = fsub(e0, o0);
   v[1] = fadd(e1, u1); v[5] = fsub(e1, u1);
   v[2] = fadd_si<S>(e2, o2); v[6] = fsub_si<S>(e2, o2);
@@ -367,7 +377,7 @@ __device__ __forceinline__ void fx_pass_a_body(const PassArgs<double>& a) {
   int st = 0;
 #pragma unroll
   for (int ls = F::LS_TOP; ls >= 0; ls -= 3) {
-    const int s = fshift(mag[st]);
+    const int s = fshift<kFxLimitFwd>(mag[st]);
     ex += s;
     m = X::template stage<true>(buf, t, ls, tw, s);
     cta_max(&mag[++st], m);
@@ -483,7 +493,7 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
   int st = 0;
 #pragma unroll
   for (int ls = F::LS_TOP; ls >= 3; ls -= 3) {
-    const int s = fshift(mag[st]);
+    const int s = fshift<kFxLimitFwd>(mag[st]);
     ex += s;
     m = X::template stage<true>(buf, t, ls, tw, s);
     cta_max(&mag[++st], m);
@@ -502,7 +512,7 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
       const int kk = ky <= (L >> 1) ? ky : L - ky;
       kf[q] = act ? __ldg(kc + kk) : 0.0;
     }
-    const int s = fshift(mag[st]);
+    const int s = fshift<kFxLimitFwd>(mag[st]);
     ex += s;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -513,10 +523,10 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
     em = kFxZero;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      // kf = +- (h 2^30 + l) 2^(ek - 60), h 2^30 + l in [2^59, 2^60)
+      // kf = +- (h 2^31 + l) 2^(ek - 62), h 2^31 + l in [2^61, 2^62)
       const int hi = __double2hiint(kf[q]), e = (hi >> 20) & 0x7ff;
-      const ll mm = (((ll)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32) | (unsigned)__double2loint(kf[q])) << 7;
-      const int h = (int)(mm >> 30), l = (int)(mm & 0x3fffffff);
+      const ll mm = (((ll)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32) | (unsigned)__double2loint(kf[q])) << 9;
+      const int h = (int)(mm >> 31), l = (int)(mm & 0x7fffffff);
       fx2 y = fmk(frmul(v[q].x, h, l), frmul(v[q].y, h, l));
       if (hi < 0) y = fmk(-y.x, -y.y);
       v[q] = y;
@@ -525,7 +535,7 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
     }
     cta_max(&emx[1], em);
     __syncthreads();
-    const int e1 = emx[1] - kFxBits;  // exponent of the aligned products, on top of ex
+    const int e1 = emx[1] - kFxBitsProd;  // exponent of the aligned products, on top of ex
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int d = e1 - ev[q];
@@ -544,13 +554,13 @@ __device__ __forceinline__ void fx_pass_b_body(const PassArgs<double>& a) {
   __syncthreads();
 #pragma unroll
   for (int ls = 3; ls <= F::LS_TOP; ls += 3) {
-    const int s = fshift(mag[st]);
+    const int s = fshift<kFxLimitInv>(mag[st]);
     ex += s;
     m = X::template stage<false>(buf, t, ls, tw, s);
     cta_max(&mag[++st], m);
     __syncthreads();
   }
-  const int s = fshift(mag[st]);
+  const int s = fshift<kFxLimitInv>(mag[st]);
   ex += s;
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
@@ -679,7 +689,7 @@ __device__ __forceinline__ void fx_pass_c_body(const PassArgs<double>& a) {
     int st = 0;
 #pragma unroll
     for (int ls = 0; ls <= F::LS_TOP; ls += 3) {
-      const int s = fshift(mag[st]);
+      const int s = fshift<kFxLimitInv>(mag[st]);
       ex += s;
       m = X::template stage<false>(buf, t, ls, tw, s);
       cta_max(&mag[++st], m);
@@ -700,7 +710,7 @@ __device__ __forceinline__ void fx_pass_c_body(const PassArgs<double>& a) {
           if (act && n < half && 2 * n + h < nx) epi_gather<double, MODE>(a, rowoff + 2 * n + h, ein[e][h]);
       }
     }
-    const int s = fshift(mag[st]);
+    const int s = fshift<kFxLimitInv>(mag[st]);
     ex += s;
     fx2 v[8];
 #pragma unroll

@@ -91,13 +91,20 @@ void launch_to_f32(const double* src, float* dst, size_t n, cudaStream_t s) {
 // power, exp(-2 pi i o q/(R s)) at (q-1) s + o for q = 1..R-1 (offsets
 // FftC::pow_off; fewer than 2^logL entries in all).  FP32: exp(-2 pi i o/(R s))
 // for o < s (radix-8 offsets tw_off8); the butterflies form the powers.
-__device__ __forceinline__ int4 fx_limbs(double2 v) {  // w 2^60 = h 2^30 + l (fx_kernels.cuh)
-  const long long x = __double2ll_rn(v.x * 1152921504606846976.0), y = __double2ll_rn(v.y * 1152921504606846976.0);
+// w 2^62 = h 2^31 + l (fx_kernels.cuh): l in [-2^30, 2^30), but where h would be
+// +-2^31 (|w| within 2^-32 of 1), which a 32-bit integer and its negative cannot
+// both hold: there h = +-(2^31 - 1) and l takes the rest (+-1 less one unit for w = +-1).
+__device__ __forceinline__ void fx_limb(double v, int& h, int& l) {
+  const long long x = __double2ll_rn(v * 4611686018427387904.0);
+  const long long lo = ((int)x << 1) >> 1, m = 0x7fffffff;
+  const long long hi = min(max((x - lo) >> 31, -m), m);
+  h = (int)hi;
+  l = (int)min(max(x - (hi << 31), -m), m);
+}
+__device__ __forceinline__ int4 fx_limbs(double2 v) {
   int4 q;
-  q.y = ((int)x << 2) >> 2;
-  q.x = (int)((x - q.y) >> 30);
-  q.w = ((int)y << 2) >> 2;
-  q.z = (int)((y - q.w) >> 30);
+  fx_limb(v.x, q.x, q.y);
+  fx_limb(v.y, q.z, q.w);
   return q;
 }
 __device__ __forceinline__ double2 unit(double turns) {  // exp(2 pi i turns)
