@@ -57,7 +57,10 @@ extern "C" {
 typedef struct bem_ctx *bem_handle;
 
 typedef struct {
-  double tol;         /* stopping tolerance; 0 = default 1e-10 (FP64) / 1e-6 (FP32) */
+  double tol;         /* stopping tolerance; 0 = default 1e-10 (FP64) / 1e-6 (FP32).
+                         An FP64 non-adhesive solve has converged with the first
+                         iteration below it and goes on for two in a row, for at
+                         most 32 iterations and within max_iter                  */
   int max_iter;       /* CG iteration cap per solve; 0 = default 20000               */
   int precision;      /* BEM_PREC_*                                                  */
   int refine_sweeps;  /* FP32_REFINE: max refinement sweeps; 0 = default 3           */
@@ -69,7 +72,8 @@ typedef struct {
   double force;             /* F = dx dy sum p  (Sec. 3.1: "sum of pressures")    */
   double area;              /* dx dy * number of elements in contact              */
   double contact_radius;    /* sqrt(area / pi)                                     */
-  double final_eps;         /* last CG stopping measure                            */
+  double final_eps;         /* last CG stopping measure (of an FP64 non-adhesive
+                               solve that converged: the last one below tol)      */
   double max_gap_violation; /* max over contact of |g|, and of -g off contact      */
   double depth;             /* d of this solve                                     */
   int iterations;           /* CG iterations (all rounds of this step)             */

@@ -68,6 +68,7 @@ struct Scalars {
   double tau, beta, delta, G, G_old, eps, bnorm, pcrit;
   double sum_p, sum_dp, n_ol, n_ic, str, eps_min;
   double stop2;      // fixed-set CG: stop once |g|^2 <= stop2 = (tol |b|)^2
+  double eps_small;  // Polonsky-Keer: eps of the last iteration below the tolerance
   int max_iter, iter, done, status, have_tau, it_min;
   int nA;        // CTAs of the last pass A launch (its partials feed pass C)
   // Debug builds only: 1 = the first persistent pass A launch of the solve
@@ -80,7 +81,9 @@ struct Scalars {
   // CG iterations counted on the device, and the cap after which the solve
   // stops unconverged (the bound of the batched while-loop graph).
   int loops, max_loops;
-  int n_small;   // Polonsky-Keer: consecutive iterations with eps below the tolerance
+  // Polonsky-Keer: consecutive iterations with eps below the tolerance, and the
+  // first such iteration (0: none yet)
+  int n_small, it_small;
   unsigned int cnt_a, cnt_c, cnt_r;  // last-block arrival counters
   // Sticky device error bits (kept across solves: init_scalars does not copy
   // this member); 1 = a kernel gave up waiting for its own asynchronous copies,
