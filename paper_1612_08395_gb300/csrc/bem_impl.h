@@ -217,7 +217,7 @@ struct CoopArgs {
   int resume, max_launch;  // as ResArgs
 };
 size_t coop_shared_bytes();
-int coop_ctas(int lm, int lp, int nsm);  // CTAs of a launch, 0 where these lengths have no kernel
+int coop_ctas(int lm, int lp, int rows, int nsm);  // CTAs of a launch, 0 where there is none for these lengths and rows
 cudaError_t launch_coop_cg(const CoopArgs& r, int lm, int lp, cudaStream_t s);
 cudaError_t launch_coop_pk(const CoopArgs& r, int lm, int lp, cudaStream_t s);
 cudaError_t coop_setup_cg();  // once per device

@@ -559,12 +559,17 @@ constexpr size_t coop_smem(int R) { return 8 * (size_t)CoopGeo<LM, LP>::work + 1
 
 // CTAs and rows per CTA of the loop over `rows` rows: as many CTAs as give every
 // one a round of columns, at most one per SM; an even number of rows each, so
-// that W is read and written in 16-byte pairs.
+// that W is read and written in 16-byte pairs.  False where a CTA's share of the
+// rows does not fit its registers' bit masks or its shared memory (a device or
+// partition of few SMs: 1024 rows of 1024 points need 128).
+constexpr size_t kCoopSmemMax = 224 * 1024;  // an SM's 227 KB less the static part
 template <int LM, int LP>
-inline void coop_shape(int rows, int nsm, int* nb, int* R) {
+inline bool coop_shape(int rows, int nsm, int* nb, int* R) {
   using Gm = CoopGeo<LM, LP>;
   *nb = std::min(std::min(nsm, kCoopMaxCtas), (Gm::M + 1 + Gm::CPR - 1) / Gm::CPR);
+  if (*nb < 1) return false;
   *R = 2 * std::max(1, (rows + 2 * *nb - 1) / (2 * *nb));
+  return *R <= Gm::RMAX && coop_smem<LM, LP>(*R) <= kCoopSmemMax;
 }
 
 template <bool PK>
@@ -583,8 +588,7 @@ cudaError_t launch_coop_kind(CoopArgs r, int lm, int lp, cudaStream_t s) {
 #define BEM_CASE(LM, LP)                                                     \
   case LM * 16 + LP: {                                                       \
     int nb = 0;                                                              \
-    coop_shape<LM, LP>(r.rows, r.one.pl.nsm, &nb, &r.R);                     \
-    if (r.R > CoopGeo<LM, LP>::RMAX) return cudaErrorInvalidValue;           \
+    if (!coop_shape<LM, LP>(r.rows, r.one.pl.nsm, &nb, &r.R)) return cudaErrorInvalidValue; \
     cfg.gridDim = dim3(nb);                                                  \
     cfg.blockDim = dim3(CoopGeo<LM, LP>::NT);                                \
     cfg.dynamicSmemBytes = coop_smem<LM, LP>(r.R);                           \

@@ -967,10 +967,10 @@ struct CoopHold {
 // 1024 x 1024.  Below, a cluster's barriers are cheaper than the grid's (128 x 128:
 // 7.4 us in a cluster); above, an SM's share of the rows does not fit its shared
 // memory.  Pass timing needs the separate passes, and the server's loops share
-// launches instead.
-int coop_applies(const bem_ctx* h, int es) {
+// launches instead.  rows: grid rows that can hold pressure.
+int coop_applies(const bem_ctx* h, int es, int rows) {
   if (es != 4 || h->timing || h->batcher || !g_coop[h->device] || (h->ny & 1)) return 0;
-  return coop_ctas(ilog2(h->px / 2), ilog2(h->py), h->plan32.nsm);
+  return coop_ctas(ilog2(h->px / 2), ilog2(h->py), rows, h->plan32.nsm);
 }
 
 // The whole CG loop over `rows` grid rows as cooperative launches of nb CTAs, each
@@ -1061,8 +1061,9 @@ int run_pk(bem_ctx* h, double d, double tol, int max_iter, bool warm, StepOut* s
   launch_pk_init<T>(plan_of<T>(h), h->h64, d, pf.c, pf.p, pf.t, warm ? 1 : 0, h->ew_ngrid, h->stream);
   h->launches += 1;
   CKR(init_scalars(h, tol, max_iter, 0.0));
-  if (const int nb = coop_applies(h, (int)sizeof(T))) {
-    CKR(run_coop(h, true, h->is_sub ? h->rows_used : h->ny, nb));
+  const int rows = h->is_sub ? h->rows_used : h->ny;
+  if (const int nb = coop_applies(h, (int)sizeof(T), rows)) {
+    CKR(run_coop(h, true, rows, nb));
   } else if (resident_applies(h, (int)sizeof(T))) {
     CKR(run_resident(h, true));
   } else {
@@ -1208,19 +1209,23 @@ int run_fixed_cg(bem_ctx* h, double tol, int max_iter, double pcrit, StepOut* so
   CKR(ensure_fields<T>(h));
   PrecFields<T>& pf = fields_of<T>(h);
   CKR(init_scalars(h, tol, max_iter, pcrit));
-  const int coop = coop_applies(h, (int)sizeof(T));
   const bool resident = resident_applies(h, (int)sizeof(T));
-  if (!h->is_sub || !(coop || resident)) {  // the passes work on the contact band
+  int rows = h->rows_used, coop = 0;
+  if (h->is_sub) {
+    coop = coop_applies(h, (int)sizeof(T), rows);
+    if (!(coop || resident)) {  // the passes work on the contact band
+      launch_box(plan_of<T>(h), h->S, h->sc, h->stream);
+      h->launches += 1;
+    }
+  } else {
     launch_box(plan_of<T>(h), h->S, h->sc, h->stream);
     h->launches += 1;
-  }
-  int rows = h->rows_used;
-  if (!h->is_sub) {
     CKR(read_box(h));
     rows = h->box[1] + 1;
     bem_ctx* sub = nullptr;
     CKR(pick_sub(h, &sub));
     if (sub) return fixed_cg_in_box<T>(h, sub, tol, max_iter, pcrit, so);
+    coop = coop_applies(h, (int)sizeof(T), rows);
   }
   if (coop || resident) {
     if (coop) CKR(run_coop(h, false, rows, coop));
