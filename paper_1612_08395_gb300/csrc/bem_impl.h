@@ -71,8 +71,9 @@ struct Scalars {
   double eps_small;  // Polonsky-Keer: eps of the last iteration below the tolerance
   int max_iter, iter, done, status, have_tau, it_min;
   int nA;        // CTAs of the last pass A launch (its partials feed pass C)
-  // Debug builds only: 1 = the first persistent pass A launch of the solve
-  // waits on a barrier that nothing completes (tests the bounded wait)
+  // Debug builds only: 1 = the first persistent pass A launch or one-launch loop
+  // of the solve waits on a barrier that nothing completes (tests the bounded
+  // wait), 2 = a cooperative loop's gathering is given up
   int inject;
   // Rows band0 .. band1 and columns col0 .. col1 hold every element of the
   // fixed contact set S (band0 > band1: S is empty); written by k_box at the
@@ -84,6 +85,7 @@ struct Scalars {
   // Polonsky-Keer: consecutive iterations with eps below the tolerance, and the
   // first such iteration (0: none yet)
   int n_small, it_small;
+  int coop_runs;  // cooperative launches whose CTAs all became resident
   unsigned int cnt_a, cnt_c, cnt_r;  // last-block arrival counters
   // Sticky device error bits (kept across solves: init_scalars does not copy
   // this member); 1 = a kernel gave up waiting for its own asynchronous copies,

@@ -584,7 +584,7 @@ __device__ __forceinline__ void pass_ap_body(const PassArgs<T>& a) {
       __shared__ unsigned long long never;
       __shared__ int inj;
       if (tid == 0) {
-        inj = atomicExch(&sc->inject, 0);
+        inj = atomicExch(&sc->inject, 0) == 1;
         if (inj) mbar_init(&never, 1);
       }
       __syncthreads();

@@ -14,8 +14,14 @@
 //     serial tail beyond the barrier.
 // Only the rows that can hold pressure (the box of the held or overlap set) are
 // transformed.  The arithmetic is that of the passes; the order of the partial
-// sums differs.  Every wait is bounded: a CTA that gives up sets the handle's
-// error word and leaves, and so do the others.
+// sums differs.
+//
+// The CTAs wait for one another, so all must be resident, and another stream's
+// long kernel may hold some of them back.  They gather first: if one has waited a
+// tenth of a second for the others, all leave, nothing has been written, and the
+// host runs the loop as passes, which need no such thing.  Once gathered, no wait
+// depends on other work; each is bounded all the same, and a CTA that gives up
+// there sets the handle's error word and leaves, and so do the others.
 //
 // Bound by the barriers and the L2 round trips of W between them.  Measured
 // (GB300, per fixed-set iteration; a Polonsky-Keer one takes twice that): 256 x 256
@@ -44,9 +50,35 @@ struct CoopGeo {
 // State of the grid barrier and the partial sums (device memory of the handle).
 constexpr int kCoopMaxCtas = 256;
 struct CoopShared {
-  unsigned int count, pad[31];           // arrivals at the grid barrier
+  unsigned int count;                    // arrivals at the grid barrier
+  unsigned int gathered;                 // 0: CTAs are missing, 1: all are here, 2: given up
+  unsigned int pad[30];
   float2 part[2][kCoopMaxCtas * 8];      // alternating between consecutive sums
 };
+
+// The gathering: thread 0 of every CTA arrives, and asks after the loads that
+// need no other CTA whether all came.  The last to arrive and the first to run out
+// of patience both try to settle it; whoever does, all CTAs see the same answer.
+constexpr unsigned long long kCoopGatherNs = 100000000ull;
+__device__ __forceinline__ void coop_arrive(CoopShared* cs, int nb) {
+  if (atomicAdd(&cs->count, 1u) + 1 == (unsigned)nb) atomicCAS(&cs->gathered, 0u, 1u);
+}
+__device__ __forceinline__ bool coop_all_came(CoopShared* cs) {
+  unsigned v;
+  unsigned long long t0 = 0;
+  for (int i = 0;; ++i) {
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&cs->gathered) : "memory");
+    if (v) return v == 1;
+    if ((i & 1023) == 1023) {
+      const unsigned long long t = global_ns();
+      if (!t0) t0 = t;
+      else if (t - t0 > kCoopGatherNs) {
+        const unsigned old = atomicCAS(&cs->gathered, 0u, 2u);
+        return old == 1;
+      }
+    }
+  }
+}
 
 // Grid barrier: every CTA's earlier global writes are visible to every CTA
 // afterwards (read with L2 loads).  One counter, polled by one thread per CTA: a
@@ -338,15 +370,28 @@ struct Coop {
     c.rows = ca.rows;
     c.nb = gridDim.x;
     c.blk = blockIdx.x;
-    c.target = 0;
+    c.target = c.nb;  // the gathering's arrivals
     c.bad = &bad;
     c.magic = (65535 + c.R / 2) / (c.R / 2);
     float2* fld = c.work + Gm::work;  // [field][row slot][M/2] pairs: p, g, t, x (c or r)
     const int pl = c.R * (M / 2);
     float2 *fp = fld, *fg = fld + pl, *ft = fld + 2 * pl, *fx = fld + 3 * pl;
-    if (tid == 0) bad = 0;
     for (int i = tid; i < (int)(sizeof(Scalars) / 4); i += Gm::NT)
       reinterpret_cast<int*>(&sc)[i] = __ldcg(reinterpret_cast<const int*>(a.sc) + i);
+#ifdef BEM_DEBUG_CHECKS
+    // Test hooks of debug builds: CTA 0 stays away from the gathering (2), or from
+    // the first grid barrier (1); the others' waits run out (bounded).
+    __syncthreads();
+    const int away = blockIdx.x == 0 ? sc.inject : 0;
+    if (away) {
+      if (tid == 0) a.sc->inject = 0;
+      if (away == 2) return;
+    }
+#endif
+    if (tid == 0) {
+      bad = 0;
+      coop_arrive(c.cs, c.nb);
+    }
     const int nx = a.pl.nx;
     const int b = tid / Gm::TR, t = tid % Gm::TR;
     const float us = (float)a.uscale;
@@ -386,7 +431,12 @@ struct Coop {
         }
       }
     }
+    if (tid == 0 && !coop_all_came(c.cs)) bad = 1;
     __syncthreads();
+    if (bad) return;  // not all CTAs are resident; nothing has been written
+#ifdef BEM_DEBUG_CHECKS
+    if (away) return;
+#endif
     bool ok = true;
     // one transform per pass of this loop, whatever it is for (see resident.cuh)
     enum { kP, kT, kG };
@@ -533,13 +583,18 @@ struct Coop {
         }
       }
     }
-    // rows past c.rows hold no pressure
+    // rows past c.rows hold no pressure (nor, in a loop that goes on, anything else)
     for (size_t i = (size_t)c.rows * nx + (size_t)blockIdx.x * Gm::NT + tid; i < (size_t)a.pl.ny * nx;
-         i += (size_t)c.nb * Gm::NT)
+         i += (size_t)c.nb * Gm::NT) {
       a.f.p[i] = 0.f;
+      if (!sc.done) a.f.g[i] = a.f.t[i] = a.f.r[i] = 0.f;
+    }
     if (blockIdx.x == 0) {  // the scalars, all but the sticky error word
       __syncthreads();
-      if (tid == 0 && fin) sc.have_tau = 0;
+      if (tid == 0) {
+        sc.coop_runs += 1;
+        if (fin) sc.have_tau = 0;
+      }
       __syncthreads();
       for (int i = tid; i < (int)(offsetof(Scalars, kerr) / 4); i += Gm::NT)
         reinterpret_cast<int*>(a.sc)[i] = reinterpret_cast<const int*>(&sc)[i];
@@ -581,8 +636,8 @@ cudaError_t launch_coop_kind(CoopArgs r, int lm, int lp, cudaStream_t s) {
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  // a fresh barrier for every launch
-  cudaError_t e = cudaMemsetAsync(r.shared, 0, sizeof(unsigned int), s);
+  // a fresh barrier and gathering for every launch
+  cudaError_t e = cudaMemsetAsync(r.shared, 0, offsetof(CoopShared, pad), s);
   if (e != cudaSuccess) return e;
   switch (lm * 16 + lp) {
 #define BEM_CASE(LM, LP)                                                     \

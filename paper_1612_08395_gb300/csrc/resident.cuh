@@ -473,7 +473,7 @@ struct Resident {
     __syncthreads();
 #ifdef BEM_DEBUG_CHECKS
     // Test hook of debug builds: a wait that nothing completes runs out (bounded).
-    if (sc.inject) {
+    if (sc.inject == 1) {
       __shared__ unsigned long long never;
       cl_sync();
       if (rank == 0 && tid == 0) {

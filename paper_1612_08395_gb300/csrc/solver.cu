@@ -495,9 +495,10 @@ int init_scalars(bem_ctx* h, double tol, int max_iter, double pcrit) {
   s.kerr = h->sc_host->kerr;
 #ifdef BEM_DEBUG_CHECKS
   // test hook: BEM_INJECT_WAIT_TIMEOUT=1 makes the solve's first persistent
-  // pass A launch run a bounded wait out (reported as BEM_ETIMEOUT)
+  // pass A launch or one-launch loop run a bounded wait out (reported as
+  // BEM_ETIMEOUT), =2 a cooperative loop its gathering (it runs as passes)
   const char* inj = getenv("BEM_INJECT_WAIT_TIMEOUT");
-  s.inject = inj && inj[0] == '1';
+  s.inject = inj && (inj[0] == '1' || inj[0] == '2') ? inj[0] - '0' : 0;
 #endif
   *h->sc_host = s;
   launch_set_scalars(s, h->sc, h->stream);
@@ -973,9 +974,12 @@ int coop_applies(const bem_ctx* h, int es, int rows) {
   return coop_ctas(ilog2(h->px / 2), ilog2(h->py), rows, h->plan32.nsm);
 }
 
-// The whole CG loop over `rows` grid rows as cooperative launches of nb CTAs, each
-// of at most kResidentIters iterations.
-int run_coop(bem_ctx* h, bool pk, int rows, int nb) {
+// The CG loop over `rows` grid rows as cooperative launches of nb CTAs, each of at
+// most kResidentIters iterations.  *finished = false: a launch's CTAs did not all
+// become resident, the loop's state is as before it (nothing or a number of whole
+// launches done) and the passes go on from there.
+int run_coop(bem_ctx* h, bool pk, int rows, int nb, bool* finished) {
+  *finished = false;
   if (!h->coop) CKR(dmalloc(h, &h->coop, coop_shared_bytes()));
   CoopHold hold;
   hold.acquire(h, nb);
@@ -985,12 +989,15 @@ int run_coop(bem_ctx* h, bool pk, int rows, int nb) {
   r.rows = rows < 1 ? 1 : rows;
   r.max_launch = kResidentIters;
   const int lm = ilog2(h->px / 2), lp = ilog2(h->py);
-  do {
+  for (int runs = 1;; ++runs) {
     CK(pk ? launch_coop_pk(r, lm, lp, h->stream) : launch_coop_cg(r, lm, lp, h->stream));
     h->launches += 1;
     CKR(read_scalars(h));
+    if (h->sc_host->coop_runs != runs) return BEM_OK;
+    if (h->sc_host->done) break;
     r.resume = 1;
-  } while (!h->sc_host->done);
+  }
+  *finished = true;
   return BEM_OK;
 }
 
@@ -1061,12 +1068,12 @@ int run_pk(bem_ctx* h, double d, double tol, int max_iter, bool warm, StepOut* s
   launch_pk_init<T>(plan_of<T>(h), h->h64, d, pf.c, pf.p, pf.t, warm ? 1 : 0, h->ew_ngrid, h->stream);
   h->launches += 1;
   CKR(init_scalars(h, tol, max_iter, 0.0));
-  const int rows = h->is_sub ? h->rows_used : h->ny;
-  if (const int nb = coop_applies(h, (int)sizeof(T), rows)) {
-    CKR(run_coop(h, true, rows, nb));
-  } else if (resident_applies(h, (int)sizeof(T))) {
+  const int rows = h->is_sub ? h->rows_used : h->ny, nb = coop_applies(h, (int)sizeof(T), rows);
+  bool finished = false;
+  if (nb) CKR(run_coop(h, true, rows, nb, &finished));
+  if (!nb && resident_applies(h, (int)sizeof(T))) {
     CKR(run_resident(h, true));
-  } else {
+  } else if (!finished) {
     if (!pf.pk_graph[0]) CKR(capture_chunk<T>(h, true, false, &pf.pk_graph[0]));
     if (h->timing && !pf.pk_graph[1]) CKR(capture_chunk<T>(h, true, true, &pf.pk_graph[1]));
     CKR(run_loop(h, pf.pk_graph[0], pf.pk_graph[1], max_iter, true, (int)sizeof(T)));
@@ -1227,23 +1234,33 @@ int run_fixed_cg(bem_ctx* h, double tol, int max_iter, double pcrit, StepOut* so
     if (sub) return fixed_cg_in_box<T>(h, sub, tol, max_iter, pcrit, so);
     coop = coop_applies(h, (int)sizeof(T), rows);
   }
-  if (coop || resident) {
-    if (coop) CKR(run_coop(h, false, rows, coop));
-    else CKR(run_resident(h, false));
+  bool finished = false;
+  if (coop) CKR(run_coop(h, false, rows, coop, &finished));
+  if (!coop && resident) {
+    CKR(run_resident(h, false));
+    finished = true;
+  }
+  if (finished) {
     so->eps = h->sc_host->iter > 0 ? sqrt(std::max(h->sc_host->G, 0.0)) / h->sc_host->bnorm : h->sc_host->eps;
   } else {
     if (!pf.cg_graph[0]) CKR(capture_chunk<T>(h, false, false, &pf.cg_graph[0]));
     if (h->timing && !pf.cg_graph[1]) CKR(capture_chunk<T>(h, false, true, &pf.cg_graph[1]));
-    const size_t n = (size_t)h->nx * h->ny;
-    launch_mask_field<T>(pf.p, h->S, n, h->stream);
-    launch_mask_field<T>(pf.t, h->S, n, h->stream);
     PassArgs<T> a = make_args<T>(h);
-    a.f.src = pf.p;
-    launch_pass_a<T>(a, A_PLAIN, h->stream);
-    launch_pass_b<T>(a, B_CONV, h->stream);
-    launch_pass_c<T>(a, C_CG_G, h->stream);
-    h->launches += 5;
-    CKR(read_scalars(h));
+    if (h->is_sub && coop) {  // the cooperative loop needs no band, the passes do
+      launch_box(plan_of<T>(h), h->S, h->sc, h->stream);
+      h->launches += 1;
+    }
+    if (h->sc_host->coop_runs == 0) {
+      const size_t n = (size_t)h->nx * h->ny;
+      launch_mask_field<T>(pf.p, h->S, n, h->stream);
+      launch_mask_field<T>(pf.t, h->S, n, h->stream);
+      a.f.src = pf.p;
+      launch_pass_a<T>(a, A_PLAIN, h->stream);
+      launch_pass_b<T>(a, B_CONV, h->stream);
+      launch_pass_c<T>(a, C_CG_G, h->stream);
+      h->launches += 5;
+      CKR(read_scalars(h));
+    }
     if (!h->sc_host->done) {
       CKR(run_loop(h, pf.cg_graph[0], pf.cg_graph[1], max_iter, false, (int)sizeof(T)));
       if (h->sc_host->have_tau) {
