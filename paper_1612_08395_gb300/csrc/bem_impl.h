@@ -73,7 +73,8 @@ struct Scalars {
   int nA;        // CTAs of the last pass A launch (its partials feed pass C)
   // Debug builds only: 1 = the first persistent pass A launch or one-launch loop
   // of the solve waits on a barrier that nothing completes (tests the bounded
-  // wait), 2 = a cooperative loop's gathering is given up
+  // wait), 2 or 3 = the gathering of a cooperative loop's first or second launch is
+  // given up
   int inject;
   // Rows band0 .. band1 and columns col0 .. col1 hold every element of the
   // fixed contact set S (band0 > band1: S is empty); written by k_box at the

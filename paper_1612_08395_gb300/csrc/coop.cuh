@@ -189,6 +189,7 @@ struct Coop {
         }
         const int km = k == 0 ? M : M - k;
         // rows_w is even: the pair is inside W's row even where y + 1 is past the last row
+        if (!bem_check(k <= M && km <= M && y + 1 < a.rows_w, a.kerr)) continue;
         __stcg(reinterpret_cast<float4*>(W + (size_t)k * a.rows_w + y), make_float4(xk0.x, xk0.y, xk1.x, xk1.y));
         if (km != k)
           __stcg(reinterpret_cast<float4*>(W + (size_t)km * a.rows_w + y), make_float4(xm0.x, xm0.y, xm1.x, xm1.y));
@@ -217,7 +218,7 @@ struct Coop {
         v[e] = make_float2(0.f, 0.f);
         if (!FC::first_half(e)) continue;
         const int y = FC::n0(t, e);
-        if (y < c.rows) v[e] = __ldcg(w + y);
+        if (y < c.rows && bem_check(kx <= M && y < a.rows_w, a.kerr)) v[e] = __ldcg(w + y);
       }
       FC::stage0_fwd(v, t, tw);
 #pragma unroll
@@ -258,7 +259,7 @@ struct Coop {
       for (int e = 0; e < 8; ++e) {
         if (!FC::first_half(e)) continue;
         const int y = FC::n0(t, e);
-        if (y < c.rows) __stcg(w + y, v[e]);
+        if (y < c.rows && bem_check(kx <= M && y < a.rows_w, a.kerr)) __stcg(w + y, v[e]);
       }
     }
   }
@@ -280,7 +281,7 @@ struct Coop {
       for (int idx = tid; idx < (M / 2 + 1) * rp; idx += Gm::NT) {
         const int k = (idx * magic) >> 16, bb = 2 * (idx - k * rp);
         const int y = c.blk * c.R + r0 + bb;
-        if (y >= c.rows) continue;
+        if (y >= c.rows || !bem_check(k <= M && y + 1 < a.rows_w, a.kerr)) continue;
         const float4 fk = __ldcg(reinterpret_cast<const float4*>(W + (size_t)k * a.rows_w + y));
         const float4 fm = __ldcg(reinterpret_cast<const float4*>(W + (size_t)(M - k) * a.rows_w + y));
         const int pk = __ldg(sp + k), pm = k ? __ldg(sp + M - k) : 0;
@@ -379,10 +380,11 @@ struct Coop {
     for (int i = tid; i < (int)(sizeof(Scalars) / 4); i += Gm::NT)
       reinterpret_cast<int*>(&sc)[i] = __ldcg(reinterpret_cast<const int*>(a.sc) + i);
 #ifdef BEM_DEBUG_CHECKS
-    // Test hooks of debug builds: CTA 0 stays away from the gathering (2), or from
-    // the first grid barrier (1); the others' waits run out (bounded).
+    // Test hooks of debug builds: CTA 0 stays away from the gathering of the loop's
+    // first launch (2) or second (3), or from the first grid barrier (1); the others'
+    // waits run out (bounded).
     __syncthreads();
-    const int away = blockIdx.x == 0 ? sc.inject : 0;
+    const int away = blockIdx.x ? 0 : sc.inject == 1 ? 1 : sc.inject >= 2 && sc.coop_runs == sc.inject - 2 ? 2 : 0;
     if (away) {
       if (tid == 0) a.sc->inject = 0;
       if (away == 2) return;

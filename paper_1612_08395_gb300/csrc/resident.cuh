@@ -313,6 +313,7 @@ struct Resident {
           split_two<float>(s1, pk, pm, w, xk1, xm1);
         }
         const int km = k == 0 ? M : M - k;
+        if (!bem_check(k / Q < CS && km / Q < CS && y0 + bb + 1 < Gm::CP, a.kerr)) continue;
         cl_st4(cl_map(colin + (k % Q) * Gm::CP + y0 + bb, k / Q), xk0, xk1);
         if (km != k) cl_st4(cl_map(colin + (km % Q) * Gm::CP + y0 + bb, km / Q), xm0, xm1);
       }
@@ -380,7 +381,7 @@ struct Resident {
           for (int e = 0; e < 8; ++e) {
             if (!FC::first_half(e)) continue;
             const int y = FC::n0(tc, e);
-            if (y < ny) cl_st2(cl_map(rowin + kx * R + y % R, y / R), v[e]);
+            if (y < ny && bem_check(kx <= M && y / R < CS, a.kerr)) cl_st2(cl_map(rowin + kx * R + y % R, y / R), v[e]);
           }
         }
       }

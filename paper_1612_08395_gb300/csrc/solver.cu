@@ -87,8 +87,16 @@ constexpr int kChunk = BEM_CHUNK;  // CG iterations per captured graph launch
 #define BEM_LOOP_BODY 4
 #endif
 constexpr int kLoopBody = BEM_LOOP_BODY;
-// CG iterations of one launch of a resident loop (resident.cuh) at most
+// CG iterations of one launch of a one-launch loop (resident.cuh, coop.cuh) at most
 constexpr int kResidentIters = 4096;
+int loop_iters() {
+#ifdef BEM_DEBUG_CHECKS
+  // test hook: loops of several launches
+  const char* e = getenv("BEM_LOOP_ITERS");
+  if (e && atoi(e) > 0) return atoi(e);
+#endif
+  return kResidentIters;
+}
 
 // Threads per CTA of the row passes (rows per CTA x M/8); 512 keeps two CTAs
 // resident per SM at the passes' register use.
@@ -496,9 +504,10 @@ int init_scalars(bem_ctx* h, double tol, int max_iter, double pcrit) {
 #ifdef BEM_DEBUG_CHECKS
   // test hook: BEM_INJECT_WAIT_TIMEOUT=1 makes the solve's first persistent
   // pass A launch or one-launch loop run a bounded wait out (reported as
-  // BEM_ETIMEOUT), =2 a cooperative loop its gathering (it runs as passes)
+  // BEM_ETIMEOUT), =2 or 3 the gathering of a cooperative loop's first or second
+  // launch (it goes on as passes)
   const char* inj = getenv("BEM_INJECT_WAIT_TIMEOUT");
-  s.inject = inj && (inj[0] == '1' || inj[0] == '2') ? inj[0] - '0' : 0;
+  s.inject = inj && inj[0] >= '1' && inj[0] <= '3' ? inj[0] - '0' : 0;
 #endif
   *h->sc_host = s;
   launch_set_scalars(s, h->sc, h->stream);
@@ -784,7 +793,7 @@ int launch_group(LoopBatcher* b, std::vector<LoopReq*>& g, const std::vector<int
   if (resident) {
     ResArgs r{};
     r.arr = reinterpret_cast<const PassArgs<float>*>(en.d_args);
-    r.max_launch = kResidentIters;
+    r.max_launch = loop_iters();
     CK(launch_resident(r, g[0]->h, g[0]->pk, n, b->stream));
   } else {
     CK(cudaGraphLaunch(en.exec, b->stream));
@@ -987,7 +996,7 @@ int run_coop(bem_ctx* h, bool pk, int rows, int nb, bool* finished) {
   r.one = make_args<float>(h);
   r.shared = h->coop;
   r.rows = rows < 1 ? 1 : rows;
-  r.max_launch = kResidentIters;
+  r.max_launch = loop_iters();
   const int lm = ilog2(h->px / 2), lp = ilog2(h->py);
   for (int runs = 1;; ++runs) {
     CK(pk ? launch_coop_pk(r, lm, lp, h->stream) : launch_coop_cg(r, lm, lp, h->stream));
@@ -1008,7 +1017,7 @@ int run_resident(bem_ctx* h, bool pk) {
   if (h->batcher) CKR(run_loop_batched(h, pk, 4, &solo));
   ResArgs r{};
   r.one = make_args<float>(h);
-  r.max_launch = kResidentIters;
+  r.max_launch = loop_iters();
   r.resume = solo ? 0 : 1;
   if (solo) {
     CK(launch_resident(r, h, pk, 1, h->stream));
