@@ -165,7 +165,9 @@ int bem_contact_set(bem_handle h, unsigned char *S_out);
  * later jobs that do fit go first, and idle cached handles are evicted least
  * recently used first.  Handles (influence spectra) are cached by
  * (Nx, Ny, dx, dy, k) and reused with bem_set_material for nu, E0, c0.
- * Results are deterministic: a job's outputs do not depend on what else runs.
+ * A job alone in the server gives the results of the same sweep on a handle of its
+ * own, bitwise; in a mix they agree to rounding, since which loops share a launch
+ * depends on what else runs.
  *
  * bem_job: the arguments of one bem_sweep (a single solve is nsteps = 1; an
  * adhesive solve is {d_preload, d}).  The job struct is copied on submit; the
@@ -191,8 +193,7 @@ int bem_contact_set(bem_handle h, unsigned char *S_out);
  *   per solve, the others as one while-loop graph in which every transform pass
  *   is a single launch over all of them, each instance stopping at its own
  *   convergence.  *launches = such launches, *loops = the solves' loops they
- *   carried.  Counts and statuses are those of the job run alone, forces and
- *   pressures agree with it to rounding.
+ *   carried.  A job alone runs its loops as its own handle would.
  *   BEM_BATCH_LOOPS=0 in the environment makes every job run its own loops.
  * bem_server_footprint: the bytes admission reserves for a job on an Nx x Ny
  *   grid (a handle after FP32 and FP64 solves plus its set-up workspace);

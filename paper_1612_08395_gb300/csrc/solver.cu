@@ -691,6 +691,12 @@ void batcher_leave(LoopBatcher* b) {
   b->cv.notify_all();  // the waiting loops may now be all there are
 }
 
+// Whether no other solve is in flight on the batcher's device.
+static bool batcher_alone(LoopBatcher* b) {
+  std::lock_guard<std::mutex> lk(b->mu);
+  return b->active <= 1;
+}
+
 void batcher_stats(LoopBatcher* b, long long* launches, long long* instances) {
   std::lock_guard<std::mutex> lk(b->mu);
   *launches += b->launches;
@@ -976,10 +982,13 @@ struct CoopHold {
 // a cluster at 256 x 256, 14 against 21 as passes at 512 x 512, 29 against 33 at
 // 1024 x 1024.  Below, a cluster's barriers are cheaper than the grid's (128 x 128:
 // 7.4 us in a cluster); above, an SM's share of the rows does not fit its shared
-// memory.  Pass timing needs the separate passes, and the server's loops share
-// launches instead.  rows: grid rows that can hold pressure.
+// memory.  Pass timing needs the separate passes, and loops of several jobs in the
+// server share launches instead (its clusters would keep a cooperative launch's
+// CTAs out); a job alone there runs as it would on a handle of its own.  rows: grid
+// rows that can hold pressure.
 int coop_applies(const bem_ctx* h, int es, int rows) {
-  if (es != 4 || h->timing || h->batcher || !g_coop[h->device] || (h->ny & 1)) return 0;
+  if (es != 4 || h->timing || !g_coop[h->device] || (h->ny & 1)) return 0;
+  if (h->batcher && !batcher_alone(h->batcher)) return 0;
   return coop_ctas(ilog2(h->px / 2), ilog2(h->py), rows, h->plan32.nsm);
 }
 
