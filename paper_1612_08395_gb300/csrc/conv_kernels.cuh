@@ -350,11 +350,21 @@ __device__ __forceinline__ void split_store(const C<T>* sm, int rs, int nb, int 
   }
 }
 
+// The row passes gather the fields of a thread's elements into small arrays first
+// (`in`, `ein`), each under the condition that the element is on the grid, and use
+// them later under the same condition.  The arrays are initialised all the same:
+// left uninitialised, k_pass_c<float, C_CG_R, 7> compiled for three CTAs per SM (40
+// registers, spilling) dropped elements of the columns from 96 on -- r kept its old
+// value and the sums missed them, deterministically, but differently for other
+// builds of the kernels that ran before it, as if a spilled value were read that had
+// not been written; launched by itself it was right.  Every second of 216 grids and
+// iteration counts was wrong, none with the arrays initialised, at the same 40
+// registers.  Initialised, the staged passes also need fewer registers and none of
+// their spills (fixed-set pass A 64 -> 56).
+//
 // Launch bounds of the row passes (A and C): the plan caps their CTAs at
-// BEM_MAX_THREADS_A threads except for the longest rows.  Two resident CTAs per
-// SM: with three (40 registers) the compiled fixed-set passes of 128-point rows
-// were wrong -- from the second iteration on, with columns past 96 in use -- while
-// the same source is right at 64 registers and above.
+// BEM_MAX_THREADS_A threads except for the longest rows; two resident CTAs per SM
+// hold the unstaged passes without spills.
 #ifndef BEM_ROW_MIN_BLOCKS
 #define BEM_ROW_MIN_BLOCKS 2
 #endif
@@ -411,7 +421,7 @@ __global__ void BEM_ROW_BOUNDS(LOGL) k_pass_a(PassArgs<T> a) {
       v[e] = mk<T>(xv[0], xv[1]);
     }
   } else {
-    PIn<T> in[8][2];
+    PIn<T> in[8][2] = {};
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       if (HALF && !F::first_half(e)) continue;
@@ -596,7 +606,7 @@ __device__ __forceinline__ void pass_ap_body(const PassArgs<T>& a) {
       return;
     }
     // ncols is a multiple of 16 here: column pairs (2n, 2n+1) are whole
-    PIn<T> in[8][2];
+    PIn<T> in[8][2] = {};
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       if (!F::first_half(e)) continue;
@@ -1395,7 +1405,7 @@ __global__ void BEM_ROW_BOUNDS(LOGL) k_pass_c(PassArgs<T> a) {
   const bool act = row < ny;
   const size_t rowoff = (size_t)row * nx;
   const int half = (nx + 1) >> 1;
-  EIn<T> ein[8][2];
+  EIn<T> ein[8][2] = {};
   if (staged) {
     cp_async_wait_all();
     __syncthreads();
@@ -1610,7 +1620,7 @@ __device__ __forceinline__ void pass_cp_body(const PassArgs<T>& a) {
     const bool act = row < ny;
     const size_t rowoff = (size_t)row * nx;
     // nx is a multiple of 16 here: column pairs (2n, 2n+1) are whole
-    EIn<T> ein[8][2];
+    EIn<T> ein[8][2] = {};
     if (MODE != C_PLAIN && MODE != C_PLAIN64) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) {

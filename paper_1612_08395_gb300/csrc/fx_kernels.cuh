@@ -326,7 +326,7 @@ __device__ __forceinline__ void fx_pass_a_body(const PassArgs<double>& a) {
 
   double x[8][2];
   {
-    PIn<double> in[8][2];
+    PIn<double> in[8][2] = {};
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       if (!F::first_half(e)) continue;
@@ -699,7 +699,7 @@ __device__ __forceinline__ void fx_pass_c_body(const PassArgs<double>& a) {
     const bool act = row < ny;
     const size_t rowoff = (size_t)row * nx;
     const int half = (nx + 1) >> 1;
-    EIn<double> ein[8][2];
+    EIn<double> ein[8][2] = {};
     if (MODE != C_PLAIN) {
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
