@@ -1183,43 +1183,48 @@ template <typename T, int MODE>
 __device__ __forceinline__ void pass_c_finalize(Scalars* sc, const double (&s2)[4], const double (&s3)[3],
                                                 const CgPre& pre) {
   if (MODE == C_PK_G) {
+    // the scalars this needs are read before any is written, so their loads overlap
+    const int have = sc->have_tau, iter = sc->iter + 1, max_iter = sc->max_iter, it_min = sc->it_min;
+    const int small_run = sc->n_small, small_first = sc->it_small;
+    const double tol = sc->tol, eps_min = sc->eps_min, G_old = sc->G_old, last_small = sc->eps_small;
+    double delta = sc->delta;
     sc->cnt_c = 0;
     const double G = s2[0], nic = s2[1];
     int done = 0;
-    if (sc->have_tau) {
+    if (have) {
+      double eps = s3[1] > 0.0 ? s3[0] / s3[1] : 0.0;
+      delta = s3[2] > 0.0 ? 0.0 : 1.0;
+      const bool small = eps < tol;
+      const int run = small ? small_run + 1 : 0, first = small && !small_first ? iter : small_first;
+      const double small_eps = small ? eps : last_small;
+      int end = SC_OK;  // how the solve ends here if no step has been small
+      if (!isfinite(eps) || !isfinite(G)) { sc->status = SC_NUMERIC; done = 1; }
+      else if (run >= kSmallSteps<T>) done = 1;
+      else if (first && iter - first >= kSmallWait) { eps = small_eps; done = 1; }
+      else if (iter >= max_iter) end = SC_NOCONV;
+      // rounding floor: no new minimum of eps for kStall iterations ends the solve
+      else if (iter == 1 || eps < 0.5 * eps_min) { sc->eps_min = eps; sc->it_min = iter; }
+      else if (iter - it_min > kStall) end = SC_STALL;
+      if (end != SC_OK) {
+        done = 1;
+        if (first) eps = small_eps;
+        else sc->status = end;
+      }
       sc->sum_dp = s3[0];
       sc->sum_p = s3[1];
       sc->n_ol = s3[2];
-      sc->iter += 1;
-      const double eps = s3[1] > 0.0 ? s3[0] / s3[1] : 0.0;
+      sc->iter = iter;
       sc->eps = eps;
-      sc->delta = s3[2] > 0.0 ? 0.0 : 1.0;
-      if (eps < sc->tol) {
-        sc->n_small += 1;
-        sc->eps_small = eps;
-        if (!sc->it_small) sc->it_small = sc->iter;
-      } else {
-        sc->n_small = 0;
-      }
-      int end = SC_OK;  // how the solve ends here if no step has been small
-      if (!isfinite(eps) || !isfinite(G)) { sc->status = SC_NUMERIC; done = 1; }
-      else if (sc->n_small >= kSmallSteps<T>) done = 1;
-      else if (sc->it_small && sc->iter - sc->it_small >= kSmallWait) { sc->eps = sc->eps_small; done = 1; }
-      else if (sc->iter >= sc->max_iter) end = SC_NOCONV;
-      // rounding floor: no new minimum of eps for kStall iterations ends the solve
-      else if (sc->iter == 1 || eps < 0.5 * sc->eps_min) { sc->eps_min = eps; sc->it_min = sc->iter; }
-      else if (sc->iter - sc->it_min > kStall) end = SC_STALL;
-      if (end != SC_OK) {
-        done = 1;
-        if (sc->it_small) sc->eps = sc->eps_small;
-        else sc->status = end;
-      }
+      sc->delta = delta;
+      sc->n_small = run;
+      sc->it_small = first;
+      sc->eps_small = small_eps;
     }
     sc->n_ic = nic;
     sc->G = G;
     if (!done) {
       if (nic == 0.0 || G == 0.0) { done = 1; }
-      else { sc->beta = sc->delta * G / sc->G_old; sc->G_old = G; }
+      else { sc->beta = delta * G / G_old; sc->G_old = G; }
     }
     if (done) sc->done = 1;
   } else if (MODE == C_PK_R) {
