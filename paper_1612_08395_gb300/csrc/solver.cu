@@ -998,7 +998,6 @@ int coop_applies(const bem_ctx* h, int es, int rows) {
 // launches done) and the passes go on from there.
 int run_coop(bem_ctx* h, bool pk, int rows, int nb, bool* finished) {
   *finished = false;
-  if (!h->coop) CKR(dmalloc(h, &h->coop, coop_shared_bytes()));
   CoopHold hold;
   hold.acquire(h, nb);
   CoopArgs r{};
@@ -1654,6 +1653,7 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
       {(void**)&h->stats, sizeof(double) * (8 + 4 * (size_t)h->stats_ngrid + 8)},
       {(void**)&h->sc, sizeof(Scalars)},
       {(void**)&h->tmw, sizeof(CUtensorMap)},
+      {&h->coop, coop_shared_bytes()},
       {(void**)&h->S, n},
       {&h->W, w_bytes},
       {(void**)&h->h64, f_bytes},
@@ -1743,7 +1743,6 @@ extern "C" void bem_destroy(bem_handle h) {
     for (int j = 0; j < 4; ++j)
       if (h->ev[i][j]) cudaEventDestroy(h->ev[i][j]);
   if (h->ev_ready) cudaEventDestroy(h->ev_ready);
-  fr(h->coop);
   fr(h->block);
   fr(h->f32.block);
   fr(h->f64.block);
