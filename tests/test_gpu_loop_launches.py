@@ -108,21 +108,23 @@ for nx, ny in ((40, 40), (30, 17), (130, 200), (255, 255), (256, 256), (300, 514
                 rec["err"] = float(np.linalg.norm(a[0] - b[0]) / max(np.linalg.norm(a[0]), 1e-300))
                 rec["counts"] = [x[2] for x in a[2]] == [x[2] for x in b[2]]
             out.append(rec)
-# the same job several times at once in the server, whose loops share launches
+# the same job several times at once in the server, whose loops share cluster launches (240: or,
+# while a job happens to be the only one in flight, run as cooperative ones)
 served = []
 for iters in (0, 3):
     env(iters)
     jobs, ps = [], []
     with bem.Server(nworkers=4, hbm_budget_bytes=8 << 30) as s:
-        for n in (100, 100, 240, 240):
+        for n in (100, 100, 120, 120, 240, 240):
             h = np.where(I.radius_grid(n, n, 1.0 / n) <= 0.45, 0.0, I.EXCLUDED)
             p = np.empty((n, n)); ps.append(p)
             s.submit(n, n, 1.0 / n, 1.0 / n, 0.3, 0.3, h, [0.01, 0.004], dgamma=1e-5, final_pressure=p, precision="fp32_refine")
         done = s.drain()
     served.append([p.copy() for p in ps])
 env()
-print(json.dumps({"runs": out, "served": [bool(np.array_equal(a, b)) for a, b in zip(*served)],
-                  "twins": [bool(np.array_equal(served[0][0], served[0][1])), bool(np.array_equal(served[0][2], served[0][3]))]}))
+a, b = served
+print(json.dumps({"runs": out, "bitwise": [bool(np.array_equal(x, y)) for x, y in zip(a[:4] + a[0:1] + a[2:3], b[:4] + a[1:2] + a[3:4])],
+                  "rounding": [float(np.linalg.norm(x - y) / np.linalg.norm(y)) for x, y in zip(a[4:] + a[4:5], b[4:] + a[5:6])]}))
 """
 
 
@@ -149,4 +151,4 @@ def test_loop_handed_to_the_passes_half_way(split):
 
 
 def test_split_loops_in_the_server(split):
-    assert all(split["served"]) and all(split["twins"])
+    assert all(split["bitwise"]) and max(split["rounding"]) <= 1e-9
