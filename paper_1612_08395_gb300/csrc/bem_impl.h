@@ -17,14 +17,12 @@ struct Geo {
   int rs;
 };
 
-// Per-length index tables on the device (int32):
-//   so[ls * 8 + r] = swz(r << ls), ls = 0..13     (112 entries)
-//   sp[k]          = swz(dig_pos(k)), k < 2^logL  (digit-reversed, swizzled)
-constexpr int kSoEntries = 112;
+// Index table of one length on the device (int32):
+//   sp[k] = swz(dig_pos(k)), k < 2^logL  (digit-reversed, swizzled)
 
 // Every table of a context, made by one launch: twiddles as [length-M stages |
 // length-Py stages | real-FFT split | radix-16 length-Py stages (FP32 only)] in
-// FP64, FP32 and as fixed-point limbs, and up to four index tables, so then sp
+// FP64, FP32 and as fixed-point limbs, and up to four index tables sp
 // (null pointers: not made).
 struct TableArgs {
   int logM, logP;
@@ -150,9 +148,7 @@ struct PassArgs {
   const int4* fxS;
   int* fx_ea;           // FP64 path: exponents of W's row groups (pass A) ...
   int* fx_eb;           // ... and of its columns kx (pass B)
-  const int* soA;       // index tables of length M and Py (see Geo)
-  const int* spA;
-  const int* soB;
+  const int* spA;       // index tables of length M and Py (see Geo)
   const int* spB;
   double* khat64_out;   // B_SPECTRUM outputs ([kx][ky])
   float* khat32_out;

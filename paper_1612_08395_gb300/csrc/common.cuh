@@ -225,8 +225,8 @@ __host__ __device__ __forceinline__ int tw_off8(int logL, int r0, int ls) {
   return (r0 ? top : 0) + (top - (8 << ls)) / 7;
 }
 
-// v[q] *= w^q, q = 1..7, with the same products as powers8 but each power
-// formed just before it is used (fewer values live at once).
+// v[q] *= w^q, q = 1..7, each power formed just before it is used (few values
+// live at once).
 template <typename T>
 __device__ __forceinline__ void twiddle8(C<T>* v, C<T> w) {
   const C<T> w2 = mul<T>(w, w);
@@ -242,7 +242,7 @@ __device__ __forceinline__ void twiddle8(C<T>* v, C<T> w) {
 }
 
 // v[q] *= pw[(q-1) s] (or its conjugate), q = 1..7: the powers read from a
-// table instead of formed by multiplication.  The FP64 path uses this: at
+// table instead of formed by multiplication.  The spectrum's FP64 set-up uses this: at
 // GB300's FP64 rate the six products that form the powers cost more than the
 // seven coalesced table loads.
 template <typename T, bool CONJ>
@@ -254,69 +254,9 @@ __device__ __forceinline__ void twiddle8_pow(C<T>* v, const C<T>* pw, int s) {
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void powers8(C<T> w, C<T>* wp) {
-  wp[1] = w;
-  wp[2] = mul<T>(w, w);
-  wp[3] = mul<T>(wp[2], w);
-  wp[4] = mul<T>(wp[2], wp[2]);
-  wp[5] = mul<T>(wp[4], w);
-  wp[6] = mul<T>(wp[3], wp[3]);
-  wp[7] = mul<T>(wp[4], wp[3]);
-}
-
 // The swizzle is linear over GF(2) (XOR of shifted, masked bits), and within
 // a stage the group base and the r * stride term occupy disjoint bits, so
-// swz(base + r s) = swz(base) ^ swz(r s).  The eight values swz(r << ls) of
-// every stride are precomputed per transform length (table `so`, 8 entries
-// per ls = 0..13), leaving one XOR per shared-memory access.
-
-// DIF radix-8 stage with stride 2^ls; thread = butterfly t (t < L/8);
-// tw = this stage's twiddle table; so8 = swz(r << ls), r = 0..7.
-template <typename T>
-__device__ __forceinline__ void dif8(C<T>* buf, int t, int ls, const C<T>* tw, const Swz& z,
-                                     const int* so8) {
-  const int o = t & ((1 << ls) - 1);
-  const int sb = swz<T>(((t >> ls) << (ls + 3)) + o, z);
-  const int4 s0 = __ldg(reinterpret_cast<const int4*>(so8));
-  const int4 s1 = __ldg(reinterpret_cast<const int4*>(so8) + 1);
-  const int ix[8] = {sb ^ s0.x, sb ^ s0.y, sb ^ s0.z, sb ^ s0.w, sb ^ s1.x, sb ^ s1.y, sb ^ s1.z, sb ^ s1.w};
-  C<T> v[8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) v[r] = buf[ix[r]];
-  dft8<T, -1>(v);
-  if (ls > 0) {
-    C<T> wp[8];
-    powers8<T>(__ldg(tw + o), wp);
-#pragma unroll
-    for (int q = 1; q < 8; ++q) v[q] = mul<T>(v[q], wp[q]);
-  }
-#pragma unroll
-  for (int q = 0; q < 8; ++q) buf[ix[q]] = v[q];
-}
-
-// DIT radix-8 inverse stage with stride 2^ls (conjugate twiddles before the butterfly).
-template <typename T>
-__device__ __forceinline__ void dit8(C<T>* buf, int t, int ls, const C<T>* tw, const Swz& z,
-                                     const int* so8) {
-  const int o = t & ((1 << ls) - 1);
-  const int sb = swz<T>(((t >> ls) << (ls + 3)) + o, z);
-  const int4 s0 = __ldg(reinterpret_cast<const int4*>(so8));
-  const int4 s1 = __ldg(reinterpret_cast<const int4*>(so8) + 1);
-  const int ix[8] = {sb ^ s0.x, sb ^ s0.y, sb ^ s0.z, sb ^ s0.w, sb ^ s1.x, sb ^ s1.y, sb ^ s1.z, sb ^ s1.w};
-  C<T> v[8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) v[r] = buf[ix[r]];
-  if (ls > 0) {
-    C<T> wp[8];
-    powers8<T>(conj<T>(__ldg(tw + o)), wp);
-#pragma unroll
-    for (int r = 1; r < 8; ++r) v[r] = mul<T>(v[r], wp[r]);
-  }
-  dft8<T, 1>(v);
-#pragma unroll
-  for (int q = 0; q < 8; ++q) buf[ix[q]] = v[q];
-}
+// swz(base + r s) = swz(base) ^ swz(r s): one XOR per shared-memory access.
 
 // ---------------------------------------------------------------------------
 // Asynchronous global -> shared copies (16-byte chunks, L2 only).

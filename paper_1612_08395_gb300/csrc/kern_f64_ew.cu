@@ -146,18 +146,11 @@ __device__ void stage16_entry(int i, int logL, float2* t32) {
     s /= 16;
   }
 }
-// Index tables of one transform length: so[ls*8 + r] = swz(r << ls) and
-// sp[k] = swz(dig_pos(k)) (see Geo).
-__device__ void geo_entry(int i, int* so, const Geo& g, int esize) {
+// Index table of one transform length: sp[k] = swz(dig_pos(k)) (see Geo).
+__device__ void geo_entry(int i, int* sp, const Geo& g, int esize) {
   const Swz z{g.sa, g.sb, g.sc, g.sd};
-  int x;
-  if (i < kSoEntries) {
-    const int ls = i >> 3, r = i & 7;
-    x = (r << ls) < (1 << g.logL) ? (r << ls) : 0;
-  } else {
-    x = dig_pos(i - kSoEntries, g.logL, g.r0);
-  }
-  so[i] = esize == 4 ? swz<float>(x, z) : swz<double>(x, z);
+  const int x = dig_pos(i, g.logL, g.r0);
+  sp[i] = esize == 4 ? swz<float>(x, z) : swz<double>(x, z);
 }
 __global__ void k_tables(TableArgs a) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -182,7 +175,7 @@ __global__ void k_tables(TableArgs a) {
 #pragma unroll
   for (int t = 0; t < 4; ++t) {
     if (!a.geo[t]) continue;
-    const int n = kSoEntries + (1 << a.g[t].logL);
+    const int n = 1 << a.g[t].logL;
     if (i < n) return geo_entry(i, a.geo[t], a.g[t], a.esize[t]);
     i -= n;
   }
@@ -191,7 +184,7 @@ void launch_tables(const TableArgs& a, cudaStream_t s) {
   const int M = 1 << a.logM, P = 1 << a.logP;
   int n = M + P + M + 1 + (a.t32 ? P : 0);
   for (int t = 0; t < 4; ++t)
-    if (a.geo[t]) n += kSoEntries + (1 << a.g[t].logL);
+    if (a.geo[t]) n += 1 << a.g[t].logL;
   k_tables<<<(n + 63) / 64, 64, 0, s>>>(a);
 }
 

@@ -113,7 +113,7 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   const size_t t_off = (k_off + sizeof(double) * (size_t)hx * hyq + 255) & ~(size_t)255;
   const size_t e_off = (t_off + sizeof(int4) * ntw + 255) & ~(size_t)255;
   const size_t g_off = (e_off + sizeof(int) * ((size_t)Ny + hx) + 255) & ~(size_t)255;
-  const size_t g_ints = 2 * bem::kSoEntries + (size_t)M + py;
+  const size_t g_ints = (size_t)M + py;
   if (g_off + sizeof(int) * g_ints > kScratchBytes)
     return bem::set_error(BEM_EINVAL, "bem_convolve_noalloc: grid needs more than the 2 MiB static scratch");
 
@@ -136,7 +136,7 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   t.logP = ilog2i(py);
   t.fx = twfx;
   t.geo[0] = geo; t.g[0] = pl.gA; t.esize[0] = 8;
-  t.geo[1] = geo + bem::kSoEntries + M; t.g[1] = pl.gB; t.esize[1] = 8;
+  t.geo[1] = geo + M; t.g[1] = pl.gB; t.esize[1] = 8;
   bem::launch_tables(t, s);
   k_transpose_spectrum<<<dim3((hx + 31) / 32, (hyq + 31) / 32), dim3(32, 8), 0, s>>>(khat, khat_t, hx, hyq);
 
@@ -154,10 +154,8 @@ extern "C" int bem_convolve_noalloc(const double* khat, int Nx, int Ny, double c
   a.fxS = twfx + M + py;
   a.fx_ea = reinterpret_cast<int*>(scratch + e_off);
   a.fx_eb = a.fx_ea + Ny;
-  a.soA = geo;
-  a.spA = geo + bem::kSoEntries;
-  a.soB = geo + bem::kSoEntries + M;
-  a.spB = geo + 2 * bem::kSoEntries + M;
+  a.spA = geo;
+  a.spB = geo + M;
   a.uscale = compliance / ((double)px * (double)py);
   bem::launch_pass_a<double>(a, bem::A_PLAIN, s);
   bem::launch_pass_b<double>(a, bem::B_CONV, s);

@@ -50,7 +50,7 @@ size_t footprint(int nx, int ny) {
   b += hyq * (M + 1) * 12;              // spectrum FP64 + FP32
   b += (2 * M + py + 1) * 40;           // twiddles (FP64, FP32, fixed point)
   b += (M + 1 + ny) * 4;                // exponents of the FP64 path's W
-  b += 2 * (224 + M + py) * 4;          // index tables
+  b += 2 * (M + py) * 4;                // index tables
   b += 16 * (M + 1) * ny;               // W (FP64 size)
   b += 3 * 8 * n + n;                   // profile, two FP64 staging fields, contact set
   b += 5 * 4 * n + 5 * 8 * n;           // FP32 and FP64 CG fields

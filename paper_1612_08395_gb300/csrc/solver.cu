@@ -267,7 +267,7 @@ struct bem_ctx {
   double dx = 0, dy = 0, k = 0, nu = 0, E0 = 0, c0 = 0, alpha = 0, A = 0;
   void* block = nullptr;    // device memory of everything below but the CG fields
   double* kq64 = nullptr;
-  int* geo = nullptr;       // index tables: [A32 | B32 | A64 | B64], each so (112) + sp (L)
+  int* geo = nullptr;       // index tables sp: [A32 | B32 | A64 | B64]
   double2* tw64 = nullptr;  // [length-M stages | length-Py stages | split], FP64
   float2* tw32 = nullptr;   // the same, FP32
   int4* twfx = nullptr;     // the first three tables as fixed-point limbs (FP64 path)
@@ -422,11 +422,8 @@ PassArgs<T> make_args(bem_ctx* h) {
   }
   a.fxA = h->twfx; a.fxB = h->twfx + M; a.fxS = h->twfx + M + P;
   a.fx_ea = h->fxe; a.fx_eb = h->fxe + h->ny;
-  const int* gt = h->geo + (sizeof(T) == 8 ? 2 * kSoEntries + M + P : 0);
-  a.soA = gt;
-  a.spA = gt + kSoEntries;
-  a.soB = gt + kSoEntries + M;
-  a.spB = gt + 2 * kSoEntries + M;
+  a.spA = h->geo + (sizeof(T) == 8 ? M + P : 0);
+  a.spB = a.spA + M;
   a.uscale = h->A / ((double)h->px * (double)h->py);
   a.partA = h->part;
   a.partC = h->partC;
@@ -1644,7 +1641,7 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
       {(void**)&h->tw32, sizeof(float2) * ntw},
       {(void**)&h->twfx, sizeof(int4) * (ntw - h->py)},
       {(void**)&h->fxe, sizeof(int) * ((size_t)Ny + M + 1)},
-      {(void**)&h->geo, sizeof(int) * 2 * (2 * kSoEntries + M + h->py)},
+      {(void**)&h->geo, sizeof(int) * 2 * ((size_t)M + h->py)},
       {(void**)&h->khat64, sizeof(double) * (size_t)hyq * (M + 1)},
       {(void**)&h->khat32, sizeof(float) * (size_t)hyq * (M + 1)},
       {(void**)&h->part, sizeof(double) * 4 * (size_t)gmax},
@@ -1686,11 +1683,11 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
     t.t32 = h->tw32;
     t.fx = h->twfx;
     int* g32 = h->geo;
-    int* g64 = h->geo + 2 * kSoEntries + M + h->py;
+    int* g64 = h->geo + M + h->py;
     t.geo[0] = g32; t.g[0] = h->plan32.gA; t.esize[0] = 4;
-    t.geo[1] = g32 + kSoEntries + M; t.g[1] = h->plan32.gB; t.esize[1] = 4;
+    t.geo[1] = g32 + M; t.g[1] = h->plan32.gB; t.esize[1] = 4;
     t.geo[2] = g64; t.g[2] = h->plan64.gA; t.esize[2] = 8;
-    t.geo[3] = g64 + kSoEntries + M; t.g[3] = h->plan64.gB; t.esize[3] = 8;
+    t.geo[3] = g64 + M; t.g[3] = h->plan64.gB; t.esize[3] = 8;
     launch_tables(t, h->stream);
   }
   // a1: influence coefficients on the offsets 0..Px/2, 0..Py/2 (Eq. 9)
@@ -1707,9 +1704,8 @@ static int create_ctx(int Nx, int Ny, double dx, double dy, double k, double nu,
     PassArgs<double> a{};
     a.pl = h->plan64;
     a.twA = h->tw64; a.twB = h->tw64 + M; a.twS = h->tw64 + M + h->py;
-    const int* g64 = h->geo + 2 * kSoEntries + M + h->py;
-    a.soA = g64; a.spA = g64 + kSoEntries;
-    a.soB = g64 + kSoEntries + M; a.spB = g64 + 2 * kSoEntries + M;
+    a.spA = h->geo + M + h->py;
+    a.spB = a.spA + M;
     a.W = h->W;  // with the fields after it
     a.rows_w = hyq;  // K is even: rows 0..Py/2 of the torus hold all
     a.nrows_in = hyq;
