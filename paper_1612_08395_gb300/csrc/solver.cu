@@ -990,9 +990,10 @@ int coop_applies(const bem_ctx* h, int es, int rows) {
 }
 
 // The CG loop over `rows` grid rows as cooperative launches of nb CTAs, each of at
-// most kResidentIters iterations.  *finished = false: a launch's CTAs did not all
-// become resident, the loop's state is as before it (nothing or a number of whole
-// launches done) and the passes go on from there.
+// most kResidentIters iterations.  *finished = false: a launch was refused (this
+// process may use too few of the device's SMs) or its CTAs did not all become
+// resident; the loop's state is as before it (nothing or a number of whole launches
+// done) and the passes go on from there.
 int run_coop(bem_ctx* h, bool pk, int rows, int nb, bool* finished) {
   *finished = false;
   CoopHold hold;
@@ -1004,7 +1005,18 @@ int run_coop(bem_ctx* h, bool pk, int rows, int nb, bool* finished) {
   r.max_launch = loop_iters();
   const int lm = ilog2(h->px / 2), lp = ilog2(h->py);
   for (int runs = 1;; ++runs) {
-    CK(pk ? launch_coop_pk(r, lm, lp, h->stream) : launch_coop_cg(r, lm, lp, h->stream));
+    cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
+#ifdef BEM_DEBUG_CHECKS
+    const char* inj = getenv("BEM_INJECT_COOP_REFUSED");  // test hook: as if the launch were refused
+    if (!(inj && inj[0] == '1'))
+#endif
+    e = pk ? launch_coop_pk(r, lm, lp, h->stream) : launch_coop_cg(r, lm, lp, h->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources) {
+      cudaGetLastError();
+      CKR(read_scalars(h));
+      return BEM_OK;
+    }
+    CK(e);
     h->launches += 1;
     CKR(read_scalars(h));
     if (h->sc_host->coop_runs != runs) return BEM_OK;

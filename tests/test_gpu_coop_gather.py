@@ -1,7 +1,8 @@
-"""The cooperative CG loop when not all of its CTAs become resident (another
-stream's kernel may hold some back): in a debug build one CTA stays away on
-request, the others give the gathering up after a tenth of a second, and the loop
-runs as passes with the result of a solve that always does.  And a CTA that stays
+"""The cooperative CG loop when its launch is refused, or not all of its CTAs become
+resident (another stream's kernel may hold some back): in a debug build the launch
+is refused or one CTA stays away on request, the others give the gathering up after
+a tenth of a second, and the loop runs as passes with the result of a solve that
+always does.  And a CTA that stays
 away from a later barrier: the bounded waits run out, the call returns
 BEM_ETIMEOUT, and the handle recovers."""
 import json
@@ -25,8 +26,9 @@ import paper_1612_08395_gb300.bem as bem
 import paper_1612_08395_gb300.inputs as I
 out = []
 def inject(v):
-    os.environ.pop("BEM_INJECT_WAIT_TIMEOUT", None)
-    if v: os.environ["BEM_INJECT_WAIT_TIMEOUT"] = str(v)
+    for k in ("BEM_INJECT_WAIT_TIMEOUT", "BEM_INJECT_COOP_REFUSED"):
+        os.environ.pop(k, None)
+    if v: os.environ["BEM_INJECT_COOP_REFUSED" if v == "refused" else "BEM_INJECT_WAIT_TIMEOUT"] = "1" if v == "refused" else str(v)
 for nx, ny, box in ((256, 256, False), (300, 514, False), (1000, 600, False), (514, 514, True)):
     dx = 1.0 / max(nx, ny)
     r = I.radius_grid(nx, ny, dx)
@@ -36,7 +38,8 @@ for nx, ny, box in ((256, 256, False), (300, 514, False), (1000, 600, False), (5
         hd.solve(h, d0, precision="fp32_refine")  # sub-grids are set up on first use
         for what in ("solve", "pull-off"):
             runs = {}
-            for name, v, timed in (("coop", 0, False), ("held back", 2, False), ("passes", 0, True)):
+            for name, v, timed in (("coop", 0, False), ("held back", 2, False), ("refused", "refused", False),
+                                   ("passes", 0, True)):
                 inject(v)
                 p = np.empty((ny, nx))
                 before = hd.info().kernel_launches
@@ -51,7 +54,7 @@ for nx, ny, box in ((256, 256, False), (300, 514, False), (1000, 600, False), (5
             inject(0)
             ref = runs["passes"][0]
             n = max(float(np.linalg.norm(ref)), 1e-300)
-            for name in ("coop", "held back"):
+            for name in ("coop", "held back", "refused"):
                 p, rc, cnt, rounds, launches = runs[name]
                 out.append({"case": [nx, ny, box, what, name], "rc": rc, "err": float(np.linalg.norm(p - ref)) / n,
                             "counts": cnt == runs["passes"][2], "rounds": rounds == runs["passes"][3],
