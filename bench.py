@@ -25,6 +25,10 @@ roofline    : the dominant transform pass, algorithmic bytes / its live average
               and rows that launch worked on (bem_pass_work).  `traffic` is the
               ncu DRAM bytes per launch of that kernel from profiles/, or null
               when the kernel sources changed since that capture
+timed_loop  : what the timed sweeps run instead of those passes: their CG loops
+              are cooperative launches (k_coop); the whole sweep's time per CG
+              iteration (refinement, detachment and statistics included) and
+              the passes' algorithmic bytes of an iteration over it
 plain_fp32  : the same sweep in plain FP32 (no refinement), and how its
               contact counts and forces compare with the timed sweep's
 full_torus  : the 2048^2 Polonsky-Keer step as the paper applies it, on the whole
@@ -404,6 +408,14 @@ def kernel_sources_sha():
     return hs.hexdigest()[:16]
 
 
+def timed_loop(sweep_s, iterations, bytes_it, hbm):
+    """The timed sweeps' CG loops (one cooperative launch each): the sweep's time per iteration,
+    everything included, and the bytes that an iteration by separate passes moves, over it."""
+    t = sweep_s / max(iterations, 1)
+    return {"kernel": "k_coop", "us_per_iteration": 1e6 * t, "bytes_per_iteration": bytes_it,
+            "achieved": bytes_it / t / 1e9, "unit": "GB/s", "frac_of_hbm": bytes_it / t / 1e9 / hbm}
+
+
 def profiled_traffic(kernel_key, bytes_per_launch):
     """ncu DRAM bytes per launch recorded in profiles/traffic_*.md for this kernel
     (lines `kernel_key:`, `source_sha16:`, `dram_bytes_per_launch:` and, when the
@@ -650,6 +662,7 @@ def main():
                              "frac": flops_dom / (avg_ms[dom] * 1e-3) / 1e12
                              / fp32_peak_tflops(clocks.get("sm_max_mhz")),
                              "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 x max SM clock"}},
+        "timed_loop": timed_loop(elapsed / args.steps, iters_total / args.steps, sum(work_bytes), hbm),
         "clocks": clocks,
         "e2e": {"value": e2e_val, "unit": UNIT, "steps": e2e_steps,
                 "h2d_bytes_per_step": 8 * N * N + 8 * len(ds),
